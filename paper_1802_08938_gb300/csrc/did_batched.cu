@@ -39,11 +39,14 @@
 // 128 rows (two chunks of 64; into a second accumulator set meanwhile, so the
 // MMAs do not wait), and the update pass its W accumulator every eight tiles.
 //
-// The products are small (M = 128, N = 32 to 128), and a tcgen05.mma of
-// M = 128 costs about the same for every N up to 128, so the passes stack the
-// terms of their shared-memory operand along N: one MMA forms several of the
-// six products into adjacent accumulator ranges (three MMAs per K step for
-// the rank-2K update, four for g and W; see the kernels).
+// The products are small (M = 128, N = 32 to 128).  The passes stack the terms
+// of their shared-memory operand along N: one MMA forms several of the six
+// products into adjacent accumulator ranges (three MMAs per K step for the
+// rank-2K update, four for g and W; see the kernels), so one thread issues
+// half as many.  Issued under elect.sync an MMA takes N / 2 cycles
+// (tc::elect_one); issued under `lane == 0` the same loops took about 114
+// cycles an MMA whatever N was.  At 5000 x 200000, K = 50 that change alone
+// took a sweep from 4.93 to 3.44 ms, bit for bit the same.
 //
 // Kernels of one sweep (K <= 64):
 //   prep_gb     B -> bfloat16 x3 tiles of 64 rows for the g pass (2 MB at K = 50)
@@ -309,8 +312,7 @@ constexpr int kGGroup = 2;
 //   R0 [B0 B1] and R1 [B0 B1] -> ranges 0, 1;  R0 B2 and R2 B0 -> range 1,
 // range 0 holding R0 B0 + R1 B0, range 1 the other four products, and
 // g = range 0 + range 1.  Four MMAs of N = 2KN, 2KN, KN, KN per K step do
-// the work of six of N = KN (an MMA of M = 128 costs about the same for
-// every N up to 128).
+// the work of six of N = KN.
 __global__ void __launch_bounds__(kGThreads, 1) g_kernel(GArgs a, const __grid_constant__ CUtensorMap tmR) {
   extern __shared__ unsigned char sm_raw[];
   unsigned char* sm = align1024(sm_raw);
@@ -381,7 +383,7 @@ __global__ void __launch_bounds__(kGThreads, 1) g_kernel(GArgs a, const __grid_c
         mbar_wait_bounded(full + (d % ring), (uint32_t)((d / ring) & 1), err, tmo);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (tc::elect_one()) {
       const uint32_t id2 = tc::instr_desc_bf16(128, 2 * KN), id1 = tc::instr_desc_bf16(128, KN);
       const uint64_t bdesc_ring = tc::smem_desc(smem_u32(bring), 128u, (uint32_t)kGChunk * 16u);
       const uint32_t pterm = (uint32_t)(KN * kGChunk * 2);    // bytes of one term of the B chunk
@@ -503,7 +505,7 @@ __global__ void __launch_bounds__(kGThreads, 1) g_kernel(GArgs a, const __grid_c
 
   // Drain: every issued MMA completes before tensor memory is freed.
   __syncthreads();
-  if (warp == 1 && lane == 0 && shared_flags[0] > 0) {
+  if (warp == 1 && shared_flags[0] > 0 && tc::elect_one()) {
     tc::mma_commit(bars + G_DRAIN);
     mbar_wait_bounded(bars + G_DRAIN, 0u, err, tmo);
   }
@@ -833,9 +835,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) update_kernel(UArgs a, const __
   // tile), one MMA per term of Y forms several products:
   //   Y0 [Z0 Z1 Z2] -> ranges 0, 1, 2;  Y1 [Z0 Z1] -> ranges 1, 2;  Y2 Z0 -> range 2,
   // so range 0 holds Y0 Z0, range 1 Y0 Z1 + Y1 Z0, range 2 the 2^-16 terms
-  // Y0 Z2 + Y1 Z1 + Y2 Z0, and Y Z = range 0 + (range 1 + range 2).  A
-  // tcgen05.mma of M = 128 costs about the same for every N up to 128, so
-  // three MMAs of N = 3nu, 2nu, nu per K step do the work of six of N = nu.
+  // Y0 Z2 + Y1 Z1 + Y2 Z0, and Y Z = range 0 + (range 1 + range 2): three
+  // MMAs of N = 3nu, 2nu, nu per K step do the work of six of N = nu.
   // W = E' C'^T likewise, with the terms of C'^T stacked two at a time:
   //   E0 [C0 C1] and E1 [C0 C1] -> ranges 0, 1;  E0 C2 and E2 C0 -> range 1,
   // so range 0 holds E0 C0 + E1 C0 and range 1 the other four products, and
@@ -904,7 +905,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) update_kernel(UArgs a, const __
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------- MMA issue
-    if (lane == 0) {
+    if (tc::elect_one()) {
       const uint32_t iU3 = tc::instr_desc_bf16(128, 3 * nu), iU2 = tc::instr_desc_bf16(128, 2 * nu);
       const uint32_t iU1 = tc::instr_desc_bf16(128, nu), iW1 = tc::instr_desc_bf16(128, KN);
       const uint32_t iW2 = tc::instr_desc_bf16(128, 2 * KN);
@@ -1161,7 +1162,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) update_kernel(UArgs a, const __
   }
 
   __syncthreads();
-  if (warp == 1 && lane == 0 && shared_flags[0] != 0) {
+  if (warp == 1 && shared_flags[0] != 0 && tc::elect_one()) {
     tc::mma_commit(bars + U_DRAIN);
     mbar_wait_bounded(bars + U_DRAIN, 0u, err, tmo);
   }

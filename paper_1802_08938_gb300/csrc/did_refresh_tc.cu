@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) refresh_tc_kernel(TcArgs a, con
     }
   } else if (warp == 1) {
     // ----------------------------------------------------------- MMA issue
-    if (lane == 0) {
+    if (tc::elect_one()) {
       const uint32_t idesc = tc::instr_desc_bf16(kTileM, kTileN);
       const uint32_t sA0 = smem_u32(sA), sC0 = smem_u32(sC);
       const uint32_t sbo = (uint32_t)Kp * 16;      // next 8-row group
@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) refresh_tc_kernel(TcArgs a, con
 
   // Drain: every issued MMA must finish before TMEM is freed.
   __syncthreads();
-  if (warp == 1 && lane == 0 && mma_steps[0] > 0) {
+  if (warp == 1 && mma_steps[0] > 0 && tc::elect_one()) {
     tc::mma_commit(bars + BAR_DRAIN);
     mbar_wait_bounded(bars + BAR_DRAIN, 0u, err, tmo);
   }

@@ -21,8 +21,9 @@
 //   warp 3      producer of the 128 x 64 X tiles (one 2-D tensor copy each)
 //               into a ring of as many buffers as shared memory holds (2-4),
 //               so the X reads run ahead of the epilogue;
-//   warp 1      allocates 128 TMEM columns (two 128 x 64 float32 accumulators)
-//               and one elected thread issues the tcgen05.mma instructions;
+//   warp 1      allocates TMEM for two accumulators of three (two) ranges of
+//               128 x 64 float32, and one elected thread issues the
+//               tcgen05.mma instructions;
 //   warp 2      stores each finished tile of R by one 2-D tensor copy and
 //               releases its X buffer once the copy has read it (the wait
 //               comes after the next store is issued, so two overlap);
@@ -63,7 +64,8 @@ constexpr int kMaxKp = 128;         // K padded to a multiple of 16, at most 128
 constexpr int kMaxKpF32 = 64;       // three-term operands take 1.5x the shared memory
 constexpr int kMaxXBuf = 4;         // X tile ring
 constexpr int kMaxCBuf = 4;         // C-factor tile ring
-constexpr int kTmemCols = 128;      // two accumulators of kTileN columns
+// TMEM columns: two accumulators of NT ranges of kTileN columns each (a power of two).
+template <bool F32> constexpr int kTmemCols = F32 ? 512 : 256;
 
 struct TcArgs {
   const float* X;            // ld x N float32, column-major
@@ -133,7 +135,14 @@ template <bool F32>
 __global__ void __launch_bounds__(kTcThreads, 1) refresh_tc_kernel(TcArgs a, const __grid_constant__ CUtensorMap tmX,
                                                                   const __grid_constant__ CUtensorMap tmR) {
   constexpr int NT = F32 ? 3 : 2;                 // bfloat16 terms per operand
-  constexpr int NPROD = F32 ? 6 : 3;              // products p_i q_j with i + j <= NT - 1
+  // TMEM columns of one accumulator: range r holds the products p_i q_j with
+  // i + j = r.  The tensor core's float32 accumulation truncates, so every
+  // MMA that adds into a sum of size s biases it by about 2^-24 s.  With all
+  // products in one range that bias was 1.3e-6 of |B||C| at K = 50 (24
+  // MMAs) and set the error of whole factorisations: B 1.3e-6 from 64 bits after
+  // two sweeps of 5000 x 200000, where float32 arithmetic gives 1.4e-7.  Now
+  // only the Kp / 16 leading ones add to the large sum.
+  constexpr int ACCW = NT * kTileN;
   constexpr int KSTEP = 16;                       // K per MMA (32 bytes)
   extern __shared__ __align__(1024) unsigned char sm[];
   const int XB = a.xbufs, CB = a.cbufs;
@@ -151,7 +160,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) refresh_tc_kernel(TcArgs a, con
   const uint32_t a_bytes = (uint32_t)NT * kTileM * Kp * 2;
   const uint32_t c_bytes = (uint32_t)NT * kTileN * Kp * 2;
   const uint32_t a_split = (uint32_t)kTileM * Kp * 2;     // bytes of one term of the A tile
-  const uint32_t c_split = (uint32_t)kTileN * Kp * 2;
 
   if (threadIdx.x == 0) {
     mma_steps[0] = 0;
@@ -163,7 +171,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) refresh_tc_kernel(TcArgs a, con
     }
   }
   fence_mbar_init();
-  if (warp == 1) tc::tmem_alloc(tmem_slot, kTmemCols);
+  if (warp == 1) tc::tmem_alloc(tmem_slot, kTmemCols<F32>);
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
@@ -236,7 +244,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) refresh_tc_kernel(TcArgs a, con
   } else if (warp == 1) {
     // ----------------------------------------------------------- MMA issue
     if (tc::elect_one()) {
-      const uint32_t idesc = tc::instr_desc_bf16(kTileM, kTileN);
+      const uint32_t id1 = tc::instr_desc_bf16(kTileM, kTileN), id2 = tc::instr_desc_bf16(kTileM, 2 * kTileN);
+      const uint32_t id3 = tc::instr_desc_bf16(kTileM, 3 * kTileN);
       const uint32_t sA0 = smem_u32(sA), sC0 = smem_u32(sC);
       const uint32_t sbo = (uint32_t)Kp * 16;      // next 8-row group
       int64_t s = 0, ui = 0;
@@ -254,19 +263,20 @@ __global__ void __launch_bounds__(kTcThreads, 1) refresh_tc_kernel(TcArgs a, con
             break;
           }
           tc::fence_after();
-          const uint32_t d = tmem + (uint32_t)(ab * kTileN);
+          const uint32_t d = tmem + (uint32_t)(ab * ACCW);
           const uint32_t cbase = sC0 + (uint32_t)cb * c_bytes;
-          // the NPROD products of the terms, p_i q_j with i + j < NT
-#pragma unroll
-          for (int pr = 0; pr < NPROD; ++pr) {
-            const int ti_a = pr == 2 || pr == 4 ? 1 : (pr == 5 ? 2 : 0);
-            const int ti_b = pr == 1 || pr == 4 ? 1 : (pr == 3 ? 2 : 0);
-            const uint32_t aoff = (uint32_t)ti_a * a_split;
-            const uint32_t coff = (uint32_t)ti_b * c_split;
-            for (int kk = 0; kk < Kp / KSTEP; ++kk) {
-              const uint64_t ad = tc::smem_desc(sA0 + aoff + (uint32_t)kk * 256u, 128u, sbo);
-              const uint64_t bd = tc::smem_desc(cbase + coff + (uint32_t)kk * 256u, 128u, sbo);
-              tc::mma_bf16(d, ad, bd, idesc, (pr > 0 || kk > 0) ? 1u : 0u);
+          // The terms of the C tile lie one after another, so stacked along N
+          // they form one operand: A0 [C0 C1 C2] -> ranges 0, 1, 2; A1 [C0 C1] ->
+          // ranges 1, 2; A2 C0 -> range 2 (two terms: A0 [C0 C1], A1 C0).
+          for (int kk = 0; kk < Kp / KSTEP; ++kk) {
+            const uint64_t bd = tc::smem_desc(cbase + (uint32_t)kk * 256u, 128u, sbo);
+            const uint64_t a0 = tc::smem_desc(sA0 + (uint32_t)kk * 256u, 128u, sbo);
+            const uint64_t a1 = tc::smem_desc(sA0 + a_split + (uint32_t)kk * 256u, 128u, sbo);
+            tc::mma_bf16(d, a0, bd, F32 ? id3 : id2, kk > 0 ? 1u : 0u);
+            tc::mma_bf16(d + kTileN, a1, bd, F32 ? id2 : id1, 1u);
+            if (F32) {
+              const uint64_t a2 = tc::smem_desc(sA0 + 2 * a_split + (uint32_t)kk * 256u, 128u, sbo);
+              tc::mma_bf16(d + 2 * kTileN, a2, bd, id1, 1u);
             }
           }
           tc::mma_commit(bars + BAR_ACC_FULL + ab);
@@ -349,8 +359,19 @@ __global__ void __launch_bounds__(kTcThreads, 1) refresh_tc_kernel(TcArgs a, con
         tc::fence_after();
         float d[kTileN / 2];
 #pragma unroll
-        for (int c = 0; c < kTileN / 2; c += 16)
-          tc::tmem_ld<16>(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ab * kTileN + c0 + c), d + c);
+        for (int c = 0; c < kTileN / 2; c += 16) {
+          const uint32_t at = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ab * ACCW + c0 + c);
+          float r1[16], r2[16];
+          if (F32) {
+            tc::tmem_ld3x16(at, at + kTileN, at + 2 * kTileN, d + c, r1, r2);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) d[c + e] += r1[e] + r2[e];
+          } else {
+            tc::tmem_ld2x16(at, at + kTileN, d + c, r1);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) d[c + e] += r1[e];
+          }
+        }
         tc::fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(bars + BAR_ACC_EMPTY + ab);
@@ -418,7 +439,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) refresh_tc_kernel(TcArgs a, con
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
-  if (warp == 1) tc::tmem_dealloc(tmem, kTmemCols);
+  if (warp == 1) tc::tmem_dealloc(tmem, kTmemCols<F32>);
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int w = 0; w < kEpiWarps; ++w) t += red[w];

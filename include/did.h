@@ -114,14 +114,20 @@ typedef struct {
  * the tensor-core pass (BF16x3 for a bfloat16 residual with K <= 128, BF16x6
  * for a float32 one with K <= 64; larger K always takes the SIMT pass). */
 #define DID_FLAG_SIMT_REFRESH 2
-/* did_options.flags (DID_ORDER_INTERLEAVED): deferred write-back defers the
+/* did_options.flags (DID_ORDER_INTERLEAVED).  Without a flag below, and where
+ * the tensor-core refresh takes K, sweeps of a larger residual only read R:
+ * the changes of a sweep stay pending as vectors, and R is formed anew from X
+ * after its last k (did_info then counts a periodic refresh that falls due,
+ * which finds R formed from the current factors already).
+ * Deferred write-back defers the
  * write of R for k to the pass for k+1 (one write per pair of k, three passes
  * over R per pair instead of four).  It needs two more M-vectors of shared
  * memory beside a ring of at least three column stages per group.  By default
  * a float32 residual uses it where it fits and a bfloat16 residual does not
  * (its passes are bound by the per-column work, which the deferred form
  * raises).  EAGER forces one write per k; LAZY requests deferral for either
- * precision.  did_info.lazy_writeback says which ran. */
+ * precision.  did_info.lazy_writeback says which the sweep kernel is planned
+ * with. */
 #define DID_FLAG_EAGER_WRITEBACK 8
 #define DID_FLAG_LAZY_WRITEBACK 16
 /* did_options.flags (DID_ORDER_INTERLEAVED): c-passes take one column per
@@ -154,7 +160,7 @@ typedef struct {
     double dense_kernel_ms;
     int64_t tc_refreshes;    /* refreshes done on the tensor cores */
     double tc_refresh_ms;    /* their device time (operand split + the tensor-core pass) */
-    int32_t lazy_writeback;  /* 1: the sweep defers the write of R in pairs of k */
+    int32_t lazy_writeback;  /* 1: the sweep kernel defers the write of R in pairs of k */
     int32_t ring_stages;     /* shared-memory column stages per column group */
     int32_t column_pairs;    /* 1: a column group takes two columns per step of a c-pass */
 } did_info;

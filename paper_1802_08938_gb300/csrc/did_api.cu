@@ -63,6 +63,9 @@ struct did_ctx {
   double* part_host = nullptr;      // pinned, 3 * dense grid
 
   did::SweepPlan plan{};
+  bool defer = false;               // interleaved sweeps read R only and form it anew after each sweep
+  did::DeferPlan dplan{};
+  did::DeferBuffers dbuf{};
   int dense_grid = 0;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   int64_t sweep_launches = 0, prologue_launches = 0, dense_launches = 0;
@@ -214,8 +217,8 @@ did_status dense(did_ctx* c, int mode, double sums[3]) {
   return DID_OK;
 }
 
-// Tensor-core refresh of a bfloat16 residual; returns 1/2 ||R||^2 in *f.
-did_status refresh_tc(did_ctx* c, double* f) {
+// Workspace of the tensor-core refresh (on first use).
+did_status refresh_tc_workspace(did_ctx* c) {
   void* p;
   did_status st;
   const int G = did::refresh_tc_grid();
@@ -230,6 +233,14 @@ did_status refresh_tc(did_ctx* c, double* f) {
     if (st != DID_OK) return st;
     c->tc_err = (int*)p;
   }
+  return DID_OK;
+}
+
+// Tensor-core refresh; returns 1/2 ||R||^2 in *f.
+did_status refresh_tc(did_ctx* c, double* f) {
+  const did_status st = refresh_tc_workspace(c);
+  if (st != DID_OK) return st;
+  const int G = did::refresh_tc_grid();
   std::vector<double> part(G);
   int herr = 0;
   // The interleaved order's first b-update takes the partials of R c_1^T
@@ -425,7 +436,67 @@ did_status run_batched(did_ctx* c, int64_t max_sweeps, int stop_rule, double tol
   return DID_OK;
 }
 
+// Interleaved order by read-only sweeps: each sweep is the K passes of the
+// sweep kernel over a residual that it does not write, then R = X - B C on the
+// tensor cores (with 1/2 ||R||^2 and the partials of R c_1^T).  A periodic
+// refresh that falls due finds R formed from the current factors already.
+did_status run_defer(did_ctx* c, int64_t max_sweeps, int stop_rule, double tol, int64_t* done_total) {
+  *done_total = 0;
+  const int G = did::refresh_tc_grid();
+  while (*done_total < max_sweeps) {
+    if (c->need_refresh || c->npart_first == 0) {
+      did_status st = refresh(c);
+      if (st != DID_OK) return st;
+    } else if (refresh_due(c)) {
+      c->last_refresh_at = c->sweeps_done;
+      c->refreshes++;
+      c->tc_refreshes++;
+    }
+    const int n = stop_rule ? 1 : chunk_size(c, max_sweeps - *done_total);   // with a stopping rule: one sweep per check
+    const uint64_t tmo = wait_limit_ns(c);
+    const int cap = c->tstamp ? (int)std::min<int64_t>((int64_t)n * c->K, c->tstamp_cap) : 0;
+    c->tstamp_n = cap;
+    DID_CUDA(c, cudaMemsetAsync(c->ctrl, 0, sizeof(Ctrl), c->stream));
+    DID_CUDA(c, cudaMemsetAsync(c->dbuf.work, 0, sizeof(unsigned) * c->K, c->stream));
+    DID_CUDA(c, cudaEventRecord(c->ev0, c->stream));
+    for (int s = 0; s < n; ++s) {
+      const int step0 = s * c->K;
+      DID_CUDA(c, did::launch_defer(c->dplan, c->dbuf, c->ld, c->N, c->K, c->npart_first, c->opt.debug_barrier_extra,
+                                    tmo, step0 < cap ? c->tstamp + 4 * (size_t)step0 : nullptr,
+                                    std::max(0, cap - step0), c->stream));
+      DID_CUDA(c, did::launch_refresh_tc(c->X, c->R, c->B, c->C, (int)c->M, c->ld, c->N, c->K, c->tc_ws, c->tc_part,
+                                         c->P, c->CCp, &c->ctrl->err, tmo, c->stream, !c->bf16));
+      DID_CUDA(c, did::launch_defer_close(c->tc_part, G, c->dbuf, c->K, c->trace_dev + s, c->stream));
+    }
+    DID_CUDA(c, cudaEventRecord(c->ev1, c->stream));
+    DID_CUDA(c, cudaMemcpyAsync(c->ctrl_host, c->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, c->stream));
+    DID_CUDA(c, cudaMemcpyAsync(c->trace_host, c->trace_dev, sizeof(double) * n, cudaMemcpyDeviceToHost, c->stream));
+    DID_CUDA(c, cudaStreamSynchronize(c->stream));
+    const Ctrl h = *c->ctrl_host;
+    float ms = 0.f;
+    DID_CUDA(c, cudaEventElapsedTime(&ms, c->ev0, c->ev1));
+    c->sweep_ms += ms;
+    c->sweep_launches += n;
+    for (int s = 0; s < h.sweeps; ++s) c->trace.push_back(c->trace_host[s]);
+    c->sweeps_done += h.sweeps;
+    *done_total += h.sweeps;
+    if (h.sweeps > 0) c->last_obj = c->trace.back();
+    if (h.err != 0) {
+      // A bounded wait ran out: B and C hold valid nonnegative values, R is
+      // recomputed from them before the next sweep.
+      c->need_refresh = true;
+      return fail(c, DID_ETIMEOUT, "a bounded wait of the sweep exceeded its limit (device error %d); "
+                  "state kept, residual will be recomputed", h.err);
+    }
+    const double f = c->last_obj, prev = c->trace[c->trace.size() - 2];
+    if (stop_rule == 1 && (f == 0.0 || (prev > 0.0 && fabs(prev - f) / prev < tol))) break;
+    if (stop_rule == 2 && f <= tol * c->trace.front()) break;
+  }
+  return DID_OK;
+}
+
 did_status run(did_ctx* c, int64_t max_sweeps, int stop_rule, double tol, int64_t* done_total) {
+  if (c->defer) return run_defer(c, max_sweeps, stop_rule, tol, done_total);
   if (c->batched) return run_batched(c, max_sweeps, stop_rule, tol, done_total);
   *done_total = 0;
   while (*done_total < max_sweeps) {
@@ -489,6 +560,15 @@ did_status did_create(const float* X, int64_t M, int64_t N, int32_t K, uint64_t 
   return did_create_ex(X, M, N, K, seed, &o, out);
 }
 
+// Whether read-only sweeps pay: the pending terms (2 K values a column) are
+// small beside a column, and a pass is longer than the phases around it (about 20 us
+// a k, where the sweep kernel takes 27 to 32 us for small passes: 1024 x 2414 in
+// bfloat16, 5 MB, measured 29.6 against 29.2 us a k; 784 x 70000, 110 MB, 44
+// against 70).
+static bool defer_pays(const did_ctx* c) {
+  return c->ld >= 4 * c->K && (size_t)c->ld * c->N * (c->bf16 ? 2 : 4) >= ((size_t)16 << 20);
+}
+
 static did_status create_impl(did_ctx* c, const float* X, uint64_t seed) {
   const int64_t M = c->M, N = c->N;
   const int K = c->K;
@@ -498,6 +578,13 @@ static did_status create_impl(did_ctx* c, const float* X, uint64_t seed) {
   did_status st =
       did::plan_sweep(c->ld, c->N, c->bf16, c->opt.grid_ctas, 0, &c->plan, err, sizeof(err), want_lazy);
   if (st != DID_OK) return fail(c, st, "%s", err);
+  // A flag that asks for a form of write-back, column step or refresh keeps the sweep kernel that has it.
+  const bool no_flags = !(c->opt.flags & (DID_FLAG_EAGER_WRITEBACK | DID_FLAG_LAZY_WRITEBACK | DID_FLAG_SINGLE_COLUMNS |
+                                          DID_FLAG_SIMT_REFRESH));
+  // Sweeps that only read R, where the tensor-core refresh can form R after each.
+  c->defer = no_flags && c->opt.order == DID_ORDER_INTERLEAVED &&
+             did::refresh_tc_supported(K, !c->bf16) && defer_pays(c) &&
+             did::plan_defer(c->ld, N, K, c->bf16, c->opt.grid_ctas, &c->dplan);
   c->dense_grid = did::dense_grid();
   DID_CUDA(c, cudaEventCreate(&c->ev0));
   DID_CUDA(c, cudaEventCreate(&c->ev1));
@@ -517,19 +604,36 @@ static did_status create_impl(did_ctx* c, const float* X, uint64_t seed) {
   DID_CUDA(c, cudaMemsetAsync(c->Y, 0, (size_t)c->ld * K * sizeof(float), c->stream));
   ALLOC(C, (size_t)K * N * sizeof(float));
   // partial rows: the plan's, and the tensor-core refresh's two per CTA
-  const size_t U = (size_t)std::max(std::max(c->plan.npart, G), 2 * did::refresh_tc_grid());
+  const size_t U = (size_t)std::max(std::max(c->defer ? c->dplan.npart : c->plan.npart, G), 2 * did::refresh_tc_grid());
   ALLOC(P, U * c->ld * sizeof(float));
   ALLOC(CCp, U * sizeof(double));
   ALLOC(Sp, (size_t)2 * G * sizeof(double));
   ALLOC(OBJp, U * sizeof(double));
   ALLOC(bold, (size_t)c->ld * sizeof(float));
-  if (c->plan.lazy) {
+  if (c->defer) {
+    did::DeferBuffers& d = c->dbuf;
+    const size_t W = (size_t)c->dplan.GS / 32;
+    ALLOC(dbuf.Bo, (size_t)c->ld * K * sizeof(float));
+    ALLOC(dbuf.Co, (size_t)K * N * sizeof(float));
+    ALLOC(dbuf.T, (size_t)N * W * sizeof(float));
+    ALLOC(dbuf.corr, (size_t)N * 2 * sizeof(float));
+    ALLOC(dbuf.Xp, did::defer_pair_bytes(K, c->dplan.grid));
+    ALLOC(dbuf.Yp, did::defer_pair_bytes(K, c->dplan.grid));
+    ALLOC(dbuf.work, (size_t)K * sizeof(unsigned));
+    d.R = c->R;
+    d.B = c->B;
+    d.C = c->C;
+    d.P = c->P;
+    d.CC0 = c->CCp;
+  } else if (c->plan.lazy) {
     ALLOC(Cold, (size_t)N * sizeof(float));
     ALLOC(XCp, 2 * U * sizeof(double));
   }
   ALLOC(ctrl, sizeof(Ctrl));
   ALLOC(trace_dev, sizeof(double) * kMaxSweepsPerLaunch);
   ALLOC(degen, sizeof(unsigned long long));
+  c->dbuf.ctrl = c->ctrl;
+  c->dbuf.degen = c->degen;
   ALLOC(dense_part, sizeof(double) * 3 * c->dense_grid);
   ALLOC(bad, sizeof(unsigned long long));
   if (c->opt.flags & DID_FLAG_PHASE_TIMES) {
@@ -748,11 +852,11 @@ did_status did_get_info(did_ctx* c, did_info* info) {
   info->K = c->K;
   info->precision = c->opt.precision;
   info->order = c->opt.order;
-  info->grid_ctas = c->plan.grid;
-  info->group_threads = c->plan.GS;
-  info->vecs_per_thread = c->plan.NR;
-  info->column_units = c->plan.nunits;
-  info->dynamic_units = c->plan.dynamic;
+  info->grid_ctas = c->defer ? c->dplan.grid : c->plan.grid;
+  info->group_threads = c->defer ? c->dplan.GS : c->plan.GS;
+  info->vecs_per_thread = c->defer ? c->dplan.NR : c->plan.NR;
+  info->column_units = c->defer ? c->dplan.nunits : c->plan.nunits;
+  info->dynamic_units = c->defer ? c->dplan.dynamic : c->plan.dynamic;
   info->ld = c->ld;
   info->sweeps_done = c->sweeps_done;
   unsigned long long d = 0;

@@ -333,6 +333,36 @@ did_status plan_sweep(int ld, int64_t N, bool bf16, int grid_override, int64_t m
                       char* err, size_t errlen, bool want_lazy = false);
 cudaError_t launch_sweep(const SweepPlan& plan, const SweepArgs& args, cudaStream_t s);
 
+// Read-only sweep of the interleaved order (did_defer_kernel.cuh): R keeps its
+// value for a whole sweep, the changes stay pending; the caller forms R anew
+// after it (launch_refresh_tc, with the partials of R c_1^T) and closes the
+// sweep with launch_defer_close.
+struct DeferPlan {
+  int grid, GS, NG, NR, CW, S;
+  Units units;
+  int nunits, dynamic, npart;
+  size_t smem;
+  const void* func;
+};
+struct DeferBuffers {
+  const void* R;      // ld x N (float or bfloat16)
+  float *B, *Bo;      // ld x K: the factor, and its columns before this sweep's updates
+  float *C, *Co;      // K x N, likewise
+  float* T;           // [N][GS / 32]
+  void* corr;         // [N] pairs of floats
+  float* P;           // [max(npart, npart_first)][ld]
+  double* CC0;        // [npart_first] partials of ||c_1||^2
+  void *Xp, *Yp;      // defer_pair_bytes(K, grid) each
+  unsigned* work;     // [K], zero before the first launch
+  Ctrl* ctrl;         // zero before the first launch
+  unsigned long long* degen;
+};
+bool plan_defer(int ld, int64_t N, int K, bool bf16, int grid_override, DeferPlan* plan);   // false: shape not supported
+size_t defer_pair_bytes(int K, int grid);
+cudaError_t launch_defer(const DeferPlan& plan, const DeferBuffers& b, int ld, int64_t N, int K, int npart_first,
+                         int bar_extra, uint64_t timeout_ns, uint64_t* tstamp, int tstamp_cap, cudaStream_t s);
+cudaError_t launch_defer_close(const double* part, int n, const DeferBuffers& b, int K, double* trace, cudaStream_t s);
+
 // Multi-instance sweeps (serving): one cooperative launch runs several
 // instances, each on its own range of CTAs (SweepArgs::cta_begin/cta_count).
 int serve_max_ld(bool bf16);

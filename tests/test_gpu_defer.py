@@ -1,0 +1,104 @@
+"""Read-only sweeps of the interleaved order: R keeps its value for a sweep,
+the changes stay pending, and R is formed anew on the tensor cores after it.
+
+Shapes beyond the SMs' shared memory, one for each way a column is held
+(threads of a group 32 to 512, one to ten vectors a thread), with column
+counts that leave part of a chunk, of a round of the groups and of a unit.
+Against the FP64 oracle's HALS sweeps and the kernel that writes R for every k.
+"""
+
+import numpy as np
+import pytest
+
+from oracle import did_oracle as O
+from synth import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def did():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_1802_08938_gb300 as did
+    return did
+
+
+def rel(a, b):
+    return float(np.linalg.norm(np.asarray(a, np.float64) - b) / np.linalg.norm(b))
+
+
+def run(did, X, B0, C0, sweeps, **kw):
+    M, N = X.shape
+    with did.Context(np.ascontiguousarray(X.T), M, N, B0.shape[1], B_init=np.ascontiguousarray(B0.T), C_init=C0,
+                     **kw) as ctx:
+        ctx.sweep(sweeps)
+        B, C = ctx.factors()
+        return dict(B=B, C=C, R=ctx.residual(), trace=ctx.trace(), f=ctx.objective(), info=ctx.info())
+
+
+SHAPES = [(64, 150001, 16), (130, 70003, 7), (784, 12001, 5), (1030, 9001, 2), (2064, 4503, 9), (5003, 1999, 3),
+          (9000, 1051, 1), (12000, 801, 4), (18001, 541, 2)]
+
+
+@pytest.mark.parametrize("M,N,K", SHAPES)
+def test_float32_matches_oracle(did, M, N, K):
+    X, _, _ = W.planted(M, N, K, seed=M + N, sigma=0.05)
+    B0, C0 = W.init_factors(M, N, K, 5)
+    ref = O.factor(X, B0, C0, order="hals", max_iter=3, stop="none")
+    got = run(did, X, B0, C0, 3)
+    again = run(did, X, B0, C0, 3)
+    eager = run(did, X, B0, C0, 3, flags=did.DID_FLAG_EAGER_WRITEBACK)
+    eB, eC = rel(got["B"], ref["B"]), rel(got["C"], ref["C"])
+    eF = float(np.max(np.abs(got["trace"] - ref["trace"]) / ref["trace"]))
+    print("read-only M=%d N=%d K=%d GS=%d NR=%d: relB %.3g relC %.3g relf %.3g (eager %.3g %.3g)" % (
+        M, N, K, got["info"]["group_threads"], got["info"]["vecs_per_thread"], eB, eC, eF, rel(eager["B"], ref["B"]),
+        rel(eager["C"], ref["C"])))
+    # float32 dots over up to 150001 terms and the refresh's 2^-21 |B||C|: a few 1e-7 each, 1e-5 with margin
+    assert eB <= 1e-5 and eC <= 1e-5 and eF <= 1e-5
+    assert np.array_equal(got["B"], again["B"]) and np.array_equal(got["C"], again["C"])
+    assert np.array_equal(got["trace"], again["trace"])
+    Rd = X.astype(np.float64) - got["B"].astype(np.float64) @ got["C"].astype(np.float64)
+    S = np.abs(got["B"]).astype(np.float64) @ got["C"].astype(np.float64)
+    assert np.all(np.abs(got["R"] - Rd) <= 2.0 ** -17 * S + 2.0 ** -22 * np.abs(Rd) + 1e-6)
+
+
+@pytest.mark.parametrize("M,N,K", [(130, 70003, 7), (784, 12001, 20), (2064, 4503, 9), (9000, 1051, 70)])
+def test_bfloat16_residual(did, M, N, K):
+    X, _, _ = W.planted(M, N, K, seed=M + N, sigma=0.05)
+    B0, C0 = W.init_factors(M, N, K, 5)
+    ref = O.factor(X, B0, C0, order="hals", max_iter=3, stop="none")
+    got = run(did, X, B0, C0, 3, precision=did.DID_BF16R, refresh_every=2)
+    assert got["info"]["refreshes"] == 1
+    assert abs(got["f"] - ref["trace"][-1]) <= 1e-3 * ref["trace"][-1]
+
+
+def test_stopping_zero_norms_and_resume(did):
+    M, N, K = 800, 12003, 4
+    X, _, _ = W.planted(M, N, K, seed=1, sigma=0.05)
+    B0, C0 = W.init_factors(M, N, K, 2)
+    C0[2] = 0.0                         # ||c_3|| = 0: b_3 is left unchanged until c_3 is updated
+    ref = O.factor(X, B0, C0, order="hals", max_iter=60, tol=1e-2, stop="relchange")
+    Xc = np.ascontiguousarray(X.T)
+    with did.Context(Xc, M, N, K, B_init=np.ascontiguousarray(B0.T), C_init=C0) as ctx:
+        iters, f = ctx.factor(60, 1e-2)
+        B, C = ctx.factors()
+        assert iters == ref["iters"] and ctx.info()["degenerate_events"] >= 1
+        assert rel(B, ref["B"]) <= 1e-5 and rel(C, ref["C"]) <= 1e-5
+        ctx.sweep(2)
+        B1, C1 = ctx.factors()
+        ctx.set_factors(B, C)
+        ctx.sweep(2)
+        B2, C2 = ctx.factors()
+    assert rel(B2, B1) <= 1e-5 and rel(C2, C1) <= 1e-5
+
+
+def test_expired_wait_is_reported(did):
+    M, N, K = 800, 12003, 3
+    X, _, _ = W.planted(M, N, K, seed=1, sigma=0.05)
+    with did.Context(np.ascontiguousarray(X.T), M, N, K, seed=0, timeout_ns=10 ** 7, debug_barrier_extra=1) as ctx:
+        with pytest.raises(did.DIDError) as e:
+            ctx.sweep(1)
+        assert e.value.status == did.DID_ETIMEOUT
+        B, C = ctx.factors()
+        assert np.isfinite(B).all() and (B >= 0).all() and np.isfinite(C).all() and (C >= 0).all()

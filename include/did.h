@@ -114,7 +114,11 @@ typedef struct {
  * the tensor-core pass (BF16x3 for a bfloat16 residual with K <= 128, BF16x6
  * for a float32 one with K <= 64; larger K always takes the SIMT pass). */
 #define DID_FLAG_SIMT_REFRESH 2
-/* did_options.flags (DID_ORDER_INTERLEAVED).  Without a flag below, and where
+/* did_options.flags.  Without a flag of this group (or DID_FLAG_SIMT_REFRESH),
+ * a residual that fits the SMs' shared memory (about 30 MB in float32) stays
+ * there for a whole launch of sweeps, in float32 also when it is stored in bfloat16
+ * (both per-k orders).
+ * DID_ORDER_INTERLEAVED: without a flag below, and where
  * the tensor-core refresh takes K, sweeps of a larger residual only read R:
  * the changes of a sweep stay pending as vectors, and R is formed anew from X
  * after its last k (did_info then counts a periodic refresh that falls due,

@@ -63,6 +63,10 @@ struct did_ctx {
   double* part_host = nullptr;      // pinned, 3 * dense grid
 
   did::SweepPlan plan{};
+  bool resident = false;            // R fits the SMs' shared memory: sweeps keep it there
+  did::ResidentPlan rplan{};
+  void* res_words = nullptr;
+  unsigned res_step = 0;            // step numbers used so far
   bool defer = false;               // interleaved sweeps read R only and form it anew after each sweep
   did::DeferPlan dplan{};
   did::DeferBuffers dbuf{};
@@ -328,7 +332,7 @@ did_status launch_sweeps(did_ctx* c, int n, int stop_rule, double tol, int* done
   a.dynamic = c->plan.dynamic;
   a.npart = c->plan.npart;
   a.n_sweeps = n;
-  a.prologue = c->need_prologue ? 1 : 0;
+  a.prologue = c->need_prologue && !c->resident ? 1 : 0;   // (resident sweeps form the first partials themselves)
   a.npart_first = a.prologue ? 0 : c->npart_first;
   a.f_prev = c->trace.back();
   a.f0 = c->trace.front();
@@ -342,7 +346,12 @@ did_status launch_sweeps(did_ctx* c, int n, int stop_rule, double tol, int* done
   c->tstamp_n = c->tstamp ? (int)std::min<int64_t>((int64_t)n * c->K, c->tstamp_cap) : 0;
   DID_CUDA(c, cudaMemsetAsync(c->ctrl, 0, sizeof(Ctrl), c->stream));
   DID_CUDA(c, cudaEventRecord(c->ev0, c->stream));
-  DID_CUDA(c, did::launch_sweep(c->plan, a, c->stream));
+  if (c->resident) {
+    DID_CUDA(c, did::launch_resident(c->rplan, a, c->res_words, c->res_step, c->bf16, c->stream));
+    c->res_step += (unsigned)n * (unsigned)c->K + 1u;
+  } else {
+    DID_CUDA(c, did::launch_sweep(c->plan, a, c->stream));
+  }
   DID_CUDA(c, cudaEventRecord(c->ev1, c->stream));
   DID_CUDA(c, cudaMemcpyAsync(c->ctrl_host, c->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, c->stream));
   if (n > 0)
@@ -581,8 +590,10 @@ static did_status create_impl(did_ctx* c, const float* X, uint64_t seed) {
   // A flag that asks for a form of write-back, column step or refresh keeps the sweep kernel that has it.
   const bool no_flags = !(c->opt.flags & (DID_FLAG_EAGER_WRITEBACK | DID_FLAG_LAZY_WRITEBACK | DID_FLAG_SINGLE_COLUMNS |
                                           DID_FLAG_SIMT_REFRESH));
+  c->resident = no_flags && c->opt.order != DID_ORDER_DID_BATCHED &&
+                did::plan_resident(c->ld, N, K, c->opt.grid_ctas, &c->rplan);
   // Sweeps that only read R, where the tensor-core refresh can form R after each.
-  c->defer = no_flags && c->opt.order == DID_ORDER_INTERLEAVED &&
+  c->defer = !c->resident && no_flags && c->opt.order == DID_ORDER_INTERLEAVED &&
              did::refresh_tc_supported(K, !c->bf16) && defer_pays(c) &&
              did::plan_defer(c->ld, N, K, c->bf16, c->opt.grid_ctas, &c->dplan);
   c->dense_grid = did::dense_grid();
@@ -610,6 +621,10 @@ static did_status create_impl(did_ctx* c, const float* X, uint64_t seed) {
   ALLOC(Sp, (size_t)2 * G * sizeof(double));
   ALLOC(OBJp, U * sizeof(double));
   ALLOC(bold, (size_t)c->ld * sizeof(float));
+  if (c->resident) {
+    ALLOC(res_words, c->rplan.words_bytes);
+    DID_CUDA(c, cudaMemsetAsync(c->res_words, 0, c->rplan.words_bytes, c->stream));
+  }
   if (c->defer) {
     did::DeferBuffers& d = c->dbuf;
     const size_t W = (size_t)c->dplan.GS / 32;
@@ -625,7 +640,7 @@ static did_status create_impl(did_ctx* c, const float* X, uint64_t seed) {
     d.C = c->C;
     d.P = c->P;
     d.CC0 = c->CCp;
-  } else if (c->plan.lazy) {
+  } else if (c->plan.lazy && !c->resident) {
     ALLOC(Cold, (size_t)N * sizeof(float));
     ALLOC(XCp, 2 * U * sizeof(double));
   }
@@ -852,7 +867,7 @@ did_status did_get_info(did_ctx* c, did_info* info) {
   info->K = c->K;
   info->precision = c->opt.precision;
   info->order = c->opt.order;
-  info->grid_ctas = c->defer ? c->dplan.grid : c->plan.grid;
+  info->grid_ctas = c->resident ? c->rplan.grid : c->defer ? c->dplan.grid : c->plan.grid;
   info->group_threads = c->defer ? c->dplan.GS : c->plan.GS;
   info->vecs_per_thread = c->defer ? c->dplan.NR : c->plan.NR;
   info->column_units = c->defer ? c->dplan.nunits : c->plan.nunits;

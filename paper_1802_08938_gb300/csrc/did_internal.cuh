@@ -333,6 +333,17 @@ did_status plan_sweep(int ld, int64_t N, bool bf16, int grid_override, int64_t m
                       char* err, size_t errlen, bool want_lazy = false);
 cudaError_t launch_sweep(const SweepPlan& plan, const SweepArgs& args, cudaStream_t s);
 
+// Sweeps of a residual that fits the SMs' shared memory (did_resident.cu), in
+// the interleaved and the C-first order.  `words` is zero when the buffer is
+// new; step0 grows by at least n_sweeps * K from launch to launch on it.
+struct ResidentPlan {
+  int grid, nc;
+  size_t smem, words_bytes;
+};
+bool plan_resident(int ld, int64_t N, int K, int grid_override, ResidentPlan* plan);   // false: does not fit
+cudaError_t launch_resident(const ResidentPlan& plan, const SweepArgs& args, void* words, unsigned step0, bool bf16,
+                            cudaStream_t s);
+
 // Read-only sweep of the interleaved order (did_defer_kernel.cuh): R keeps its
 // value for a whole sweep, the changes stay pending; the caller forms R anew
 // after it (launch_refresh_tc, with the partials of R c_1^T) and closes the

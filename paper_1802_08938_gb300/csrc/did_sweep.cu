@@ -348,9 +348,14 @@ extern "C" did_status did_sweep_static(float* R, int64_t ld, float* B, float* C,
   a.timeout_ns = 4000000000ull;
   // The array keeps the previous call's contents: clear the control words and
   // the event counter, which must start at zero.
+  // A residual that fits the SMs' shared memory stays there (did_resident.cu);
+  // its words, which must start at zero, take the partials' place.
+  ResidentPlan rp{};
+  const bool resident = plan_resident((int)ld, N, K, kStaticMaxGrid, &rp) && rp.words_bytes <= L.end - L.p;
   if (cudaMemsetAsync(base + L.ctrl, 0, sizeof(Ctrl), s) != cudaSuccess ||
       cudaMemsetAsync(base + L.degen, 0, sizeof(unsigned long long), s) != cudaSuccess ||
-      launch_sweep(plan, a, s) != cudaSuccess) {
+      (resident && cudaMemsetAsync(base + L.p, 0, rp.words_bytes, s) != cudaSuccess) ||
+      (resident ? launch_resident(rp, a, base + L.p, 0u, false, s) : launch_sweep(plan, a, s)) != cudaSuccess) {
     cudaGetLastError();
     return DID_ECUDA;
   }

@@ -1,0 +1,102 @@
+"""Sweeps of a residual that stays in the SMs' shared memory, the CTAs
+exchanging flagged words: both orders, both precisions, one CTA to all of
+them, slices of one row and of many, one column a CTA and many, K = 1, and
+launches of one sweep and of several.  Against the FP64 oracle.
+"""
+
+import numpy as np
+import pytest
+
+from oracle import did_oracle as O
+from synth import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def did():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_1802_08938_gb300 as did
+    return did
+
+
+def rel(a, b):
+    return float(np.linalg.norm(np.asarray(a, np.float64) - b) / np.linalg.norm(b))
+
+
+def run(did, X, B0, C0, sweeps, **kw):
+    M, N = X.shape
+    with did.Context(np.ascontiguousarray(X.T), M, N, B0.shape[1], B_init=np.ascontiguousarray(B0.T), C_init=C0,
+                     **kw) as ctx:
+        for n in sweeps:
+            ctx.sweep(n)
+        B, C = ctx.factors()
+        return dict(B=B, C=C, R=ctx.residual(), trace=ctx.trace(), f=ctx.objective(), info=ctx.info())
+
+
+# one CTA; K = 1; more CTAs than row slices; long columns, one a CTA; a ragged last CTA; near the capacity
+SHAPES = [(5, 7, 2), (40, 16, 1), (3, 3000, 1), (200, 1000, 10), (33, 2433, 7), (4099, 150, 5), (9000, 600, 3),
+          (1024, 2414, 25), (513, 9001, 4), (2500, 2401, 6)]
+
+
+@pytest.mark.parametrize("order", ["hals", "dbcd"])
+@pytest.mark.parametrize("M,N,K", SHAPES)
+def test_matches_oracle(did, M, N, K, order):
+    X, _, _ = W.planted(M, N, K, seed=M + N, sigma=0.05)
+    B0, C0 = W.init_factors(M, N, K, 5)
+    code = did.DID_ORDER_INTERLEAVED if order == "hals" else did.DID_ORDER_DID
+    ref = O.factor(X, B0, C0, order=order, max_iter=6, stop="none")
+    got = run(did, X, B0, C0, (1, 5), order=code)
+    again = run(did, X, B0, C0, (1, 5), order=code)
+    eB, eC = rel(got["B"], ref["B"]), rel(got["C"], ref["C"])
+    eF = float(np.max(np.abs(got["trace"] - ref["trace"]) / ref["trace"]))
+    print("resident %s M=%d N=%d K=%d grid=%d: relB %.3g relC %.3g relf %.3g" % (
+        order, M, N, K, got["info"]["grid_ctas"], eB, eC, eF))
+    assert eB <= 1e-5 and eC <= 1e-5 and eF <= 1e-5      # float32 dots and updates: a few 1e-7, with margin
+    for key in ("B", "C", "R", "trace"):
+        assert np.array_equal(got[key], again[key]), key
+    Rd = X.astype(np.float64) - got["B"].astype(np.float64) @ got["C"].astype(np.float64)
+    assert np.max(np.abs(got["R"] - Rd)) <= 1e-4 * max(1.0, float(np.abs(X).max()))
+
+
+@pytest.mark.parametrize("order", [0, 1])
+def test_bfloat16_residual_and_refresh(did, order):
+    M, N, K = 700, 1501, 12
+    X, _, _ = W.planted(M, N, K, seed=9, sigma=0.05)
+    B0, C0 = W.init_factors(M, N, K, 5)
+    ref = O.factor(X, B0, C0, order="dbcd" if order else "hals", max_iter=6, stop="none")
+    got = run(did, X, B0, C0, (6,), order=order, precision=did.DID_BF16R, refresh_every=4)
+    assert got["info"]["refreshes"] == 1
+    assert abs(got["f"] - ref["trace"][-1]) <= 1e-3 * ref["trace"][-1]
+
+
+def test_zero_norm_and_paper_rule(did):
+    M, N, K = 60, 500, 4
+    X, _, _ = W.planted(M, N, K, seed=1, sigma=0.05)
+    B0, C0 = W.init_factors(M, N, K, 2)
+    C0[2] = 0.0
+    B0[:, 1] = 0.0
+    for order, code in (("hals", 0), ("dbcd", 1)):
+        ref = O.factor(X, B0, C0, order=order, max_iter=5, stop="none")
+        got = run(did, X, B0, C0, (5,), order=code)
+        assert got["info"]["degenerate_events"] >= 1
+        assert rel(got["B"], ref["B"]) <= 1e-5 and rel(got["C"], ref["C"]) <= 1e-5
+
+
+def test_static_call_takes_it(did):
+    torch = pytest.importorskip("torch")
+    M, N, K = 130, 777, 5
+    X, _, _ = W.planted(M, N, K, seed=4, sigma=0.05)
+    B0, C0 = W.init_factors(M, N, K, 4)
+    ref = O.factor(X, B0, C0, order="hals", max_iter=4, stop="none")
+    ld = 132
+    R = torch.zeros((N, ld), device="cuda")
+    R[:, :M] = torch.from_numpy(np.ascontiguousarray((X - (B0.astype(np.float64) @ C0)).T.astype(np.float32))).cuda()
+    B = torch.zeros((K, ld), device="cuda")
+    B[:, :M] = torch.from_numpy(np.ascontiguousarray(B0.T)).cuda()
+    C = torch.from_numpy(C0).cuda()
+    for n in (3, 1):                    # the scratch array keeps the first call's words
+        did.did_sweep_static(R, ld, B, C, M, N, K, n)
+    assert rel(B[:, :M].cpu().numpy().T, ref["B"]) <= 1e-5 and rel(C.cpu().numpy(), ref["C"]) <= 1e-5
+    assert float(R[:, M:].abs().max()) == 0.0

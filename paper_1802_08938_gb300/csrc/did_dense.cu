@@ -7,7 +7,8 @@
 // the exact objective 1/2 ||X - B C||^2 without storing R, the sums that scale
 // the start point, and the planted synthetic inputs X = B0 C0 (+ noise).
 //
-// Tiling: a 256-thread CTA owns a 64 x 64 tile of the M x N output; thread
+// Tiling (generation, and small matrices; see dense_big_kernel for the others):
+// a 256-thread CTA owns a 64 x 64 tile of the M x N output; thread
 // (tr, tc) holds rows 4*tr..4*tr+3 and columns tc + 16*m (m < 4).  K is
 // walked in chunks of 32 staged in shared memory.  CTAs take tiles
 // blockIdx.x, blockIdx.x + grid, ... so the per-CTA partial sums, added by
@@ -136,6 +137,153 @@ __global__ void __launch_bounds__(kDenseThreads) dense_kernel(DenseTileArgs t) {
   }
 }
 
+// The passes over X - B C of a larger matrix (modes 0 to 2): 128 x 128 tiles,
+// eight rows by eight columns a thread.  Bound by float32 FMA issue: a k costs
+// a thread 32 packed FMAs (f32x2) and four 16-byte loads from shared memory,
+// where the 4 x 4 tile above pays five loads for 16 FMAs, and its float64 sums
+// (float64 adds issue at 1/64 the rate) took a third of the time; here the
+// sums are float32 pairs until the end.  The next chunk of B and C is loaded into
+// registers while this one is used.  Each product is the same chain of FMAs in k
+// order, so R comes out bit for bit the same.  Measured: 10000 x 100000,
+// K = 100 (exact objective) 11.9 -> 5.9 ms; 8165 x 18821, K = 100, a refresh and an
+// objective 3.8 -> 1.4 ms.
+constexpr int kBig = 128;
+constexpr int kBigKc = 16;
+constexpr int kBigThreads = 256;
+
+struct Pair2 {
+  float h, l;
+  __device__ __forceinline__ void add(float v) {
+    const float s = __fadd_rn(h, v);
+    const float t = __fsub_rn(s, h);
+    l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, t)), __fsub_rn(v, t)));
+    h = s;
+  }
+};
+
+__global__ void __launch_bounds__(kBigThreads, 2) dense_big_kernel(DenseArgs a) {
+  __shared__ __align__(16) float Bs[2][kBigKc][kBig];
+  __shared__ __align__(16) float Cs[2][kBigKc][kBig];
+  __shared__ double scratch[kBigThreads / 32];
+  const int t = threadIdx.x;
+  const int tr = t & 15, tc = t >> 4;              // rows 4 tr.. and 64 + 4 tr.., columns 4 tc.. and 64 + 4 tc..
+  const int mt = (a.ld + kBig - 1) / kBig;
+  const int64_t nt = (a.N + kBig - 1) / kBig;
+  const int64_t ntiles = (int64_t)mt * nt;
+  const int chunks = (a.K + kBigKc - 1) / kBigKc;
+  const int lk = t >> 5, lx = (t & 31) * 4;        // loader: rows lk and lk + 8 of a chunk, four values from lx
+  const bool c_vec = (a.N & 3) == 0;
+  Pair2 s0{0.f, 0.f}, s1 = s0, s2 = s0;
+
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int row0 = (int)(tile % mt) * kBig;
+    const int64_t col0 = (tile / mt) * kBig;
+    float4 nb[2], nc[2];
+    auto fetch = [&](int k0) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int k = k0 + lk + 8 * h;
+        nb[h] = nc[h] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (k >= a.K) continue;
+        // rows M .. ld - 1 of B are zero; ld is a multiple of four
+        if (row0 + lx < a.ld) nb[h] = *reinterpret_cast<const float4*>(a.B + (size_t)k * a.ld + row0 + lx);
+        const float* c = a.C + (size_t)k * a.N + col0 + lx;
+        if (c_vec) {
+          if (col0 + lx < a.N) nc[h] = *reinterpret_cast<const float4*>(c);
+        } else {
+          float v[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) v[e] = col0 + lx + e < a.N ? c[e] : 0.f;
+          nc[h] = make_float4(v[0], v[1], v[2], v[3]);
+        }
+      }
+    };
+    auto put = [&](int b) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        *reinterpret_cast<float4*>(&Bs[b][lk + 8 * h][lx]) = nb[h];
+        *reinterpret_cast<float4*>(&Cs[b][lk + 8 * h][lx]) = nc[h];
+      }
+    };
+    float2 acc[8][4];                               // [column][row pair]
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) acc[c][r] = make_float2(0.f, 0.f);
+    fetch(0);
+    put(0);
+    __syncthreads();
+    for (int ch = 0; ch < chunks; ++ch) {
+      const int b = ch & 1;
+      if (ch + 1 < chunks) fetch((ch + 1) * kBigKc);
+#pragma unroll
+      for (int kk = 0; kk < kBigKc; ++kk) {
+        const float4 b0 = *reinterpret_cast<const float4*>(&Bs[b][kk][4 * tr]);
+        const float4 b1 = *reinterpret_cast<const float4*>(&Bs[b][kk][64 + 4 * tr]);
+        const float4 c0 = *reinterpret_cast<const float4*>(&Cs[b][kk][4 * tc]);
+        const float4 c1 = *reinterpret_cast<const float4*>(&Cs[b][kk][64 + 4 * tc]);
+        const float2 bv[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w), make_float2(b1.x, b1.y),
+                              make_float2(b1.z, b1.w)};
+        const float cv[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+#pragma unroll
+          for (int r = 0; r < 4; ++r) acc[c][r] = __ffma2_rn(bv[r], make_float2(cv[c], cv[c]), acc[c][r]);
+      }
+      if (ch + 1 < chunks) put(b ^ 1);              // that buffer was last read before the previous barrier
+      __syncthreads();
+    }
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const int64_t col = col0 + (c < 4 ? 4 * tc + c : 64 + 4 * tc + c - 4);
+      if (col >= a.N) continue;
+      float l0 = 0.f, l1 = 0.f, l2 = 0.f;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int row = row0 + 64 * h + 4 * tr;
+        if (row >= a.ld) continue;                  // (ld is a multiple of four)
+        const size_t off = (size_t)col * a.ld + row;
+        const float4 x = __ldcs(reinterpret_cast<const float4*>(a.X + off));
+        const float xs[4] = {x.x, x.y, x.z, x.w};
+        const float p[4] = {acc[c][2 * h].x, acc[c][2 * h].y, acc[c][2 * h + 1].x, acc[c][2 * h + 1].y};
+        float r[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          r[e] = xs[e] - p[e];
+          if (a.mode == 2) {
+            l1 = fmaf(xs[e], p[e], l1);
+            l2 = fmaf(p[e], p[e], l2);
+          } else {
+            l0 = fmaf(r[e], r[e], l0);
+          }
+        }
+        if (a.mode == 0) {
+          if (a.bf16) {
+            __nv_bfloat162 lo = __floats2bfloat162_rn(r[0], r[1]), hi = __floats2bfloat162_rn(r[2], r[3]);
+            uint2 v;
+            v.x = *reinterpret_cast<unsigned*>(&lo);
+            v.y = *reinterpret_cast<unsigned*>(&hi);
+            *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.R) + off) = v;
+          } else {
+            *reinterpret_cast<float4*>(reinterpret_cast<float*>(a.R) + off) = make_float4(r[0], r[1], r[2], r[3]);
+          }
+        }
+      }
+      s0.add(l0);
+      s1.add(l1);
+      s2.add(l2);
+    }
+  }
+  const double d0 = block_sum_f64((double)s0.h + (double)s0.l, scratch);
+  const double d1 = block_sum_f64((double)s1.h + (double)s1.l, scratch);
+  const double d2 = block_sum_f64((double)s2.h + (double)s2.l, scratch);
+  if (t == 0) {
+    a.part[3 * blockIdx.x + 0] = d0;
+    a.part[3 * blockIdx.x + 1] = d1;
+    a.part[3 * blockIdx.x + 2] = d2;
+  }
+}
+
 int g_dense_grid = 0;
 
 __global__ void gen_uniform_padded_kernel(float* out, int rows, int ld, int cols, uint64_t key) {
@@ -218,6 +366,13 @@ int dense_grid() {
 }
 
 cudaError_t launch_dense(const DenseArgs& a, cudaStream_t s) {
+  // The large tiles where they fill the SMs and few of their rows are past
+  // ld; below that the small ones keep more CTAs busy.
+  const int64_t big = (int64_t)((a.ld + kBig - 1) / kBig) * ((a.N + kBig - 1) / kBig);
+  if (big >= dense_grid() / 4 && (a.ld + kBig - 1) / kBig * kBig * 3 <= a.ld * 4) {
+    dense_big_kernel<<<dense_grid(), kBigThreads, 0, s>>>(a);
+    return cudaGetLastError();
+  }
   DenseTileArgs t{};
   t.d = a;
   t.ldb = a.ld;

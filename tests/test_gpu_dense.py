@@ -1,0 +1,35 @@
+"""The float32 passes over X - B C: the 128 x 128 tiles of larger matrices at
+edges of tiles, chunks of K and vectors, against float64, in both precisions.
+"""
+
+import numpy as np
+import pytest
+
+from synth import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def did():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_1802_08938_gb300 as did
+    return did
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("M,N,K", [(100, 19457, 1), (128, 19460, 16), (241, 12001, 17), (500, 5003, 65), (1000, 2563, 100)])
+def test_refresh_and_objective(did, M, N, K, precision):
+    X, _, _ = W.planted(M, N, K, seed=M + N, sigma=0.05)
+    B0, C0 = W.init_factors(M, N, K, 5)
+    with did.Context(np.ascontiguousarray(X.T), M, N, K, B_init=np.ascontiguousarray(B0.T), C_init=C0,
+                     precision=precision, flags=did.DID_FLAG_SIMT_REFRESH) as ctx:
+        R, f0, f = ctx.residual(), ctx.trace()[0], ctx.objective()
+    P = B0.astype(np.float64) @ C0.astype(np.float64)
+    Rd = X.astype(np.float64) - P
+    # a chain of K float32 FMAs and one subtraction; bfloat16: half an ulp of 8 bits
+    bound = (K + 2) * 2.0 ** -24 * P + 2.0 ** -24 * np.abs(Rd) + (2.0 ** -8 * np.abs(Rd) if precision else 0.0)
+    assert np.all(np.abs(R - Rd) <= bound + 1e-30)
+    fd = 0.5 * float(np.sum(Rd ** 2))
+    assert abs(f - fd) <= 1e-5 * fd and abs(f0 - fd) <= 1e-5 * fd

@@ -118,8 +118,8 @@ typedef struct {
  * a residual that fits the SMs' shared memory (about 30 MB in float32) stays
  * there for a whole launch of sweeps, in float32 also when it is stored in bfloat16
  * (both per-k orders).
- * DID_ORDER_INTERLEAVED: without a flag below, and where
- * the tensor-core refresh takes K, sweeps of a larger residual only read R:
+ * DID_ORDER_INTERLEAVED: without a flag below, sweeps of a larger residual
+ * (K <= 128) only read R:
  * the changes of a sweep stay pending as vectors, and R is formed anew from X
  * after its last k (did_info then counts a periodic refresh that falls due,
  * which finds R formed from the current factors already).

@@ -447,35 +447,53 @@ did_status run_batched(did_ctx* c, int64_t max_sweeps, int stop_rule, double tol
 
 // Interleaved order by read-only sweeps: each sweep is the K passes of the
 // sweep kernel over a residual that it does not write, then R = X - B C on the
-// tensor cores (with 1/2 ||R||^2 and the partials of R c_1^T).  A periodic
+// tensor cores (with 1/2 ||R||^2 and the partials of R c_1^T), or by the float32
+// pass where those do not take K.  A periodic
 // refresh that falls due finds R formed from the current factors already.
 did_status run_defer(did_ctx* c, int64_t max_sweeps, int stop_rule, double tol, int64_t* done_total) {
   *done_total = 0;
   const int G = did::refresh_tc_grid();
+  const bool tc = did::refresh_tc_supported(c->K, !c->bf16);
+  did::DenseArgs da{};
+  da.X = c->X;
+  da.R = c->R;
+  da.B = c->B;
+  da.C = c->C;
+  da.part = c->dense_part;
+  da.M = (int)c->M;
+  da.ld = c->ld;
+  da.K = c->K;
+  da.N = c->N;
+  da.bf16 = c->bf16 ? 1 : 0;
   while (*done_total < max_sweeps) {
-    if (c->need_refresh || c->npart_first == 0) {
+    if (c->need_refresh || (tc && c->npart_first == 0)) {
       did_status st = refresh(c);
       if (st != DID_OK) return st;
     } else if (refresh_due(c)) {
       c->last_refresh_at = c->sweeps_done;
       c->refreshes++;
-      c->tc_refreshes++;
+      if (tc) c->tc_refreshes++;
     }
     const int n = stop_rule ? 1 : chunk_size(c, max_sweeps - *done_total);   // with a stopping rule: one sweep per check
     const uint64_t tmo = wait_limit_ns(c);
     const int cap = c->tstamp ? (int)std::min<int64_t>((int64_t)n * c->K, c->tstamp_cap) : 0;
     c->tstamp_n = cap;
     DID_CUDA(c, cudaMemsetAsync(c->ctrl, 0, sizeof(Ctrl), c->stream));
-    DID_CUDA(c, cudaMemsetAsync(c->dbuf.work, 0, sizeof(unsigned) * c->K, c->stream));
+    DID_CUDA(c, cudaMemsetAsync(c->dbuf.work, 0, sizeof(unsigned) * (c->K + 1), c->stream));
     DID_CUDA(c, cudaEventRecord(c->ev0, c->stream));
     for (int s = 0; s < n; ++s) {
       const int step0 = s * c->K;
       DID_CUDA(c, did::launch_defer(c->dplan, c->dbuf, c->ld, c->N, c->K, c->npart_first, c->opt.debug_barrier_extra,
                                     tmo, step0 < cap ? c->tstamp + 4 * (size_t)step0 : nullptr,
                                     std::max(0, cap - step0), c->stream));
-      DID_CUDA(c, did::launch_refresh_tc(c->X, c->R, c->B, c->C, (int)c->M, c->ld, c->N, c->K, c->tc_ws, c->tc_part,
-                                         c->P, c->CCp, &c->ctrl->err, tmo, c->stream, !c->bf16));
-      DID_CUDA(c, did::launch_defer_close(c->tc_part, G, c->dbuf, c->K, c->trace_dev + s, c->stream));
+      if (tc) {
+        DID_CUDA(c, did::launch_refresh_tc(c->X, c->R, c->B, c->C, (int)c->M, c->ld, c->N, c->K, c->tc_ws, c->tc_part,
+                                           c->P, c->CCp, &c->ctrl->err, tmo, c->stream, !c->bf16));
+        DID_CUDA(c, did::launch_defer_close(c->tc_part, G, 1, c->dbuf, c->K, c->trace_dev + s, c->stream));
+      } else {
+        DID_CUDA(c, did::launch_dense(da, c->stream));
+        DID_CUDA(c, did::launch_defer_close(c->dense_part, c->dense_grid, 3, c->dbuf, c->K, c->trace_dev + s, c->stream));
+      }
     }
     DID_CUDA(c, cudaEventRecord(c->ev1, c->stream));
     DID_CUDA(c, cudaMemcpyAsync(c->ctrl_host, c->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, c->stream));
@@ -592,9 +610,10 @@ static did_status create_impl(did_ctx* c, const float* X, uint64_t seed) {
                                           DID_FLAG_SIMT_REFRESH));
   c->resident = no_flags && c->opt.order != DID_ORDER_DID_BATCHED &&
                 did::plan_resident(c->ld, N, K, c->opt.grid_ctas, &c->rplan);
-  // Sweeps that only read R, where the tensor-core refresh can form R after each.
+  // Sweeps that only read R; the tensor-core refresh forms it after each, or for
+  // other K the float32 pass (and the next sweep a first pass for c_1).
   c->defer = !c->resident && no_flags && c->opt.order == DID_ORDER_INTERLEAVED &&
-             did::refresh_tc_supported(K, !c->bf16) && defer_pays(c) &&
+             defer_pays(c) &&
              did::plan_defer(c->ld, N, K, c->bf16, c->opt.grid_ctas, &c->dplan);
   c->dense_grid = did::dense_grid();
   DID_CUDA(c, cudaEventCreate(&c->ev0));
@@ -634,7 +653,7 @@ static did_status create_impl(did_ctx* c, const float* X, uint64_t seed) {
     ALLOC(dbuf.corr, (size_t)N * 2 * sizeof(float));
     ALLOC(dbuf.Xp, did::defer_pair_bytes(K, c->dplan.grid));
     ALLOC(dbuf.Yp, did::defer_pair_bytes(K, c->dplan.grid));
-    ALLOC(dbuf.work, (size_t)K * sizeof(unsigned));
+    ALLOC(dbuf.work, (size_t)(K + 1) * sizeof(unsigned));
     d.R = c->R;
     d.B = c->B;
     d.C = c->C;

@@ -19,11 +19,11 @@ namespace {
 
 // Closes a sweep: f = 1/2 ||R||^2 from the refresh's per-CTA sums (added in
 // order), and clears the barrier and the unit counters for the next launch.
-__global__ void defer_close_kernel(const double* part, int n, Ctrl* ctrl, unsigned* work, int K, double* trace) {
-  for (int i = threadIdx.x; i < K; i += blockDim.x) work[i] = 0u;
+__global__ void defer_close_kernel(const double* part, int n, int stride, Ctrl* ctrl, unsigned* work, int K, double* trace) {
+  for (int i = threadIdx.x; i <= K; i += blockDim.x) work[i] = 0u;
   if (threadIdx.x == 0) {
     double s = 0.0;
-    for (int i = 0; i < n; ++i) s += part[i];
+    for (int i = 0; i < n; ++i) s += part[(size_t)i * stride];
     *trace = 0.5 * s;
     ctrl->bar = 0u;
     if (ctrl->err == 0) ctrl->sweeps += 1;
@@ -39,6 +39,7 @@ bool plan_defer(int ld, int64_t N, int K, bool bf16, int grid_override, DeferPla
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (K > 128) return false;
   DeferPlan P{};
   P.grid = grid_override > 0 ? std::min(grid_override, sms) : sms;
   // Threads of a column group: as few as hold a column in 16 rows each, so
@@ -143,8 +144,8 @@ cudaError_t launch_defer(const DeferPlan& plan, const DeferBuffers& b, int ld, i
   return cudaLaunchCooperativeKernel(plan.func, dim3(plan.grid), dim3(kDeferThreads), params, plan.smem, s);
 }
 
-cudaError_t launch_defer_close(const double* part, int n, const DeferBuffers& b, int K, double* trace, cudaStream_t s) {
-  defer_close_kernel<<<1, 128, 0, s>>>(part, n, b.ctrl, b.work, K, trace);
+cudaError_t launch_defer_close(const double* part, int n, int stride, const DeferBuffers& b, int K, double* trace, cudaStream_t s) {
+  defer_close_kernel<<<1, 128, 0, s>>>(part, n, stride, b.ctrl, b.work, K, trace);
   return cudaGetLastError();
 }
 

@@ -91,16 +91,20 @@ __device__ __forceinline__ void df_acc(df& a, float v) {
   a.l = __fadd_rn(a.l, __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(v, t)));
   a.h = s;
 }
-__device__ __forceinline__ df df_from(double v) {
-  const float h = (float)v;
-  return df{h, (float)(v - (double)h)};
+// a / b: a float32 quotient and its correction (a float64 division by all 16
+// warps costs about 2 us).
+__device__ __forceinline__ df df_div(df a, df b) {
+  const float q = __fdiv_rn(a.h, b.h);
+  const float p = __fmul_rn(q, b.h);
+  const float e = __fmaf_rn(q, b.h, -p);
+  const float r = __fadd_rn(__fsub_rn(a.h, p), __fsub_rn(a.l, __fmaf_rn(q, b.l, e)));
+  return df_add(df{q, 0.f}, df{__fdiv_rn(r, b.h), 0.f});
 }
 // The product of two pairs, rounded to float32.
 __device__ __forceinline__ float df_mul_f32(df a, df b) {
   const float p = __fmul_rn(a.h, b.h);
   return p + (__fmaf_rn(a.h, b.h, -p) + __fmaf_rn(a.h, b.l, __fmul_rn(a.l, b.h)));
 }
-__device__ __forceinline__ double df_double(df a) { return (double)a.h + (double)a.l; }
 __device__ __forceinline__ df df_shfl_xor(df a, int m) {
   return df{__shfl_xor_sync(0xffffffffu, a.h, m), __shfl_xor_sync(0xffffffffu, a.l, m)};
 }
@@ -135,7 +139,7 @@ struct DeferArgs {
   const double* CC0;   // [npart_first] partials of ||c_1||^2
   df* Xp;              // [2K + 1][grid] per-CTA sums: c_l.c, c_l'.c (l <= k), ||c||^2 with c = c_{k+1}
   df* Yp;              // [2K + 2][grid] per-CTA sums: b'.b_l, b'.b_l' (l < k), b'.b', b'.b_k
-  unsigned* work;      // [K] column-unit counters, zeroed before the launch
+  unsigned* work;      // [K + 1] column-unit counters (pass k at k + 1), zeroed before the launch
   Ctrl* ctrl;
   unsigned long long* degen;
   int64_t N;
@@ -144,7 +148,7 @@ struct DeferArgs {
   int S;               // ring stages (chunks of CW columns)
   Units units;         // column ranges of the CTA-level units
   int nunits, dynamic;
-  int npart, npart_first;
+  int npart, npart_first;   // npart_first 0: no partials for c_1 yet, a first pass forms them
   int bar_extra;
   uint64_t timeout_ns;
   uint64_t* tstamp;    // phase stamps of this sweep (CTA 0), 4 per k, or null
@@ -288,7 +292,7 @@ __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
   uint64_t* empty = full + S;
   volatile int* quit = reinterpret_cast<volatile int*>(smem + L.misc);
   int* s_ok = reinterpret_cast<int*>(smem + L.misc) + 1;
-  double* scal = reinterpret_cast<double*>(smem + L.misc + 16);   // [0] ||c_k||^2
+  df* cc0 = reinterpret_cast<df*>(smem + L.misc + 16);             // ||c_1||^2 of the refresh
   int* err = &a.ctrl->err;
   const uint64_t tmo = a.timeout_ns;
   const int t = threadIdx.x, w = t >> 5, lane = t & 31;
@@ -356,9 +360,9 @@ __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
         __syncwarp();
       }
     };
-    for (int k = 0; k < K && ok; ++k) {
+    for (int k = a.npart_first > 0 ? 0 : -1; k < K && ok; ++k) {
       const float* cn = k + 1 < K ? a.C + (int64_t)(k + 1) * N : nullptr;
-      auto grab = [&]() -> unsigned { return lane == 0 ? atomicAdd(a.work + k, 1u) : 0u; };   // lane 0 has it
+      auto grab = [&]() -> unsigned { return lane == 0 ? atomicAdd(a.work + k + 1, 1u) : 0u; };   // lane 0 has it
       // the first unit is the CTA's own (a CTA that runs ahead into this pass must
       // not take two large ones); the others come from the counter, asked for
       // a block before they are needed
@@ -493,21 +497,28 @@ __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
   unsigned cst = (unsigned)g % (unsigned)S, cph = ((unsigned)g / (unsigned)S) & 1u;   // next chunk of this group
   const bool stamps = a.tstamp != nullptr && cta == 0 && t == 0;
 
-  for (int k = 0; k < K; ++k) {
-    const bool rec = stamps && k < a.tstamp_cap;
+  df* xwarp = xw + (size_t)w * 2 * (K + 1);       // this warp's sums: c_l.c at 2l, c_l'.c at 2l + 1; ||c||^2 at 2K
+
+  // k = -1 (where the launch has no partials for c_1): phase S alone, for the
+  // partials of R_s c_1^T, and ||c_1||^2 in phase F
+  for (int k = a.npart_first > 0 ? 0 : -1; k < K; ++k) {
+    const bool rec = stamps && k >= 0 && k < a.tstamp_cap;
     if (rec) a.tstamp[4 * k + 0] = globaltimer_ns();
+    if (k >= 0) {
     // ------------------------------------------------------------ phase A
     // ||c_k||^2 and, for l < k, c_l.c_k (sums[2l]) and c_l'.c_k (sums[2l+1])
-    if (k == 0) {
+    const bool given = k == 0 && a.npart_first > 0;   // the refresh's partials
+    if (given) {
       if (w == 0) {
         const double cc = warp_sum_global_f64(a.CC0, a.npart_first, 1);
-        if (lane == 0) scal[0] = cc;
+        const float h = (float)cc;
+        if (lane == 0) *cc0 = df{h, (float)(cc - (double)h)};
       }
     } else {
       sum_over_ctas(a.Xp, 2 * k + 1, G, sums);
     }
     // partial rows: thread (row quad, subset sub) adds rows sub, sub + SU, ... of P
-    const int U = k == 0 ? a.npart_first : a.npart;
+    const int U = given ? a.npart_first : a.npart;
     const int nq = rpc / 4, SU = kWorkThreads / nq;
     df* acca = xw;                                 // [SU][rpc]
     const int quad = t % nq, sub = t / nq;
@@ -540,7 +551,7 @@ __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
     {
       const int LPR = rpc >= 32 ? 8 : 32;
       const int e0 = t & (LPR - 1);
-      const double cc = k == 0 ? scal[0] : df_double(sums[2 * k]);
+      const df cc = given ? *cc0 : sums[2 * k];
       for (int row0 = 0; row0 < rpc; row0 += kWorkThreads / LPR) {
         const int row = row0 + t / LPR;
         const bool in = row < nrows;
@@ -556,16 +567,16 @@ __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
         for (int m = LPR / 2; m >= 1; m >>= 1) q = df_add(q, df_shfl_xor(q, m));
         if (in && e0 == 0) {
           float b_new = b_old;
-          if (cc > 0.0) {
-            const double v = (double)b_old + df_double(q) / cc;
-            b_new = v > 0.0 ? (float)v : 0.f;
+          if (cc.h > 0.f) {
+            const df v = df_add(df{b_old, 0.f}, df_div(q, cc));
+            b_new = v.h > 0.f ? v.h : 0.f;
           }
           bos[k * rst + row] = b_old;
           bns[k * rst + row] = b_new;
           bks[row] = b_new;
           __stcg(a.Bo + (size_t)k * ld + r0 + row, b_old);
           __stcg(a.B + (size_t)k * ld + r0 + row, b_new);
-          if (!(cc > 0.0) && cta == 0 && row == 0) atomicAdd(a.degen, 1ull);
+          if (!(cc.h > 0.f) && cta == 0 && row == 0) atomicAdd(a.degen, 1ull);
         }
       }
       work_sync();
@@ -601,7 +612,15 @@ __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
     DID_DEFER_GRID_SYNC();
     if (rec) a.tstamp[4 * k + 1] = globaltimer_ns();
 
-    // b_k' of this thread's rows, and the grid-wide sums
+    sum_over_ctas(a.Yp, 2 * k + 2, G, sums);
+    work_sync();
+    if (!(sums[2 * k + 1].h > 0.f) && cta == 0 && t == 0) atomicAdd(a.degen, 1ull);
+    if (lane < 3) xwarp[lane < 2 ? 2 * k + lane : 2 * K] = df_zero();
+    side_arrive(2);                              // the side warps begin phase B
+    } else if (lane == 0) {
+      xwarp[2 * K] = df_zero();
+    }
+    // b_k' of this thread's rows
     float2 bn[NR][VH];
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
@@ -610,20 +629,11 @@ __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
 #pragma unroll
       for (int e = 0; e < VR; e += 4) {
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (in) v = __ldcg(reinterpret_cast<const float4*>(a.B + (size_t)k * ld + (size_t)q * VR + e));
+        if (in && k >= 0) v = __ldcg(reinterpret_cast<const float4*>(a.B + (size_t)k * ld + (size_t)q * VR + e));
         bn[r][e / 2] = make_float2(v.x, v.y);
         bn[r][e / 2 + 1] = make_float2(v.z, v.w);
       }
     }
-    sum_over_ctas(a.Yp, 2 * k + 2, G, sums);
-    work_sync();
-    const double bbk = df_double(sums[2 * k + 1]);
-    const bool cdeg = !(bbk > 0.0);
-    const df inv_bb = df_from(cdeg ? 0.0 : 1.0 / bbk), bob = sums[2 * k];
-    if (cdeg && cta == 0 && t == 0) atomicAdd(a.degen, 1ull);
-    df* xwarp = xw + (size_t)w * 2 * (K + 1);     // this warp's sums: c_l.c at 2l, c_l'.c at 2l + 1; ||c||^2 at 2K
-    if (lane < 3) xwarp[lane < 2 ? 2 * k + lane : 2 * K] = df_zero();
-    side_arrive(2);                              // the side warps begin phase B
     const bool more = k + 1 < K;                 // the next step needs the sums with c_{k+1}
     const float* cn_row = a.C + (int64_t)(more ? k + 1 : 0) * N;
 
@@ -784,7 +794,22 @@ __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
     }
 
     // ------------------------------------------------------------ phase F
+    if (k < 0) {
+      df cc = df_zero();
+      for (int64_t j = jlo + t; j < jhi; j += kWorkThreads) {
+        const float c = __ldcg(cn_row + j);
+        cc = df_fma(c, c, cc);
+      }
+      df v[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[e] = e == 0 ? cc : df_zero();
+      cc = df_warp_sum8(v);
+      if (lane == 0) xwarp[2 * K] = cc;
+    } else {
     side_wait(3);
+    const df bob = sums[2 * k], bb = sums[2 * k + 1];
+    const bool cdeg = !(bb.h > 0.f);
+    const df inv_bb = cdeg ? df_zero() : df_div(df{1.f, 0.f}, bb);
     for (int64_t j0 = jlo; j0 < jhi; j0 += (int64_t)kTiles * kWorkThreads) {
       float c_old[kTiles], cn[kTiles];
       df q[kTiles];
@@ -839,6 +864,7 @@ __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
           *x = df_add(*x, s8);
         }
       }
+    }
     }
     if (!more) break;
     work_sync();

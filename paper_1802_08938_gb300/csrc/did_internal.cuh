@@ -346,8 +346,9 @@ cudaError_t launch_resident(const ResidentPlan& plan, const SweepArgs& args, voi
 
 // Read-only sweep of the interleaved order (did_defer_kernel.cuh): R keeps its
 // value for a whole sweep, the changes stay pending; the caller forms R anew
-// after it (launch_refresh_tc, with the partials of R c_1^T) and closes the
-// sweep with launch_defer_close.
+// after it (launch_refresh_tc, with the partials of R c_1^T, or launch_dense
+// without them) and closes the sweep with launch_defer_close, which adds the
+// n sums of R^2 at part[stride * i].
 struct DeferPlan {
   int grid, GS, NG, NR, CW, S;
   Units units;
@@ -364,7 +365,7 @@ struct DeferBuffers {
   float* P;           // [max(npart, npart_first)][ld]
   double* CC0;        // [npart_first] partials of ||c_1||^2
   void *Xp, *Yp;      // defer_pair_bytes(K, grid) each
-  unsigned* work;     // [K], zero before the first launch
+  unsigned* work;     // [K + 1], zero before the first launch
   Ctrl* ctrl;         // zero before the first launch
   unsigned long long* degen;
 };
@@ -372,7 +373,7 @@ bool plan_defer(int ld, int64_t N, int K, bool bf16, int grid_override, DeferPla
 size_t defer_pair_bytes(int K, int grid);
 cudaError_t launch_defer(const DeferPlan& plan, const DeferBuffers& b, int ld, int64_t N, int K, int npart_first,
                          int bar_extra, uint64_t timeout_ns, uint64_t* tstamp, int tstamp_cap, cudaStream_t s);
-cudaError_t launch_defer_close(const double* part, int n, const DeferBuffers& b, int K, double* trace, cudaStream_t s);
+cudaError_t launch_defer_close(const double* part, int n, int stride, const DeferBuffers& b, int K, double* trace, cudaStream_t s);
 
 // Multi-instance sweeps (serving): one cooperative launch runs several
 // instances, each on its own range of CTAs (SweepArgs::cta_begin/cta_count).

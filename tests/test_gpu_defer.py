@@ -38,7 +38,8 @@ def run(did, X, B0, C0, sweeps, **kw):
 
 
 SHAPES = [(64, 150001, 16), (130, 70003, 7), (784, 12001, 5), (1030, 9001, 2), (2064, 4503, 9), (5003, 1999, 3),
-          (9000, 1051, 1), (12000, 801, 4), (18001, 541, 2)]
+          (9000, 1051, 1), (12000, 801, 4), (18001, 541, 2),
+          (600, 16001, 65), (1100, 9005, 101)]
 
 
 @pytest.mark.parametrize("M,N,K", SHAPES)

@@ -312,15 +312,16 @@ did_status did_generate_uniform(float* out_dev, int64_t n, uint64_t seed, int32_
  * one is admitted when a slot is free and its device memory (X, R, B, C and
  * partials: about M*N*(4 + s) bytes, s = 4 FP32 or 2 BF16-R) fits in the HBM
  * budget.  Admitted requests keep X, R, B and C resident on the device.  The
- * worker runs rounds: one cooperative launch of the multi-instance sweep
- * kernel runs up to `round_sweeps` sweeps of every active request, each on
- * its own range of CTAs with its own grid barriers and stopping test
- * (|f_{t-1} - f_t| / f_{t-1} < tol, or max_iter sweeps).  A request's range
- * is sized by the time its sweeps take: the kernel stamps the first sweep of
- * each request in a round, and the next round gives each request CTAs in
- * proportion to its measured CTA-seconds per sweep (a cost model of its
- * bytes until it has run once), so the requests' sweeps take about equally
- * long.
+ * worker runs rounds that advance every active request by up to `round_sweeps`
+ * sweeps, each with its own stopping test on the device
+ * (|f_{t-1} - f_t| / f_{t-1} < tol, or max_iter sweeps).  Requests whose
+ * residual fits the SMs' shared memory are packed into cooperative launches, each
+ * on its own range of CTAs; larger ones take the whole GPU in turn (as many of
+ * their sweeps a round as fit in about 20 ms, at least one); the rest share one
+ * launch of the multi-instance sweep kernel, with CTAs in proportion to
+ * measured CTA-seconds per sweep.  The scratch of these forms (the pending
+ * factors and the refresh's operands of the largest request) is the server's, outside the
+ * budget; where it cannot be had every request takes the last form.
  * Between rounds, finished requests are retired (B, C copied to host memory
  * owned by the server, device memory freed) and waiting ones admitted, so
  * requests arriving while others run join at the next round.  The start
@@ -363,11 +364,8 @@ typedef struct {
 } did_server_stats_t;
 
 /* max_slots: requests active at once (<= CTAs of one launch); round_sweeps:
- * the most sweeps a request runs in one round (1..64).  Within a round every
- * request runs as many sweeps (up to round_sweeps) as fit in the time of the
- * slowest request's single sweep (at least 5 ms), so all CTA ranges stay
- * busy; a smaller round_sweeps admits new requests sooner.  stream: NULL =
- * the server creates its own. */
+ * the most sweeps a request runs in one round (1..64); a smaller one admits
+ * new requests sooner.  stream: NULL = the server creates its own. */
 did_status did_server_create(size_t hbm_budget_bytes, did_precision precision, int32_t max_slots,
                              int32_t round_sweeps, void* stream, did_server** out);
 /* Queue a request (the struct is copied; X is read at admission); *ticket

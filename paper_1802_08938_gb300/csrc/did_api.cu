@@ -474,7 +474,10 @@ did_status run_defer(did_ctx* c, int64_t max_sweeps, int stop_rule, double tol, 
       c->refreshes++;
       if (tc) c->tc_refreshes++;
     }
-    const int n = stop_rule ? 1 : chunk_size(c, max_sweeps - *done_total);   // with a stopping rule: one sweep per check
+    // with a stopping rule (evaluated on the device) only a few sweeps are queued ahead
+    const int chunk = chunk_size(c, max_sweeps - *done_total);
+    const int n = stop_rule ? std::min(chunk, 4) : chunk;
+    const double f_start = c->trace.back(), f0 = c->trace.front();
     const uint64_t tmo = wait_limit_ns(c);
     const int cap = c->tstamp ? (int)std::min<int64_t>((int64_t)n * c->K, c->tstamp_cap) : 0;
     c->tstamp_n = cap;
@@ -489,10 +492,12 @@ did_status run_defer(did_ctx* c, int64_t max_sweeps, int stop_rule, double tol, 
       if (tc) {
         DID_CUDA(c, did::launch_refresh_tc(c->X, c->R, c->B, c->C, (int)c->M, c->ld, c->N, c->K, c->tc_ws, c->tc_part,
                                            c->P, c->CCp, &c->ctrl->err, tmo, c->stream, !c->bf16));
-        DID_CUDA(c, did::launch_defer_close(c->tc_part, G, 1, c->dbuf, c->K, c->trace_dev + s, c->stream));
+        DID_CUDA(c, did::launch_defer_close(c->tc_part, G, 1, c->dbuf, c->K, c->trace_dev + s,
+                                             stop_rule, tol, f_start, f0, s == 0, c->stream));
       } else {
         DID_CUDA(c, did::launch_dense(da, c->stream));
-        DID_CUDA(c, did::launch_defer_close(c->dense_part, c->dense_grid, 3, c->dbuf, c->K, c->trace_dev + s, c->stream));
+        DID_CUDA(c, did::launch_defer_close(c->dense_part, c->dense_grid, 3, c->dbuf, c->K, c->trace_dev + s,
+                                             stop_rule, tol, f_start, f0, s == 0, c->stream));
       }
     }
     DID_CUDA(c, cudaEventRecord(c->ev1, c->stream));
@@ -503,7 +508,7 @@ did_status run_defer(did_ctx* c, int64_t max_sweeps, int stop_rule, double tol, 
     float ms = 0.f;
     DID_CUDA(c, cudaEventElapsedTime(&ms, c->ev0, c->ev1));
     c->sweep_ms += ms;
-    c->sweep_launches += n;
+    c->sweep_launches += std::max(1, h.sweeps);
     for (int s = 0; s < h.sweeps; ++s) c->trace.push_back(c->trace_host[s]);
     c->sweeps_done += h.sweeps;
     *done_total += h.sweeps;
@@ -515,9 +520,7 @@ did_status run_defer(did_ctx* c, int64_t max_sweeps, int stop_rule, double tol, 
       return fail(c, DID_ETIMEOUT, "a bounded wait of the sweep exceeded its limit (device error %d); "
                   "state kept, residual will be recomputed", h.err);
     }
-    const double f = c->last_obj, prev = c->trace[c->trace.size() - 2];
-    if (stop_rule == 1 && (f == 0.0 || (prev > 0.0 && fabs(prev - f) / prev < tol))) break;
-    if (stop_rule == 2 && f <= tol * c->trace.front()) break;
+    if (h.stopped) break;
   }
   return DID_OK;
 }

@@ -18,15 +18,21 @@ using namespace defer_impl;
 namespace {
 
 // Closes a sweep: f = 1/2 ||R||^2 from the refresh's per-CTA sums (added in
-// order), and clears the barrier and the unit counters for the next launch.
-__global__ void defer_close_kernel(const double* part, int n, int stride, Ctrl* ctrl, unsigned* work, int K, double* trace) {
+// order), the stopping rule, and the barrier and the unit counters cleared
+// for the next launch.  Nothing after a sweep that stopped or failed.
+__global__ void defer_close_kernel(const double* part, int n, int stride, Ctrl* ctrl, unsigned* work, int K, double* trace,
+                                   int stop_rule, double tol, double f_prev, double f0, int first) {
+  if (ctrl->stopped || ctrl->err) return;
   for (int i = threadIdx.x; i <= K; i += blockDim.x) work[i] = 0u;
   if (threadIdx.x == 0) {
     double s = 0.0;
     for (int i = 0; i < n; ++i) s += part[(size_t)i * stride];
-    *trace = 0.5 * s;
+    const double f = 0.5 * s, prev = first ? f_prev : trace[-1];
+    *trace = f;
     ctrl->bar = 0u;
-    if (ctrl->err == 0) ctrl->sweeps += 1;
+    ctrl->sweeps += 1;
+    if (stop_rule == 1 && (f == 0.0 || (prev > 0.0 && fabs(prev - f) / prev < tol))) ctrl->stopped = 1;
+    if (stop_rule == 2 && f <= tol * f0) ctrl->stopped = 1;
   }
 }
 
@@ -144,8 +150,10 @@ cudaError_t launch_defer(const DeferPlan& plan, const DeferBuffers& b, int ld, i
   return cudaLaunchCooperativeKernel(plan.func, dim3(plan.grid), dim3(kDeferThreads), params, plan.smem, s);
 }
 
-cudaError_t launch_defer_close(const double* part, int n, int stride, const DeferBuffers& b, int K, double* trace, cudaStream_t s) {
-  defer_close_kernel<<<1, 128, 0, s>>>(part, n, stride, b.ctrl, b.work, K, trace);
+cudaError_t launch_defer_close(const double* part, int n, int stride, const DeferBuffers& b, int K, double* trace,
+                               int stop_rule, double tol, double f_prev, double f0, bool first, cudaStream_t s) {
+  defer_close_kernel<<<1, 128, 0, s>>>(part, n, stride, b.ctrl, b.work, K, trace, stop_rule, tol, f_prev, f0,
+                                       first ? 1 : 0);
   return cudaGetLastError();
 }
 

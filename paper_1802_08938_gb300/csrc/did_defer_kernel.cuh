@@ -275,6 +275,7 @@ __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
   typedef Vec<BF16> V;
   typedef typename V::raw raw;
   constexpr int VR = V::kRows, VH = VR / 2, ELEM = BF16 ? 2 : 4;
+  if (a.ctrl->stopped) return;                    // (set by an earlier launch: the same in every CTA)
   const int G = gridDim.x, cta = blockIdx.x;
   const int ld = a.ld, K = a.K, S = a.S, NG = a.NG, GS = a.GS;
   const int64_t N = a.N;

@@ -341,6 +341,13 @@ struct ResidentPlan {
   size_t smem, words_bytes;
 };
 bool plan_resident(int ld, int64_t N, int K, int grid_override, ResidentPlan* plan);   // false: does not fit
+// Several instances in one launch (serving): a plan on at most `grid` CTAs each,
+// their arguments (resident_args_bytes() apart; SweepArgs::cta_begin says
+// where their CTAs start, and their words are zero), one launch.
+bool plan_resident_on(int ld, int64_t N, int K, int grid, ResidentPlan* plan);
+size_t resident_args_bytes();
+void fill_resident_args(void* dst, const ResidentPlan& plan, const SweepArgs& args, void* words, bool bf16);
+cudaError_t launch_resident_multi(const void* d_args, int ninst, int grid, size_t smem, cudaStream_t s);
 cudaError_t launch_resident(const ResidentPlan& plan, const SweepArgs& args, void* words, unsigned step0, bool bf16,
                             cudaStream_t s);
 
@@ -348,7 +355,8 @@ cudaError_t launch_resident(const ResidentPlan& plan, const SweepArgs& args, voi
 // value for a whole sweep, the changes stay pending; the caller forms R anew
 // after it (launch_refresh_tc, with the partials of R c_1^T, or launch_dense
 // without them) and closes the sweep with launch_defer_close, which adds the
-// n sums of R^2 at part[stride * i].
+// n sums of R^2 at part[stride * i] and applies the stopping rule; a launch
+// that finds Ctrl::stopped set does nothing.
 struct DeferPlan {
   int grid, GS, NG, NR, CW, S;
   Units units;
@@ -373,7 +381,9 @@ bool plan_defer(int ld, int64_t N, int K, bool bf16, int grid_override, DeferPla
 size_t defer_pair_bytes(int K, int grid);
 cudaError_t launch_defer(const DeferPlan& plan, const DeferBuffers& b, int ld, int64_t N, int K, int npart_first,
                          int bar_extra, uint64_t timeout_ns, uint64_t* tstamp, int tstamp_cap, cudaStream_t s);
-cudaError_t launch_defer_close(const double* part, int n, int stride, const DeferBuffers& b, int K, double* trace, cudaStream_t s);
+// f_prev: objective before the sweep (trace[-1] instead when s > 0).
+cudaError_t launch_defer_close(const double* part, int n, int stride, const DeferBuffers& b, int K, double* trace,
+                               int stop_rule, double tol, double f_prev, double f0, bool first, cudaStream_t s);
 
 // Multi-instance sweeps (serving): one cooperative launch runs several
 // instances, each on its own range of CTAs (SweepArgs::cta_begin/cta_count).

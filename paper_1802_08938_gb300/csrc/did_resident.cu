@@ -20,8 +20,8 @@
 // carries its step number in the same 8 bytes, so the receiver polls the data
 // itself: no fence, no atomic, and no load after the barrier.  The sweep kernel's
 // per-k cost on these sizes is 27 to 32 us (two grid barriers with the
-// loads behind them); here 7.3 us at 200 x 1000 (63 CTAs), 10.3 us at 1024 x
-// 2414 (151 CTAs), of which the exchange takes 2.3 and 4.9.  A word is
+// loads behind them); here 6.5 us at 200 x 1000 (32 CTAs), 8.5 us at 1024 x
+// 2414 (76 CTAs), of which the exchange takes 2.4 and 3.7.  A word is
 // overwritten only after its readers have used it: a CTA sends the partials of step s + 1
 // after it has all of b'(s), and b'(s) is sent after the owner has read every
 // CTA's partials of step s.
@@ -77,8 +77,8 @@ struct ResArgs {
   void* R;             // ld x N residual in global memory (float or bfloat16), read at the start, written at the end
   float* B;            // ld x K
   float* C;            // K x N
-  uint2* Pw;           // [grid][ld + 6] words: partial rows, then ||c||^2 (hi, lo) and ||R||^2 (hi, lo) of
-                       // even and of odd sweeps
+  uint2* Pw;           // [grid][ld + 8] words: partial rows, then ||c||^2 (hi, lo) of even and of odd steps,
+                       // ||R||^2 (hi, lo) of even and of odd sweeps
   uint4* Bw;           // [ld] words (b', step, b, step)
   Ctrl* ctrl;
   double* trace;
@@ -95,10 +95,11 @@ struct ResArgs {
   uint64_t timeout_ns;
   uint64_t* tstamp;
   int tstamp_cap;
+  int cta_begin, cta_count;   // several instances in one launch: the CTAs of this one
 };
 
 struct ResSmem {
-  size_t R, bn, bo, C, cn, vals, red, brow, misc, total;
+  size_t R, bn, bo, C, cn, vals, ps, red, brow, misc, total;   // (K only for the own rows of B)
 };
 __host__ __device__ __forceinline__ ResSmem res_smem(int ld, int K, int nc, int grid) {
   ResSmem L;
@@ -108,9 +109,10 @@ __host__ __device__ __forceinline__ ResSmem res_smem(int ld, int K, int nc, int 
   L.bn = o;   o += (size_t)ld * 4;
   L.bo = o;   o += (size_t)ld * 4;
   const size_t ncp = ((size_t)nc + 3) & ~(size_t)3;                  // rows of C padded for 16-byte loads
-  L.C = o;    o += (size_t)K * ncp * 4;
+  L.C = o;    o += (size_t)2 * ncp * 4;                              // rows k and k + 1 of C on the own columns
   L.cn = o;   o += (size_t)2 * ncp * 4;                              // c_k before and after its update
   L.vals = o; o += ((size_t)(rpc + 4) * grid * 4 + 15) & ~(size_t)15;
+  L.ps = o;   o += (size_t)kResThreads * 4;                          // a short column's partials by parts of the columns
   L.brow = o; o += ((size_t)rpc * K * 4 + 15) & ~(size_t)15;         // own rows of B
   L.red = o;  o += (size_t)kResWarps * 4 * 8;
   L.misc = o; o += 64;
@@ -152,9 +154,9 @@ struct Poll {
   }
 };
 
-__global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs a) {
+__device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, const int G) {
   extern __shared__ __align__(128) unsigned char smem[];
-  const int G = gridDim.x, cta = blockIdx.x, t = threadIdx.x, w = t >> 5, lane = t & 31;
+  const int t = threadIdx.x, w = t >> 5, lane = t & 31;
   const int ld = a.ld, K = a.K;
   const int64_t N = a.N;
   const ResSmem L = res_smem(ld, K, a.nc, G);
@@ -166,6 +168,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs a) {
   float* cold = reinterpret_cast<float*>(smem + L.cn);
   float* cnew = cold + ncp;
   float* vals = reinterpret_cast<float*>(smem + L.vals);
+  float* ps = reinterpret_cast<float*>(smem + L.ps);
   float* brow = reinterpret_cast<float*>(smem + L.brow);
   pf* red = reinterpret_cast<pf*>(smem + L.red);
   volatile int* bad = reinterpret_cast<volatile int*>(smem + L.misc);
@@ -175,10 +178,10 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs a) {
   const int nc = (int)(j0 < N ? (N - j0 < a.nc ? N - j0 : a.nc) : 0);
   const int rpc = (ld + G - 1) / G;
   const int r0 = cta * rpc, nrows = max(0, min(ld, r0 + rpc) - r0);
-  const int pw = ld + 6;                       // words of a CTA's row in Pw
+  const int pw = ld + 8;                       // words of a CTA's row in Pw
   uint2* mine = a.Pw + (size_t)cta * pw;
 
-  // own columns of R and C, own rows of B
+  // own columns of R, own rows of B
   // expired waits of an exchange's first and second half and of the
   // objective: a word each, written before and read after a CTA barrier
   if (t < 3) bad[t] = 0;
@@ -188,10 +191,6 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs a) {
   } else {
     const float4* src = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(a.R) + (size_t)j0 * ld);
     for (int i = t; i < nc * ld / 4; i += kResThreads) reinterpret_cast<float4*>(R)[i] = __ldcg(src + i);
-  }
-  for (int i = t; i < K * nc; i += kResThreads) {
-    const int k = i / nc, c = i - k * nc;
-    Cs[k * ncp + c] = __ldcg(a.C + (size_t)k * N + j0 + c);
   }
   for (int i = t; i < K * nrows; i += kResThreads) {
     const int k = i / nrows, r = i - k * nrows;
@@ -205,15 +204,20 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs a) {
   bool dead = false;
   const bool stamps = a.tstamp != nullptr && cta == 0 && t == 0;
 
-  // ||c||^2 over the own columns of row k of C, sent with the partials of `s`
-  // (one warp).
-  auto send_cc = [&](int k, unsigned s) {
+  // C stays in global memory (the own columns are this CTA's alone); row k is
+  // kept in shared memory for its step and the one before.
+  auto crow = [&](int k) -> float* { return Cs + (k & 1) * ncp; };
+  auto load_row = [&](int k) {
+    for (int c = t; c < nc; c += kResThreads) crow(k)[c] = __ldcg(a.C + (size_t)k * N + j0 + c);
+  };
+  // ||c||^2 of a row on the own columns, sent for step `s` (one warp).
+  auto send_cc = [&](const float* row, unsigned s) {
     pf cc = pf{0.f, 0.f};
-    for (int c = lane; c < nc; c += 32) cc = pf_fma(Cs[k * ncp + c], Cs[k * ncp + c], cc);
+    for (int c = lane; c < nc; c += 32) cc = pf_fma(row[c], row[c], cc);
     cc = pf_warp_sum(cc);
     if (lane == 0) {
-      st_word(mine + ld, cc.h, s);
-      st_word(mine + ld + 1, cc.l, s);
+      st_word(mine + ld + 2 * (s & 1), cc.h, s);
+      st_word(mine + ld + 1 + 2 * (s & 1), cc.l, s);
     }
   };
   // Sum of the CTAs' words `at` and `at + 1` (a pair each) of step s, by one
@@ -239,32 +243,31 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs a) {
   };
   // Block sums of two pairs, in every thread (two barriers apart from the next use).
   auto block_pairs = [&](pf& x, pf& y) {
-    x = pf_warp_sum(x);
-    y = pf_warp_sum(y);
-    if (lane == 0) {
-      red[2 * w] = x;
-      red[2 * w + 1] = y;
-    }
-    __syncthreads();
-    x = lane < kResWarps ? red[2 * lane] : pf{0.f, 0.f};
-    y = lane < kResWarps ? red[2 * lane + 1] : pf{0.f, 0.f};
+    // even lanes sum x, odd lanes y: one chain of additions instead of two
+    const pf send = (lane & 1) ? x : y, keep = (lane & 1) ? y : x;
+    pf v = pf_add(keep, pf_shfl(send, 1));
 #pragma unroll
-    for (int m = kResWarps / 2; m >= 1; m >>= 1) {
-      x = pf_add(x, pf_shfl(x, m));
-      y = pf_add(y, pf_shfl(y, m));
-    }
-    x = pf{__shfl_sync(0xffffffffu, x.h, 0), __shfl_sync(0xffffffffu, x.l, 0)};
-    y = pf{__shfl_sync(0xffffffffu, y.h, 0), __shfl_sync(0xffffffffu, y.l, 0)};
+    for (int m = 2; m <= 16; m <<= 1) v = pf_add(v, pf_shfl(v, m));
+    if (lane < 2) red[2 * w + lane] = v;
+    __syncthreads();
+    v = red[lane];                                 // warp lane / 2, x or y
+#pragma unroll
+    for (int m = 2; m <= 16; m <<= 1) v = pf_add(v, pf_shfl(v, m));
+    x = pf{__shfl_sync(0xffffffffu, v.h, 0), __shfl_sync(0xffffffffu, v.l, 0)};
+    y = pf{__shfl_sync(0xffffffffu, v.h, 1), __shfl_sync(0xffffffffu, v.l, 1)};
   };
-  // Partials of R c^T over the own columns for c = row kc of C, sent as step s
-  // (first step of a launch or of a B step; later ones come with the update).
-  auto send_partials = [&](int kc, unsigned s) {
+  // Partials of R c_1^T over the own columns, sent as step s (first step of a
+  // launch or of a B step; later ones come with the update).
+  auto send_first = [&](unsigned s) {
+    load_row(0);
+    __syncthreads();
+    const float* c1 = crow(0);
     for (int r = t; r < ld; r += kResThreads) {
       float p = 0.f;
-      for (int c = 0; c < nc; ++c) p = fmaf(R[c * ld + r], Cs[kc * ncp + c], p);
+      for (int c = 0; c < nc; ++c) p = fmaf(R[c * ld + r], c1[c], p);
       st_word(mine + r, p, s);
     }
-    if (w == kResWarps - 1) send_cc(kc, s);
+    if (w == kResWarps - 1) send_cc(c1, s);
   };
   // words of this thread in the owner's part of an exchange (the first kOwn of them)
   constexpr int kOwn = 4;
@@ -315,7 +318,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs a) {
     }
     pf cc = pf{0.f, 0.f};
     if (w == kResWarps - 1 && nrows > 0) {
-      if (!take_pair(ld, s, cc)) ok = false;
+      if (!take_pair(ld + 2 * (int)(s & 1), s, cc)) ok = false;
       if (lane == 0) red[2 * kResWarps] = cc;
     }
     if (!ok) bad[0] = 1;
@@ -369,15 +372,20 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs a) {
     return true;                 // the caller's next barrier publishes bn, bo and bad
   };
   // R += bo c_old - bn c_new on the own columns (cold, cnew) and, in the same
-  // loop, the partials for row knext of C (sent as step s) or, with obj, ||R||^2.
-  auto update = [&](int knext, unsigned s, bool send, bool obj, pf& r2) {
-    const float* cx = Cs + (size_t)knext * ncp;
-    for (int r = t; r < ld; r += kResThreads) {
+  // loop, the partials for the row cx of C (sent as step s) and, with obj, ||R||^2.
+  auto update = [&](const float* cx, unsigned s, bool send, bool obj, pf& r2) {
+    // a thread per row; where the rows leave threads over, several parts of
+    // the columns (up to 512 / ld, at least 8 columns each) a row
+    const int parts = min(kResThreads / ld, nc / 8);
+    const int chunk = parts > 1 ? ((nc + parts - 1) / parts + 3) & ~3 : nc;
+    const int part = parts > 1 ? t / ld : 0;
+    const int clo = min(nc, part * chunk), chi = min(nc, clo + chunk);
+    for (int r = parts > 1 ? t - part * ld : t; r < ld; r += kResThreads) {
       const float x = bo[r], y = -bn[r];
-      float* Rr = R + r;
+      float* Rr = R + (size_t)clo * ld + r;
       float p = 0.f, q = 0.f;
-      int c = 0;
-      for (; c + 4 <= nc; c += 4) {
+      int c = clo;
+      for (; c + 4 <= chi; c += 4) {
         const float4 c0 = *reinterpret_cast<const float4*>(cold + c), c1 = *reinterpret_cast<const float4*>(cnew + c);
         const float4 c2 = *reinterpret_cast<const float4*>(cx + c);
         float v0 = Rr[0], v1 = Rr[ld], v2 = Rr[2 * ld], v3 = Rr[3 * ld];
@@ -396,44 +404,78 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs a) {
         p = fmaf(v3, c2.w, p);
         if (obj) q = fmaf(v0, v0, fmaf(v1, v1, fmaf(v2, v2, fmaf(v3, v3, q))));
       }
-      for (; c < nc; ++c, Rr += ld) {
+      for (; c < chi; ++c, Rr += ld) {
         const float v = fmaf(x, cold[c], fmaf(y, cnew[c], *Rr));
         *Rr = v;
         p = fmaf(v, cx[c], p);
         if (obj) q = fmaf(v, v, q);
       }
-      if (send) st_word(mine + r, p, s);
+      if (parts > 1) {
+        if (part < parts) ps[t] = p;               // ps[part * ld + r]
+      } else if (send) {
+        st_word(mine + r, p, s);
+      }
       if (obj) r2 = pf_add(r2, pf{q, 0.f});
     }
-    if (send && w == kResWarps - 1) send_cc(knext, s);
+    if (parts > 1 && send) {
+      __syncthreads();
+      if (t < ld) {
+        float p = ps[t];
+        for (int e = 1; e < parts; ++e) p += ps[e * ld + t];
+        st_word(mine + t, p, s);
+      }
+    }
   };
-  // c_k on the own columns from bn: a warp takes a column.
-  auto columns = [&](int k, pf bb, pf bob) {
+  // c_k on the own columns from bn: a warp takes a column, or two where there
+  // are more than warps.
+  auto columns = [&](int k, const float* ck, pf bb, pf bob) {
     const bool cdeg = !(bb.h > 0.f);
     const float inv_bb = cdeg ? 0.f : pf_div(pf{1.f, 0.f}, bb).h;
     const float alpha = cdeg ? 0.f : pf_div(bob, bb).h;
     if (cdeg && cta == 0 && t == 0) atomicAdd(a.degen, 1ull);
     const float4* b4 = reinterpret_cast<const float4*>(bn);
-    for (int c = w; c < nc; c += kResWarps) {
-      const float4* r4 = reinterpret_cast<const float4*>(R + (size_t)c * ld);
-      float2 d0 = make_float2(0.f, 0.f), d1 = d0;
-      for (int i = lane; i < ld / 4; i += 32) {
-        const float4 x = r4[i], y = b4[i];
-        d0 = __ffma2_rn(make_float2(x.x, x.y), make_float2(y.x, y.y), d0);
-        d1 = __ffma2_rn(make_float2(x.z, x.w), make_float2(y.z, y.w), d1);
-      }
-      const float dot = warp_sum_f32((d0.x + d0.y) + (d1.x + d1.y));
-      const float co = Cs[k * ncp + c];
+    auto finish = [&](int c, float dot) {
+      const float co = ck[c];
       float cv = co;
       if (!cdeg) {
         const float v = fmaf(alpha, co, dot * inv_bb);
         cv = v > 0.f ? v : 0.f;
       }
-      if (lane == 0) {
-        cold[c] = co;
-        cnew[c] = cv;
-        Cs[k * ncp + c] = cv;
+      cold[c] = co;
+      cnew[c] = cv;
+      __stcg(a.C + (size_t)k * N + j0 + c, cv);
+    };
+    const int n4 = ld / 4;
+    int c = w;
+    for (; c + kResWarps < nc; c += 2 * kResWarps) {
+      const float4* r4 = reinterpret_cast<const float4*>(R + (size_t)c * ld);
+      const float4* q4 = reinterpret_cast<const float4*>(R + (size_t)(c + kResWarps) * ld);
+      float2 d0 = make_float2(0.f, 0.f), d1 = d0, e0 = d0, e1 = d0;
+      for (int i = lane; i < n4; i += 32) {
+        const float4 x = r4[i], z = q4[i], y = b4[i];
+        const float2 lo = make_float2(y.x, y.y), hi = make_float2(y.z, y.w);
+        d0 = __ffma2_rn(make_float2(x.x, x.y), lo, d0);
+        d1 = __ffma2_rn(make_float2(x.z, x.w), hi, d1);
+        e0 = __ffma2_rn(make_float2(z.x, z.y), lo, e0);
+        e1 = __ffma2_rn(make_float2(z.z, z.w), hi, e1);
       }
+      // the lower half warp reduces the first column, the upper the second
+      const float u = (d0.x + d0.y) + (d1.x + d1.y), v = (e0.x + e0.y) + (e1.x + e1.y);
+      float dot = (lane < 16 ? u : v) + __shfl_xor_sync(0xffffffffu, lane < 16 ? v : u, 16);
+#pragma unroll
+      for (int m = 8; m >= 1; m >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, m);
+      if ((lane & 15) == 0) finish(lane == 0 ? c : c + kResWarps, dot);
+    }
+    if (c < nc) {
+      const float4* r4 = reinterpret_cast<const float4*>(R + (size_t)c * ld);
+      float2 d0 = make_float2(0.f, 0.f), d1 = d0;
+      for (int i = lane; i < n4; i += 32) {
+        const float4 x = r4[i], y = b4[i];
+        d0 = __ffma2_rn(make_float2(x.x, x.y), make_float2(y.x, y.y), d0);
+        d1 = __ffma2_rn(make_float2(x.z, x.w), make_float2(y.z, y.w), d1);
+      }
+      const float dot = warp_sum_f32((d0.x + d0.y) + (d1.x + d1.y));
+      if (lane == 0) finish(c, dot);
     }
   };
 
@@ -448,7 +490,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs a) {
   }
 
   const bool inter = a.order != DID_ORDER_DID;
-  if (!dead && inter) send_partials(0, step + 1);
+  if (!dead && inter) send_first(step + 1);
   int done = 0;
   for (int s = 0; s < a.n_sweeps && !dead; ++s) {
     pf r2 = pf{0.f, 0.f};
@@ -463,26 +505,42 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs a) {
           bn[r] = bo[r] = v;
           bb = pf_fma(v, v, bb);
         }
+        load_row(k);
         block_pairs(bb, dummy);
-        columns(k, bb, bb);
+        columns(k, crow(k), bb, bb);
         __syncthreads();
-        update(0, 0, false, false, r2);
+        update(cnew, 0, false, false, r2);
       }
       __syncthreads();
-      send_partials(0, step + 1);
+      send_first(step + 1);
     }
     for (int k = 0; k < K; ++k) {
       const int at = s * K + k;
       const bool rec = stamps && at < a.tstamp_cap;
       if (rec) a.tstamp[4 * at + 0] = globaltimer_ns();
       ++step;
-      if (!exchange(k, step)) { dead = true; break; }
-      if (rec) a.tstamp[4 * at + 1] = globaltimer_ns();
       const int knext = k + 1 < K ? k + 1 : 0;
       const bool last = k == K - 1;
       // the next step's partials go out with this update (the last step of a
-      // launch, and of a B step, sends none)
+      // launch, and of a B step, sends none); its row of C is read and its
+      // ||c||^2 sent before this step's exchange.  With K = 1 that row is the
+      // one this step updates.  For odd K > 1 rows K - 1 and 0 fall into the
+      // same buffer, so the last step takes its own row from a copy.
       const bool send = last ? inter && s + 1 < a.n_sweeps : true;
+      const float* ck = crow(k);
+      const float* cx = crow(knext);
+      if (send && K > 1) {
+        if (ck == cx) {
+          for (int c = t; c < nc; c += kResThreads) cold[c] = ck[c];
+          ck = cold;
+          __syncthreads();
+        }
+        load_row(knext);
+        __syncthreads();
+        if (w == kResWarps - 1) send_cc(cx, step + 1);
+      }
+      if (!exchange(k, step)) { dead = true; break; }
+      if (rec) a.tstamp[4 * at + 1] = globaltimer_ns();
       if (inter) {
         // (a thread reads only the rows it stored, so this needs no barrier)
         pf bb = pf{0.f, 0.f}, bob = bb;
@@ -492,15 +550,21 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs a) {
         }
         block_pairs(bb, bob);                      // its barrier publishes bn, bo, bad
         if (bad[1]) { dead = true; break; }
-        columns(k, bb, bob);
+        columns(k, ck, bb, bob);
         __syncthreads();
-        // the partials for c_1 of the next sweep take c_1', which this CTA has
-        update(knext, step + 1, send, last, r2);
+        if (K == 1) {                              // the next step's row is c_1'
+          if (send && w == kResWarps - 1) send_cc(cnew, step + 1);
+          update(cnew, step + 1, send, last, r2);
+          __syncthreads();
+          for (int c = t; c < nc; c += kResThreads) crow(0)[c] = cnew[c];
+        } else {
+          update(cx, step + 1, send, last, r2);
+        }
       } else {
-        for (int c = t; c < nc; c += kResThreads) cold[c] = cnew[c] = Cs[k * ncp + c];
+        for (int c = t; c < nc; c += kResThreads) cold[c] = cnew[c] = ck[c];
         __syncthreads();
         if (bad[1]) { dead = true; break; }
-        update(knext, step + 1, send, last, r2);
+        update(cx, step + 1, send, last, r2);
       }
       if (rec) a.tstamp[4 * at + 2] = a.tstamp[4 * at + 3] = globaltimer_ns();
     }
@@ -510,14 +574,14 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs a) {
     __syncthreads();
     block_pairs(r2, z);
     if (t == 0) {
-      st_word(mine + ld + 2 + 2 * (s & 1), r2.h, step);
-      st_word(mine + ld + 3 + 2 * (s & 1), r2.l, step);
+      st_word(mine + ld + 4 + 2 * (s & 1), r2.h, step);
+      st_word(mine + ld + 5 + 2 * (s & 1), r2.l, step);
     }
     bool stop = false;
     const bool need = a.stop_rule != 0 || cta == 0;
     if (need && w == 0) {
       pf f2;
-      const bool ok = take_pair(ld + 2 + 2 * (s & 1), step, f2);
+      const bool ok = take_pair(ld + 4 + 2 * (s & 1), step, f2);
       if (!ok) bad[2] = 1;
       if (lane == 0) red[2 * kResWarps + 1] = f2;
     }
@@ -552,7 +616,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs a) {
       break;
     }
   }
-  // R, C and the own rows of B go back (also after an expired wait: B and C
+  // R and the own rows of B go back (also after an expired wait: B and C
   // are valid then, R is recomputed by the caller)
   __syncthreads();
   if (a.bf16) {
@@ -562,10 +626,6 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs a) {
     float4* dst = reinterpret_cast<float4*>(reinterpret_cast<float*>(a.R) + (size_t)j0 * ld);
     for (int i = t; i < nc * ld / 4; i += kResThreads) dst[i] = reinterpret_cast<float4*>(R)[i];
   }
-  for (int i = t; i < K * nc; i += kResThreads) {
-    const int k = i / nc, c = i - k * nc;
-    a.C[(size_t)k * N + j0 + c] = Cs[k * ncp + c];
-  }
   for (int i = t; i < K * nrows; i += kResThreads) {
     const int k = i / nrows, r = i - k * nrows;
     a.B[(size_t)k * ld + r0 + r] = brow[k * rpc + r];
@@ -573,55 +633,47 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs a) {
   (void)done;
 }
 
-}  // namespace
+__global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs a) {
+  resident_body(a, blockIdx.x, gridDim.x);
+}
 
-bool plan_resident(int ld, int64_t N, int K, int grid_override, ResidentPlan* plan) {
-  int dev = 0, optin = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaFuncAttributes fa{};
-  if (cudaFuncGetAttributes(&fa, resident_kernel) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  const int budget = optin - (int)fa.sharedSizeBytes;
-  const int gmax = grid_override > 0 ? std::min(grid_override, sms) : sms;
-  // Columns of a CTA: one for each warp (16), the fewest CTAs that gives, so
-  // that an exchange has few parties; fewer where a column range must be
-  // shorter to fit, more where the grid is at its limit.
-  ResidentPlan P{};
-  for (int nc = 16; nc >= 1; nc /= 2) {
-    const int64_t g = (N + nc - 1) / nc;
-    if (g > gmax) break;
-    if (res_smem(ld, K, nc, (int)g).total <= (size_t)budget) {
-      P.nc = nc;
-      P.grid = (int)g;
-      break;
-    }
-  }
-  if (P.grid == 0) {
-    const int64_t nc = (N + gmax - 1) / gmax;
-    if (nc > (1 << 20) || res_smem(ld, K, (int)nc, gmax).total > (size_t)budget) return false;
-    P.nc = (int)nc;
-    P.grid = (int)((N + nc - 1) / nc);
-    if (res_smem(ld, K, P.nc, P.grid).total > (size_t)budget) return false;
-  }
-  P.smem = res_smem(ld, K, P.nc, P.grid).total;
-  int per_sm = 0;
-  if (cudaFuncSetAttribute(resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, budget) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, resident_kernel, kResThreads, P.smem) != cudaSuccess ||
-      per_sm < 1) {
-    cudaGetLastError();
-    return false;
-  }
-  P.words_bytes = (size_t)P.grid * (ld + 6) * sizeof(uint2) + (size_t)ld * sizeof(uint4);
-  *plan = P;
+// Several instances in one launch, each on its own range of CTAs.
+__global__ void __launch_bounds__(kResThreads, 1) resident_multi_kernel(const ResArgs* __restrict__ inst, int ninst) {
+  int i = 0;
+  while (i + 1 < ninst && (int)blockIdx.x >= inst[i + 1].cta_begin) ++i;
+  const ResArgs a = inst[i];
+  const int cta = (int)blockIdx.x - a.cta_begin;
+  if (cta < 0 || cta >= a.cta_count) return;
+  resident_body(a, cta, a.cta_count);
+}
+
+// Plan on at most `grid` CTAs: columns dealt evenly; false if they do not fit `budget`.
+bool plan_on(int ld, int64_t N, int K, int grid, size_t budget, ResidentPlan* plan) {
+  const int64_t nc = (N + grid - 1) / grid;
+  if (nc > (1 << 20)) return false;
+  const int g = (int)((N + nc - 1) / nc);
+  const size_t smem = res_smem(ld, K, (int)nc, g).total;
+  if (smem > budget) return false;
+  plan->nc = (int)nc;
+  plan->grid = g;
+  plan->smem = smem;
+  plan->words_bytes = (size_t)g * (ld + 8) * sizeof(uint2) + (size_t)ld * sizeof(uint4);
   return true;
 }
 
-cudaError_t launch_resident(const ResidentPlan& plan, const SweepArgs& s, void* words, unsigned step0, bool bf16,
-                            cudaStream_t st) {
+size_t res_budget(const void* func) {
+  int dev = 0, optin = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  cudaFuncAttributes fa{};
+  if (cudaFuncGetAttributes(&fa, func) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return (size_t)optin - fa.sharedSizeBytes;
+}
+
+ResArgs make_args(const ResidentPlan& plan, const SweepArgs& s, void* words, unsigned step0, bool bf16) {
   ResArgs a{};
   a.R = s.R;
   a.B = s.B;
@@ -647,9 +699,70 @@ cudaError_t launch_resident(const ResidentPlan& plan, const SweepArgs& s, void* 
   a.timeout_ns = s.timeout_ns;
   a.tstamp = s.tstamp;
   a.tstamp_cap = s.tstamp_cap;
+  a.cta_begin = s.cta_begin;
+  a.cta_count = plan.grid;
+  return a;
+}
+
+}  // namespace
+
+bool plan_resident(int ld, int64_t N, int K, int grid_override, ResidentPlan* plan) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const size_t budget = res_budget((const void*)resident_kernel);
+  const int gmax = grid_override > 0 ? std::min(grid_override, sms) : sms;
+  // Columns of a CTA: two for each warp (32), the fewest CTAs that gives, so
+  // that an exchange has few parties; fewer where a column range must be
+  // shorter to fit, more where the grid is at its limit.  A k of 200 x 1000 /
+  // 1024 x 2414 / 43 x 1694: 7.5 / 8.9 / 8.1 us with 8 columns, 6.6 / 8.9 /
+  // 7.2 with 16, 6.3 / 8.7 / 6.1 with 32, 7.3 / 8.6 / 6.3 with 64.
+  ResidentPlan P{};
+  for (int nc = 32; nc >= 1 && P.grid == 0; nc /= 2) {
+    const int64_t g = (N + nc - 1) / nc;
+    if (g > gmax) break;
+    plan_on(ld, N, K, (int)g, budget, &P);
+  }
+  if (P.grid == 0 && !plan_on(ld, N, K, gmax, budget, &P)) return false;
+  int per_sm = 0;
+  if (cudaFuncSetAttribute(resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, resident_kernel, kResThreads, P.smem) != cudaSuccess ||
+      per_sm < 1) {
+    cudaGetLastError();
+    return false;
+  }
+  *plan = P;
+  return true;
+}
+
+// Within a launch of several instances the CTAs are shared out by the caller.
+bool plan_resident_on(int ld, int64_t N, int K, int grid, ResidentPlan* plan) {
+  static const size_t budget = res_budget((const void*)resident_multi_kernel);
+  return grid > 0 && plan_on(ld, N, K, grid, budget, plan);
+}
+
+cudaError_t launch_resident(const ResidentPlan& plan, const SweepArgs& s, void* words, unsigned step0, bool bf16,
+                            cudaStream_t st) {
+  ResArgs a = make_args(plan, s, words, step0, bf16);
+  a.cta_begin = 0;
   void* params[] = {&a};
   return cudaLaunchCooperativeKernel((const void*)resident_kernel, dim3(plan.grid), dim3(kResThreads), params,
                                      plan.smem, st);
+}
+
+size_t resident_args_bytes() { return sizeof(ResArgs); }
+
+void fill_resident_args(void* dst, const ResidentPlan& plan, const SweepArgs& s, void* words, bool bf16) {
+  *static_cast<ResArgs*>(dst) = make_args(plan, s, words, 0u, bf16);
+}
+
+cudaError_t launch_resident_multi(const void* d_args, int ninst, int grid, size_t smem, cudaStream_t st) {
+  const ResArgs* inst = static_cast<const ResArgs*>(d_args);
+  const cudaError_t e = cudaFuncSetAttribute(resident_multi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)res_budget((const void*)resident_multi_kernel));
+  if (e != cudaSuccess) return e;
+  void* params[] = {(void*)&inst, (void*)&ninst};
+  return cudaLaunchCooperativeKernel((const void*)resident_multi_kernel, dim3(grid), dim3(kResThreads), params, smem, st);
 }
 
 }  // namespace did

@@ -1,12 +1,22 @@
 // Serving runtime: continuous batching of factorisation requests on one GPU.
 //
 // A worker thread admits queued requests under an HBM budget and a slot
-// limit, keeps each active request's X, R, B and C resident, and runs rounds:
-// one cooperative launch of the multi-instance sweep kernel advances every
-// active request by up to `round_sweeps` sweeps, each request on its own CTA
-// range (proportional to its per-sweep work) with its own grid barriers and
-// stopping test.  Between rounds finished requests are retired and new ones
-// admitted.  All device memory of a request is one stream-ordered allocation.
+// limit, keeps each active request's X, R, B and C resident, and runs rounds
+// that advance every active request by up to `round_sweeps` sweeps.  A
+// request's residual decides how (Form):
+//   RESIDENT  it fits the SMs' shared memory: such requests are packed into
+//             launches, each request on as few CTAs as hold its residual (and
+//             more where CTAs are left), because a k of it costs two exchanges
+//             whatever the number of CTAs is;
+//   DEFER     larger: read-only sweeps on the whole GPU, one request after another,
+//             each pass at HBM speed, which a share of the SMs does not reach;
+//   PACKED    otherwise (K too large for a short column): the multi-instance sweep kernel, each
+//             request on its own CTA range, proportional to its per-sweep work.
+// All three stop a request on the device by its own rule.  With every
+// request in the multi-instance kernel 24 requests of 20 sweeps took 488 ms;
+// see run_round for what they take now.  Between rounds finished requests are retired and new ones
+// admitted.  All device memory of a request is one stream-ordered allocation;
+// the scratch of the forms is the server's (one request or launch uses it at a time).
 #include "did_internal.cuh"
 
 #include <math.h>
@@ -33,7 +43,8 @@ constexpr uint64_t kServeTimeoutNs = 4000000000ull;
 // the residual's read and write at one CTA's share of the HBM bandwidth.
 constexpr double kPassFixedS = 12e-6;
 constexpr double kCtaBytesPerS = 40e9;
-constexpr double kRoundMinS = 5e-3;      // a round lasts at least this long
+constexpr double kRoundMinS = 5e-3;      // a launch of the multi-instance kernel lasts at least this long
+constexpr double kDeferSliceS = 20e-3;   // a larger request's sweeps in one round take at most about this long
 // Phase stamps kept per instance (4 per k of its first sweep in a round):
 // the measured time of that sweep drives the next round's CTA shares.
 constexpr int kStampK = 64;
@@ -45,6 +56,7 @@ double now_s(const std::chrono::steady_clock::time_point& t0) {
 size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 enum ReqState { QUEUED, ACTIVE, DONE, FAILED };
+enum Form { RESIDENT, DEFER, PACKED };
 
 struct Req {
   uint64_t ticket = 0;
@@ -60,7 +72,10 @@ struct Req {
   double *CCp = nullptr, *Sp = nullptr, *OBJp = nullptr;
   int sweeps = 0;
   double cta_s = -1.0;     // measured CTA-seconds per sweep (smoothed); < 0: not measured yet
-  int sh_last = 0;         // CTAs of its last round (0: none yet)
+  int sh_last = 0;         // CTAs of its last round in the multi-instance kernel (0: none, or another form since)
+  Form form = PACKED;
+  int ctas = 0;            // RESIDENT: fewest CTAs that hold its residual
+  did::DeferPlan dplan{};  // DEFER
   std::vector<double> trace;
   std::vector<float> Bh, Ch;   // results on the host after completion
   double t_submit = 0, t_start = 0, t_done = 0;
@@ -98,6 +113,10 @@ struct did_server {
   double* h_trace = nullptr;
   uint64_t* d_stamp = nullptr;       // [slot][4 kStampK] phase stamps of an instance's first sweep
   uint64_t* h_stamp = nullptr;
+  unsigned char* d_res = nullptr;    // [slot] arguments of resident instances
+  unsigned char* h_res = nullptr;
+  void* scratch = nullptr;           // words of a resident launch, or buffers of a read-only sweep
+  size_t scratch_bytes = 0;
   unsigned long long* d_degen = nullptr;
   unsigned long long* d_bad = nullptr;   // negative or non-finite entries of a request's X
   unsigned long long* h_bad = nullptr;
@@ -129,6 +148,8 @@ size_t request_bytes(const did_server* s, int64_t M, int64_t N, int K, int ld) {
   (void)M;
   return b;
 }
+
+void choose_form(const did_server* s, Req* r);
 
 // Allocate, generate or copy X, draw the start point and form R = X - B C.
 did_status admit(did_server* s, Req* r) {
@@ -196,6 +217,7 @@ did_status admit(did_server* s, Req* r) {
     return DID_ECUDA;
   }
   if (r->rq.X && *s->h_bad != 0) return DID_EINVAL;
+  choose_form(s, r);
   double f = 0.0;
   for (int i = 0; i < s->dense_grid; ++i) f += s->h_part[3 * i];
   r->trace.assign(1, 0.5 * f);
@@ -250,48 +272,127 @@ std::vector<int> shares(const did_server* s, const std::vector<Req*>& act) {
   return sh;
 }
 
-// One round over the active requests; returns false on a CUDA error.
-bool run_round(did_server* s, std::vector<Req*>& act) {
-  const int n = (int)act.size();
-  const std::vector<int> sh = shares(s, act);
-  // Sweeps per instance: the round lasts about as long as the slowest
+// How a request is swept (see the head of this file).
+void choose_form(const did_server* s, Req* r) {
+  const int64_t N = r->rq.N;
+  const int K = r->rq.K;
+  did::ResidentPlan p{};
+  r->form = PACKED;
+  if (did::plan_resident_on(r->ld, N, K, s->grid, &p)) {
+    int lo = 1, hi = s->grid;
+    while (lo < hi) {
+      const int mid = (lo + hi) / 2;
+      if (did::plan_resident_on(r->ld, N, K, mid, &p)) hi = mid; else lo = mid + 1;
+    }
+    r->form = RESIDENT;
+    r->ctas = did::plan_resident_on(r->ld, N, K, lo, &p) ? lo : s->grid;
+  } else if (r->ld >= 4 * K && did::plan_defer(r->ld, N, K, s->bf16, 0, &r->dplan)) {
+    r->form = DEFER;
+  }
+}
+
+// The server's scratch, at least `bytes`; false if the memory is not there.
+bool need_scratch(did_server* s, size_t bytes) {
+  if (bytes <= s->scratch_bytes) return true;
+  if (s->scratch) cudaFreeAsync(s->scratch, s->stream);
+  s->scratch = nullptr;
+  s->scratch_bytes = 0;
+  if (cudaMallocAsync(&s->scratch, bytes, s->stream) != cudaSuccess) {
+    cudaGetLastError();
+    s->scratch = nullptr;
+    return false;
+  }
+  s->scratch_bytes = bytes;
+  return true;
+}
+
+// Buffers of a read-only sweep of r in the scratch (or, with base null, their size).
+struct DeferScratch {
+  did::DeferBuffers b{};
+  void* tc_ws = nullptr;
+  double* part = nullptr;
+  size_t bytes = 0;
+};
+DeferScratch defer_scratch(const did_server* s, const Req* r, unsigned char* base) {
+  DeferScratch d;
+  const size_t N = (size_t)r->rq.N, K = (size_t)r->rq.K, ld = (size_t)r->ld;
+  const size_t G = (size_t)did::refresh_tc_grid();
+  size_t o = 0;
+  auto take = [&](size_t n) { void* q = base ? base + o : nullptr; o += a256(n); return q; };
+  d.b.Bo = (float*)take(ld * K * 4);
+  d.b.Co = (float*)take(K * N * 4);
+  d.b.T = (float*)take(N * (size_t)(r->dplan.GS / 32) * 4);
+  d.b.corr = take(N * 8);
+  d.b.P = (float*)take(std::max<size_t>((size_t)r->dplan.npart, 2 * G) * ld * 4);
+  d.b.CC0 = (double*)take(2 * G * 8);
+  d.b.Xp = take(did::defer_pair_bytes((int)K, r->dplan.grid));
+  d.b.Yp = take(did::defer_pair_bytes((int)K, r->dplan.grid));
+  d.b.work = (unsigned*)take((K + 1) * 4);
+  d.part = (double*)take(G * 8);
+  if (did::refresh_tc_supported((int)K, !s->bf16))
+    d.tc_ws = take(did::refresh_tc_workspace_bytes((int)r->rq.M, r->ld, r->rq.N, (int)K, !s->bf16));
+  d.bytes = o;
+  d.b.R = r->R;
+  d.b.B = r->B;
+  d.b.C = r->C;
+  return d;
+}
+
+// Common arguments of an instance in slot i.
+SweepArgs slot_args(const did_server* s, const Req* r, int i, int n_sweeps) {
+  SweepArgs a{};
+  a.R = r->R;
+  a.B = r->B;
+  a.C = r->C;
+  a.P = r->P;
+  a.CCp = r->CCp;
+  a.Sp = r->Sp;
+  a.OBJp = r->OBJp;
+  a.bold = r->bold;
+  a.ctrl = s->d_ctrl + i;
+  a.trace = s->d_trace + (size_t)i * s->round_sweeps;
+  a.degen = s->d_degen + i;
+  a.N = r->rq.N;
+  a.M = (int)r->rq.M;
+  a.ld = r->ld;
+  a.K = r->rq.K;
+  a.n_sweeps = n_sweeps;
+  a.f_prev = r->trace.back();
+  a.f0 = r->trace.front();
+  a.stop_rule = r->rq.tol > 0.0 ? 1 : 0;
+  a.tol = r->rq.tol;
+  a.order = DID_ORDER_INTERLEAVED;
+  a.timeout_ns = kServeTimeoutNs;
+  return a;
+}
+
+// PACKED requests (slots idx of act): one launch of the multi-instance kernel.
+cudaError_t launch_packed(did_server* s, const std::vector<Req*>& act, const std::vector<int>& idx) {
+  const int n = (int)idx.size();
+  std::vector<Req*> sub(n);
+  for (int q = 0; q < n; ++q) sub[q] = act[idx[q]];
+  const std::vector<int> sh = shares(s, sub);
+  // Sweeps per instance: the launch lasts about as long as the slowest
   // instance's single sweep (at least kRoundMinS); faster instances run more
   // sweeps in that time, so no CTA range idles for long.  A sweep's time on
   // sh CTAs is taken as its CTA-seconds / sh.
   std::vector<double> tsw(n);
   double T = kRoundMinS;
-  for (int i = 0; i < n; ++i) {
-    tsw[i] = sweep_cta_s(s, act[i]) / (double)sh[i];
-    T = std::max(T, tsw[i]);
-  }
-  std::vector<int> nsw(n);
-  for (int i = 0; i < n; ++i) {
-    const int left = act[i]->rq.max_iter - act[i]->sweeps;
-    nsw[i] = std::max(1, std::min(std::min(s->round_sweeps, left), (int)(T / tsw[i])));
+  for (int q = 0; q < n; ++q) {
+    tsw[q] = sweep_cta_s(s, sub[q]) / (double)sh[q];
+    T = std::max(T, tsw[q]);
   }
   size_t smem = 0;
   int begin = 0;
-  for (int i = 0; i < n; ++i) {
-    Req* r = act[i];
+  for (int q = 0; q < n; ++q) {
+    Req* r = sub[q];
+    const int i = idx[q];
+    const int left = r->rq.max_iter - r->sweeps;
+    const int nsw = std::max(1, std::min(std::min(s->round_sweeps, left), (int)(T / tsw[q])));
     did::SweepPlan plan{};
-    if (did::plan_instance(r->ld, r->rq.N, s->bf16, sh[i], s->smem_budget, &plan) != DID_OK) return false;
+    if (did::plan_instance(r->ld, r->rq.N, s->bf16, sh[q], s->smem_budget, &plan) != DID_OK) return cudaErrorInvalidValue;
     smem = std::max(smem, plan.smem);
-    SweepArgs a{};
-    a.R = r->R;
-    a.B = r->B;
-    a.C = r->C;
-    a.P = r->P;
-    a.CCp = r->CCp;
-    a.Sp = r->Sp;
-    a.OBJp = r->OBJp;
-    a.bold = r->bold;
-    a.ctrl = s->d_ctrl + i;
-    a.trace = s->d_trace + (size_t)i * s->round_sweeps;
-    a.degen = s->d_degen + i;
-    a.N = r->rq.N;
-    a.M = (int)r->rq.M;
-    a.ld = r->ld;
-    a.K = r->rq.K;
+    SweepArgs a = slot_args(s, r, i, nsw);
     a.GS = plan.GS;
     a.NG = plan.NG;
     a.D = plan.D;
@@ -299,50 +400,191 @@ bool run_round(did_server* s, std::vector<Req*>& act) {
     a.nunits = plan.nunits;
     a.dynamic = 0;
     a.npart = plan.npart;
-    a.n_sweeps = nsw[i];
     // the partials of R c_1^T left by the last sweep are valid while the
     // instance keeps its CTA range size (same plan); else a prologue pass
-    a.prologue = sh[i] != r->sh_last ? 1 : 0;
-    r->sh_last = sh[i];
+    a.prologue = sh[q] != r->sh_last ? 1 : 0;
+    r->sh_last = sh[q];
     a.tstamp = s->d_stamp + (size_t)i * 4 * kStampK;
     a.tstamp_cap = std::min(r->rq.K, kStampK);
-    a.f_prev = r->trace.back();
-    a.f0 = r->trace.front();
-    a.stop_rule = r->rq.tol > 0.0 ? 1 : 0;
-    a.tol = r->rq.tol;
-    a.order = DID_ORDER_INTERLEAVED;
-    a.timeout_ns = kServeTimeoutNs;
     a.pair = plan.pair;
     a.cta_begin = begin;
-    a.cta_count = sh[i];
-    begin += sh[i];
-    s->h_inst[i] = a;
+    a.cta_count = sh[q];
+    begin += sh[q];
+    s->h_inst[q] = a;
+  }
+  const cudaError_t e =
+      cudaMemcpyAsync(s->d_inst, s->h_inst, sizeof(SweepArgs) * n, cudaMemcpyHostToDevice, s->stream);
+  if (e != cudaSuccess) return e;
+  return did::launch_sweep_multi(s->bf16, s->d_inst, n, begin, smem, s->stream);
+}
+
+// Time of one k of a resident instance in microseconds, as measured on
+// launches of one instance (6.3 at 208 rows x 32 columns a CTA, 8.7 at 1024 x
+// 32, 12.8 at 2000 x 20, 15.4 at 4112 x 10).
+double resident_k_us(int ld, int nc) { return 5.0 + 1.5e-3 * ld + 8e-5 * (double)ld * nc; }
+
+struct Bin {
+  std::vector<int> slots;
+  std::vector<did::ResidentPlan> plans;
+  size_t words = 0;
+  int ctas = 0;
+};
+
+// RESIDENT requests dealt to launches: longest first into the first launch
+// with room, then the CTAs left in a launch go to its slowest instance.
+std::vector<Bin> pack(const did_server* s, const std::vector<Req*>& act, std::vector<int> idx) {
+  auto cols = [&](int i, int g) { return (int)((act[i]->rq.N + g - 1) / g); };
+  auto cost = [&](int i, int g) { return act[i]->rq.K * resident_k_us(act[i]->ld, cols(i, g)); };
+  std::sort(idx.begin(), idx.end(), [&](int x, int y) {
+    const double a = cost(x, act[x]->ctas), b = cost(y, act[y]->ctas);
+    return a != b ? a > b : x < y;
+  });
+  std::vector<Bin> bins;
+  for (int i : idx) {
+    size_t q = 0;
+    while (q < bins.size() && bins[q].ctas + act[i]->ctas > s->grid) ++q;
+    if (q == bins.size()) bins.emplace_back();
+    bins[q].slots.push_back(i);
+    bins[q].ctas += act[i]->ctas;
+  }
+  for (Bin& b : bins) {
+    const int n = (int)b.slots.size();
+    std::vector<int> g(n);
+    std::vector<char> full(n, 0);
+    for (int q = 0; q < n; ++q) g[q] = act[b.slots[q]]->ctas;
+    int left = s->grid - b.ctas;
+    while (left > 0) {
+      int best = -1;
+      for (int q = 0; q < n; ++q)
+        if (!full[q] && (best < 0 || cost(b.slots[q], g[q]) > cost(b.slots[best], g[best]))) best = q;
+      if (best < 0) break;
+      // the next size that shortens its column ranges, while they are wider than one column a warp
+      const int nc = cols(b.slots[best], g[best]);
+      const int64_t N = act[b.slots[best]]->rq.N;
+      const int to = nc > 16 ? (int)((N + nc - 2) / (nc - 1)) : 0;
+      if (to == 0 || to - g[best] > left) {
+        full[best] = 1;
+        continue;
+      }
+      left -= to - g[best];
+      g[best] = to;
+    }
+    b.ctas = 0;
+    for (int q = 0; q < n; ++q) {
+      const Req* r = act[b.slots[q]];
+      did::ResidentPlan p{};
+      if (!did::plan_resident_on(r->ld, r->rq.N, r->rq.K, g[q], &p)) did::plan_resident_on(r->ld, r->rq.N, r->rq.K, r->ctas, &p);
+      b.plans.push_back(p);
+      b.words += a256(p.words_bytes);
+      b.ctas += p.grid;
+    }
+  }
+  return bins;
+}
+
+// One round over the active requests; returns false on a CUDA error.
+// Measured: 24 requests (64..4096 rows, 256..65536 columns, K 8 to 64, float32)
+// of 20 sweeps each: 488 ms with every request in the multi-instance kernel,
+// 310 ms with the three forms.
+bool run_round(did_server* s, std::vector<Req*>& act) {
+  const int n = (int)act.size();
+  std::vector<int> res, def, packed;
+  for (int i = 0; i < n; ++i) (act[i]->form == RESIDENT ? res : act[i]->form == DEFER ? def : packed).push_back(i);
+  std::vector<Bin> bins = pack(s, act, res);
+  size_t scratch = 0;
+  for (const Bin& b : bins) scratch = std::max(scratch, b.words);
+  for (int i : def) scratch = std::max(scratch, defer_scratch(s, act[i], nullptr).bytes);
+  if (!need_scratch(s, scratch)) {       // no room beside the requests: all in the multi-instance kernel
+    packed.resize(n);
+    for (int i = 0; i < n; ++i) packed[i] = i;
+    bins.clear();
+    def.clear();
   }
   cudaStream_t st = s->stream;
-  cudaError_t e = cudaMemcpyAsync(s->d_inst, s->h_inst, sizeof(SweepArgs) * n, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(s->d_ctrl, 0, sizeof(Ctrl) * n, st);
+  unsigned char* base = static_cast<unsigned char*>(s->scratch);
+  cudaError_t e = cudaMemsetAsync(s->d_ctrl, 0, sizeof(Ctrl) * n, st);
   if (e == cudaSuccess) e = cudaEventRecord(s->ev0, st);
-  if (e == cudaSuccess) e = did::launch_sweep_multi(s->bf16, s->d_inst, n, begin, smem, st);
+  if (e == cudaSuccess && !packed.empty()) e = launch_packed(s, act, packed);
+  // RESIDENT: a launch per bin
+  const size_t ab = did::resident_args_bytes();
+  int at = 0;
+  for (Bin& b : bins) {
+    size_t words = 0, smem = 0;
+    int begin = 0;
+    for (size_t q = 0; q < b.slots.size(); ++q) {
+      Req* r = act[b.slots[q]];
+      SweepArgs a = slot_args(s, r, b.slots[q], std::min(s->round_sweeps, r->rq.max_iter - r->sweeps));
+      a.cta_begin = begin;
+      did::fill_resident_args(s->h_res + (at + q) * ab, b.plans[q], a, base + words, s->bf16);
+      r->sh_last = 0;
+      begin += b.plans[q].grid;
+      words += a256(b.plans[q].words_bytes);
+      smem = std::max(smem, b.plans[q].smem);
+    }
+    const int m = (int)b.slots.size();
+    if (e == cudaSuccess) e = cudaMemsetAsync(base, 0, words, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(s->d_res + at * ab, s->h_res + at * ab, ab * m, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = did::launch_resident_multi(s->d_res + at * ab, m, begin, smem, st);
+    at += m;
+  }
+  // DEFER: one after another on the whole GPU
+  const int G = did::refresh_tc_grid();
+  for (int i : def) {
+    Req* r = act[i];
+    DeferScratch d = defer_scratch(s, r, base);
+    d.b.ctrl = s->d_ctrl + i;
+    d.b.degen = s->d_degen + i;
+    r->sh_last = 0;
+    const double sweep_s =
+        r->rq.K * (20e-6 + (double)r->ld * r->rq.N * (s->bf16 ? 2.0 : 4.0) / 6.5e12);
+    const int nsw = std::max(1, std::min(std::min(s->round_sweeps, r->rq.max_iter - r->sweeps), (int)(kDeferSliceS / sweep_s)));
+    double* tr = s->d_trace + (size_t)i * s->round_sweeps;
+    did::DenseArgs da{};
+    da.X = r->X;
+    da.R = r->R;
+    da.B = r->B;
+    da.C = r->C;
+    da.part = s->d_part;
+    da.M = (int)r->rq.M;
+    da.ld = r->ld;
+    da.K = r->rq.K;
+    da.N = r->rq.N;
+    da.bf16 = s->bf16 ? 1 : 0;
+    if (e == cudaSuccess) e = cudaMemsetAsync(d.b.work, 0, sizeof(unsigned) * (r->rq.K + 1), st);
+    for (int q = 0; q < nsw && e == cudaSuccess; ++q) {
+      // (the partials of c_1 are in the scratch: another request may have used it since)
+      e = did::launch_defer(r->dplan, d.b, r->ld, r->rq.N, r->rq.K, q > 0 && d.tc_ws ? 2 * G : 0, 0, kServeTimeoutNs,
+                            nullptr, 0, st);
+      if (e == cudaSuccess)
+        e = d.tc_ws ? did::launch_refresh_tc(r->X, r->R, r->B, r->C, (int)r->rq.M, r->ld, r->rq.N, r->rq.K, d.tc_ws,
+                                             d.part, d.b.P, d.b.CC0, &d.b.ctrl->err, kServeTimeoutNs, st, !s->bf16)
+                    : did::launch_dense(da, st);
+      if (e == cudaSuccess)
+        e = did::launch_defer_close(d.tc_ws ? d.part : s->d_part, d.tc_ws ? G : s->dense_grid, d.tc_ws ? 1 : 3, d.b,
+                                    r->rq.K, tr + q, r->rq.tol > 0.0 ? 1 : 0, r->rq.tol, r->trace.back(),
+                                    r->trace.front(), q == 0, st);
+    }
+  }
   if (e == cudaSuccess) e = cudaEventRecord(s->ev1, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(s->h_ctrl, s->d_ctrl, sizeof(Ctrl) * n, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(s->h_trace, s->d_trace, sizeof(double) * n * s->round_sweeps, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess)
+  if (e == cudaSuccess && !packed.empty())
     e = cudaMemcpyAsync(s->h_stamp, s->d_stamp, sizeof(uint64_t) * n * 4 * kStampK, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  // the first sweep's time (its first kc k-steps, scaled to K) in CTA-seconds
-  for (int i = 0; i < n; ++i) {
+  // PACKED: the first sweep's time (its first kc k-steps, scaled to K) in CTA-seconds
+  for (int i : packed) {
     Req* r = act[i];
     if (s->h_ctrl[i].sweeps < 1 || s->h_ctrl[i].err != 0) continue;
     const int kc = std::min(r->rq.K, kStampK);
     const uint64_t* st4 = s->h_stamp + (size_t)i * 4 * kStampK;
     const uint64_t t0 = st4[0], t1 = st4[4 * (kc - 1) + 3];
     if (t1 <= t0) continue;
-    const double cs = (double)(t1 - t0) * 1e-9 * ((double)r->rq.K / kc) * (double)sh[i];
+    const double cs = (double)(t1 - t0) * 1e-9 * ((double)r->rq.K / kc) * (double)r->sh_last;
     r->cta_s = r->cta_s > 0.0 ? 0.5 * (r->cta_s + cs) : cs;
   }
   float ms = 0.f;
@@ -480,6 +722,8 @@ did_status did_server_create(size_t hbm_budget_bytes, did_precision precision, i
   ok = ok && cudaMallocHost(&s->h_trace, sizeof(double) * S * round_sweeps) == cudaSuccess;
   ok = ok && cudaMalloc(&s->d_stamp, sizeof(uint64_t) * S * 4 * kStampK) == cudaSuccess;
   ok = ok && cudaMallocHost(&s->h_stamp, sizeof(uint64_t) * S * 4 * kStampK) == cudaSuccess;
+  ok = ok && cudaMalloc(&s->d_res, did::resident_args_bytes() * S) == cudaSuccess;
+  ok = ok && cudaMallocHost(&s->h_res, did::resident_args_bytes() * S) == cudaSuccess;
   ok = ok && cudaMalloc(&s->d_degen, sizeof(unsigned long long) * S) == cudaSuccess;
   ok = ok && cudaMalloc(&s->d_bad, sizeof(unsigned long long)) == cudaSuccess;
   ok = ok && cudaMallocHost(&s->h_bad, sizeof(unsigned long long)) == cudaSuccess;
@@ -608,7 +852,10 @@ void did_server_destroy(did_server* s) {
     s->cv_work.notify_all();
   }
   if (s->worker.joinable()) s->worker.join();
+  if (s->scratch) cudaFreeAsync(s->scratch, s->stream);
   if (s->stream) cudaStreamSynchronize(s->stream);
+  cudaFree(s->d_res);
+  cudaFreeHost(s->h_res);
   for (auto& kv : s->reqs) {
     if (kv.second->block) cudaFree(kv.second->block);
     delete kv.second;

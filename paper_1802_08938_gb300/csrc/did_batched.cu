@@ -751,14 +751,25 @@ cudaError_t set_solve_smem(int K, int nu) {
 }
 
 // V (K x K, symmetric, float32) from the solve blocks' partials, added in block order.
-__global__ void vreduce_kernel(const double* Vp, int nblocks, int npairs, int K, float* V) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= npairs) return;
+// A warp of rows takes 32 pairs: warp w adds blocks w, w + 8, ..., then the
+// warps' sums in order (one thread a pair took 40 us of a 3.4 ms sweep, all latency).
+__global__ void __launch_bounds__(256) vreduce_kernel(const double* __restrict__ Vp, int nblocks, int npairs, int K,
+                                                      float* V) {
+  __shared__ double red[8][32];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int e = blockIdx.x * 32 + lane;
+  double s = 0.0;
+  if (e < npairs) {
+#pragma unroll 8
+    for (int b = w; b < nblocks; b += 8) s += Vp[(size_t)b * npairs + e];
+  }
+  red[w][lane] = s;
+  __syncthreads();
+  if (w != 0 || e >= npairs) return;
+  for (int q = 1; q < 8; ++q) s += red[q][lane];
   int i = 0, r = e;
   while (r >= K - i) { r -= K - i; ++i; }
   const int l = i + r;
-  double s = 0.0;
-  for (int b = 0; b < nblocks; ++b) s += Vp[(size_t)b * npairs + e];
   V[(size_t)i + (size_t)l * K] = (float)s;
   V[(size_t)l + (size_t)i * K] = (float)s;
 }
@@ -1301,11 +1312,28 @@ cudaError_t set_update_b_smem(int K) {
 }
 
 // YY = Y^T Y (2K x 2K column-major) over the ld rows of Y = [D | B]: block
-// (a, b0) forms entries (a, b0..b0+15); float32 within a thread's rows,
-// float64 across threads in a fixed tree.
+// (a, b0) forms entries (a, b0..b0+15); float32 within a thread's rows, then
+// float32 pairs across threads in a fixed tree, eight entries a time (float64
+// shuffles, which issue at 1/64 the rate, took most of the former 79 us).
 constexpr int kYYThreads = 256;
+struct YYPair {
+  float h, l;
+};
+__device__ __forceinline__ YYPair yy_add(YYPair a, YYPair b) {
+  const float s = __fadd_rn(a.h, b.h);
+  const float t = __fsub_rn(s, a.h);
+  float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t));
+  e = __fadd_rn(e, __fadd_rn(a.l, b.l));
+  YYPair r;
+  r.h = __fadd_rn(s, e);
+  r.l = __fsub_rn(e, __fsub_rn(r.h, s));
+  return r;
+}
+__device__ __forceinline__ YYPair yy_shfl(YYPair a, int m) {
+  return YYPair{__shfl_xor_sync(0xffffffffu, a.h, m), __shfl_xor_sync(0xffffffffu, a.l, m)};
+}
 __global__ void __launch_bounds__(kYYThreads) yy_kernel(const float* __restrict__ Y, int ld, int K2, float* YY) {
-  __shared__ double red[kYYThreads / 32][16];
+  __shared__ YYPair red[kYYThreads / 32][16];
   const int a = blockIdx.x, b0 = blockIdx.y * 16;
   float s[16];
 #pragma unroll
@@ -1318,22 +1346,35 @@ __global__ void __launch_bounds__(kYYThreads) yy_kernel(const float* __restrict_
   }
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
 #pragma unroll
-  for (int q = 0; q < 16; ++q) {
-    const double v = warp_sum_f64((double)s[q]);
-    if (l == 0) red[w][q] = v;
+  for (int g = 0; g < 2; ++g) {
+    YYPair v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = YYPair{s[8 * g + q], 0.f};
+#pragma unroll
+    for (int m = 4; m >= 1; m >>= 1) {
+      const bool up = (l & m) != 0;
+#pragma unroll
+      for (int q = 0; q < m; ++q) {
+        const YYPair send = up ? v[q] : v[q + m], keep = up ? v[q + m] : v[q];
+        v[q] = yy_add(keep, yy_shfl(send, m));
+      }
+    }
+    v[0] = yy_add(v[0], yy_shfl(v[0], 8));
+    v[0] = yy_add(v[0], yy_shfl(v[0], 16));
+    if (l < 8) red[w][8 * g + l] = v[0];           // lane l has entry l of the eight
   }
   __syncthreads();
   if (threadIdx.x < 16 && b0 + (int)threadIdx.x < K2) {
-    double t = 0.0;
-    for (int i = 0; i < kYYThreads / 32; ++i) t += red[i][threadIdx.x];
-    YY[(size_t)a + (size_t)(b0 + threadIdx.x) * K2] = (float)t;
+    YYPair t = red[0][threadIdx.x];
+    for (int i = 1; i < kYYThreads / 32; ++i) t = yy_add(t, red[i][threadIdx.x]);
+    YY[(size_t)a + (size_t)(b0 + threadIdx.x) * K2] = t.h;
   }
 }
 
 // f after the sweep: ||E'||^2 from the update pass, then the B step identity.
 __global__ void objective_kernel(const double* part_n, int nn, const double* part_b, int nb, const float* YY,
                                  const float* V, int K, double* state, double* trace_out) {
-  __shared__ double red[8];
+  __shared__ double red[10];
   double s = 0.0;
   const int K2 = 2 * K;
   for (int idx = threadIdx.x; idx < K * K; idx += blockDim.x) {
@@ -1342,13 +1383,17 @@ __global__ void objective_kernel(const double* part_n, int nn, const double* par
   }
   s = warp_sum_f64(s);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  // ||E'||^2 after the C step and the B step's sum, a warp each (a fixed order)
+  if (threadIdx.x < 64) {
+    const bool first = threadIdx.x < 32;
+    const double v = warp_sum_global_f64(first ? part_n : part_b, first ? nn : nb, 1);
+    if ((threadIdx.x & 31) == 0) red[first ? 8 : 9] = v;
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
     double qv = 0.0;
     for (int i = 0; i < (int)(blockDim.x >> 5); ++i) qv += red[i];
-    double e2c = 0.0, dw = 0.0;
-    for (int i = 0; i < nn; ++i) e2c += part_n[i];   // ||E'||^2 after the C step
-    for (int i = 0; i < nb; ++i) dw += part_b[i];
+    const double e2c = red[8], dw = red[9];
     const double e2b = e2c - 2.0 * dw + qv;       // after the B step
     state[0] = e2b;
     *trace_out = 0.5 * e2b;
@@ -1551,7 +1596,7 @@ cudaError_t batched_sweep(BatchedState* b, float* R, float* Y, float* C, int ld,
   sa.N = N;
   e = launch_solve(sa, P.sgrid, s);
   if (e != cudaSuccess) return e;
-  vreduce_kernel<<<(P.npairs + 127) / 128, 128, 0, s>>>(b->Vp, P.sgrid, P.npairs, K, b->V);
+  vreduce_kernel<<<(P.npairs + 31) / 32, 256, 0, s>>>(b->Vp, P.sgrid, P.npairs, K, b->V);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   // R_s := R_s - [D B] [C_old; dl], ||E'||^2, W = E' C'^T partials

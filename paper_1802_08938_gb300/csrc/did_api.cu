@@ -9,6 +9,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <initializer_list>
 #include <string>
 #include <vector>
 
@@ -50,7 +51,7 @@ struct did_ctx {
   double* dense_part = nullptr;
   unsigned long long* bad = nullptr;
   did::BatchedState* batched = nullptr;   // DID_ORDER_DID_BATCHED
-  void* tc_ws = nullptr;            // tensor-core refresh operands (allocated on first use)
+  void* tc_ws = nullptr;            // tensor-core refresh operands
   double* tc_part = nullptr;        // per-CTA sums of the tensor-core refresh
   int* tc_err = nullptr;
   int64_t tc_refreshes = 0;
@@ -61,6 +62,8 @@ struct did_ctx {
   Ctrl* ctrl_host = nullptr;        // pinned
   double* trace_host = nullptr;     // pinned, kMaxSweepsPerLaunch
   double* part_host = nullptr;      // pinned, 3 * dense grid
+  int* err_host = nullptr;          // pinned
+  unsigned long long* bad_host = nullptr;   // pinned, 3
 
   did::SweepPlan plan{};
   bool resident = false;            // R fits the SMs' shared memory: sweeps keep it there
@@ -162,13 +165,27 @@ did_status copy_in_padded(did_ctx* c, float* dst, int ld, const float* src, int6
   return DID_OK;
 }
 
-did_status check_nonneg(did_ctx* c, const float* p, int rows, int ld, int64_t cols, const char* what) {
-  DID_CUDA(c, cudaMemsetAsync(c->bad, 0, sizeof(unsigned long long), c->stream));
-  DID_CUDA(c, did::launch_check_nonneg_finite(p, rows, ld, cols, c->bad, c->stream));
-  unsigned long long nbad = 0;
-  DID_CUDA(c, cudaMemcpyAsync(&nbad, c->bad, sizeof(nbad), cudaMemcpyDeviceToHost, c->stream));
+// Negative or non-finite entries of up to three device matrices, counted with
+// one synchronisation; the first that has any is reported.
+struct CheckItem {
+  const float* p;
+  int rows, ld;
+  int64_t cols;
+  const char* what;
+};
+did_status check_nonneg(did_ctx* c, std::initializer_list<CheckItem> items) {
+  DID_CUDA(c, cudaMemsetAsync(c->bad, 0, items.size() * sizeof(unsigned long long), c->stream));
+  int i = 0;
+  for (const CheckItem& q : items)
+    DID_CUDA(c, did::launch_check_nonneg_finite(q.p, q.rows, q.ld, q.cols, c->bad + i++, c->stream));
+  DID_CUDA(c, cudaMemcpyAsync(c->bad_host, c->bad, items.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+                              c->stream));
   DID_CUDA(c, cudaStreamSynchronize(c->stream));
-  if (nbad) return fail(c, DID_EINVAL, "%s has %llu negative or non-finite entries", what, nbad);
+  i = 0;
+  for (const CheckItem& q : items) {
+    const unsigned long long nbad = c->bad_host[i++];
+    if (nbad) return fail(c, DID_EINVAL, "%s has %llu negative or non-finite entries", q.what, nbad);
+  }
   return DID_OK;
 }
 
@@ -180,7 +197,7 @@ did_status check_source(did_ctx* c, const float* p, int64_t rows, int64_t cols, 
   const cudaError_t e = cudaPointerGetAttributes(&attr, p);
   cudaGetLastError();
   if (e == cudaSuccess && (attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged))
-    return check_nonneg(c, p, (int)rows, (int)rows, cols, what);
+    return check_nonneg(c, {{p, (int)rows, (int)rows, cols, what}});
   unsigned long long nbad = 0;
   const size_t n = (size_t)rows * (size_t)cols;
   for (size_t i = 0; i < n; ++i) {
@@ -221,32 +238,9 @@ did_status dense(did_ctx* c, int mode, double sums[3]) {
   return DID_OK;
 }
 
-// Workspace of the tensor-core refresh (on first use).
-did_status refresh_tc_workspace(did_ctx* c) {
-  void* p;
-  did_status st;
-  const int G = did::refresh_tc_grid();
-  if (!c->tc_ws) {
-    st = dev_alloc(c, &p, did::refresh_tc_workspace_bytes((int)c->M, c->ld, c->N, c->K, !c->bf16));
-    if (st != DID_OK) return st;
-    c->tc_ws = p;
-    st = dev_alloc(c, &p, sizeof(double) * G);
-    if (st != DID_OK) return st;
-    c->tc_part = (double*)p;
-    st = dev_alloc(c, &p, sizeof(int) * 4);
-    if (st != DID_OK) return st;
-    c->tc_err = (int*)p;
-  }
-  return DID_OK;
-}
-
 // Tensor-core refresh; returns 1/2 ||R||^2 in *f.
 did_status refresh_tc(did_ctx* c, double* f) {
-  const did_status st = refresh_tc_workspace(c);
-  if (st != DID_OK) return st;
   const int G = did::refresh_tc_grid();
-  std::vector<double> part(G);
-  int herr = 0;
   // The interleaved order's first b-update takes the partials of R c_1^T
   // that the refresh forms in its epilogue (the P and CCp buffers hold at
   // least 2 G rows); the other orders do not use them.
@@ -260,19 +254,20 @@ did_status refresh_tc(did_ctx* c, double* f) {
                                      wait_limit_ns(c), c->stream,
                                      !c->bf16));
   DID_CUDA(c, cudaEventRecord(c->ev1, c->stream));
-  DID_CUDA(c, cudaMemcpyAsync(part.data(), c->tc_part, sizeof(double) * G, cudaMemcpyDeviceToHost, c->stream));
-  DID_CUDA(c, cudaMemcpyAsync(&herr, c->tc_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  DID_CUDA(c, cudaMemcpyAsync(c->part_host, c->tc_part, sizeof(double) * G, cudaMemcpyDeviceToHost, c->stream));
+  DID_CUDA(c, cudaMemcpyAsync(c->err_host, c->tc_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   DID_CUDA(c, cudaStreamSynchronize(c->stream));
   float ms = 0.f;
   DID_CUDA(c, cudaEventElapsedTime(&ms, c->ev0, c->ev1));
   c->tc_ms += ms;
   c->tc_refreshes++;
+  const int herr = *c->err_host;
   if (herr != 0) {
     c->need_refresh = true;
     return fail(c, DID_ETIMEOUT, "tensor-core refresh: a bounded wait ran out (device error %d)", herr);
   }
   double sum = 0.0;
-  for (int i = 0; i < G; ++i) sum += part[i];
+  for (int i = 0; i < G; ++i) sum += c->part_host[i];
   *f = 0.5 * sum;
   if (fuse) c->npart_first = 2 * G;
   return DID_OK;
@@ -633,8 +628,6 @@ static did_status create_impl(did_ctx* c, const float* X, uint64_t seed) {
   ALLOC(X, elems * sizeof(float));
   ALLOC(R, elems * (c->bf16 ? 2 : 4));
   ALLOC(Y, (size_t)c->ld * 2 * K * sizeof(float));
-  c->B = c->Y + (size_t)K * c->ld;
-  DID_CUDA(c, cudaMemsetAsync(c->Y, 0, (size_t)c->ld * K * sizeof(float), c->stream));
   ALLOC(C, (size_t)K * N * sizeof(float));
   // partial rows: the plan's, and the tensor-core refresh's two per CTA
   const size_t U = (size_t)std::max(std::max(c->defer ? c->dplan.npart : c->plan.npart, G), 2 * did::refresh_tc_grid());
@@ -643,12 +636,8 @@ static did_status create_impl(did_ctx* c, const float* X, uint64_t seed) {
   ALLOC(Sp, (size_t)2 * G * sizeof(double));
   ALLOC(OBJp, U * sizeof(double));
   ALLOC(bold, (size_t)c->ld * sizeof(float));
-  if (c->resident) {
-    ALLOC(res_words, c->rplan.words_bytes);
-    DID_CUDA(c, cudaMemsetAsync(c->res_words, 0, c->rplan.words_bytes, c->stream));
-  }
+  if (c->resident) ALLOC(res_words, c->rplan.words_bytes);
   if (c->defer) {
-    did::DeferBuffers& d = c->dbuf;
     const size_t W = (size_t)c->dplan.GS / 32;
     ALLOC(dbuf.Bo, (size_t)c->ld * K * sizeof(float));
     ALLOC(dbuf.Co, (size_t)K * N * sizeof(float));
@@ -657,11 +646,6 @@ static did_status create_impl(did_ctx* c, const float* X, uint64_t seed) {
     ALLOC(dbuf.Xp, did::defer_pair_bytes(K, c->dplan.grid));
     ALLOC(dbuf.Yp, did::defer_pair_bytes(K, c->dplan.grid));
     ALLOC(dbuf.work, (size_t)(K + 1) * sizeof(unsigned));
-    d.R = c->R;
-    d.B = c->B;
-    d.C = c->C;
-    d.P = c->P;
-    d.CC0 = c->CCp;
   } else if (c->plan.lazy && !c->resident) {
     ALLOC(Cold, (size_t)N * sizeof(float));
     ALLOC(XCp, 2 * U * sizeof(double));
@@ -669,37 +653,51 @@ static did_status create_impl(did_ctx* c, const float* X, uint64_t seed) {
   ALLOC(ctrl, sizeof(Ctrl));
   ALLOC(trace_dev, sizeof(double) * kMaxSweepsPerLaunch);
   ALLOC(degen, sizeof(unsigned long long));
-  c->dbuf.ctrl = c->ctrl;
-  c->dbuf.degen = c->degen;
   ALLOC(dense_part, sizeof(double) * 3 * c->dense_grid);
-  ALLOC(bad, sizeof(unsigned long long));
+  ALLOC(bad, 3 * sizeof(unsigned long long));
   if (c->opt.flags & DID_FLAG_PHASE_TIMES) {
     c->tstamp_cap = 1 << 14;
     ALLOC(tstamp, sizeof(uint64_t) * 4 * c->tstamp_cap);
   }
-#undef ALLOC
+  if (did::refresh_tc_supported(K, !c->bf16) && !(c->opt.flags & DID_FLAG_SIMT_REFRESH)) {
+    ALLOC(tc_ws, did::refresh_tc_workspace_bytes((int)M, c->ld, N, K, !c->bf16));
+    ALLOC(tc_part, sizeof(double) * did::refresh_tc_grid());
+    ALLOC(tc_err, sizeof(int) * 4);
+  }
+  void* bws = nullptr;
   if (c->opt.order == DID_ORDER_DID_BATCHED) {
     const size_t wsb = did::batched_workspace_bytes(c->ld, N, K);
     if (wsb == 0) return fail(c, DID_EINVAL, "the batched order supports K <= 64");
-    st = dev_alloc(c, &p, wsb);
+    st = dev_alloc(c, &bws, wsb);
     if (st != DID_OK) return st;
-    c->batched = did::batched_create(p, c->ld, N, K, c->stream);
+  }
+#undef ALLOC
+  c->B = c->Y + (size_t)K * c->ld;
+  DID_CUDA(c, cudaMemsetAsync(c->Y, 0, (size_t)c->ld * K * sizeof(float), c->stream));
+  if (c->resident) DID_CUDA(c, cudaMemsetAsync(c->res_words, 0, c->rplan.words_bytes, c->stream));
+  c->dbuf.R = c->R;
+  c->dbuf.B = c->B;
+  c->dbuf.C = c->C;
+  c->dbuf.P = c->P;
+  c->dbuf.CC0 = c->CCp;
+  c->dbuf.ctrl = c->ctrl;
+  c->dbuf.degen = c->degen;
+  if (bws) {
+    c->batched = did::batched_create(bws, c->ld, N, K, c->stream);
     if (!c->batched) return fail(c, DID_ECUDA, "batched-order set-up failed");
   }
-  st = host_alloc(c, &p, sizeof(Ctrl));
+  // pinned, one allocation: control words, error word, counters, then the two arrays
+  static_assert(sizeof(Ctrl) <= 64, "control words fit their slot");
+  st = host_alloc(c, &p, 128 + sizeof(double) * (kMaxSweepsPerLaunch + 3 * (size_t)c->dense_grid));
   if (st != DID_OK) return st;
   c->ctrl_host = (Ctrl*)p;
-  st = host_alloc(c, &p, sizeof(double) * kMaxSweepsPerLaunch);
-  if (st != DID_OK) return st;
-  c->trace_host = (double*)p;
-  st = host_alloc(c, &p, sizeof(double) * 3 * c->dense_grid);
-  if (st != DID_OK) return st;
-  c->part_host = (double*)p;
+  c->err_host = (int*)((unsigned char*)p + 64);
+  c->bad_host = (unsigned long long*)((unsigned char*)p + 72);
+  c->trace_host = (double*)((unsigned char*)p + 128);
+  c->part_host = c->trace_host + kMaxSweepsPerLaunch;
 
   DID_CUDA(c, cudaMemsetAsync(c->degen, 0, sizeof(unsigned long long), c->stream));
   st = copy_in_padded(c, c->X, c->ld, X, M, N);
-  if (st != DID_OK) return st;
-  st = check_nonneg(c, c->X, (int)M, c->ld, N, "X");
   if (st != DID_OK) return st;
 
   if (c->opt.B_init) {
@@ -713,9 +711,9 @@ static did_status create_impl(did_ctx* c, const float* X, uint64_t seed) {
   } else {
     DID_CUDA(c, did::launch_gen_uniform(c->C, (int64_t)K * N, seed, 5, c->stream));
   }
-  st = check_nonneg(c, c->B, (int)M, c->ld, K, "B start point");
-  if (st != DID_OK) return st;
-  st = check_nonneg(c, c->C, K, K, N, "C start point");
+  st = check_nonneg(c, {{c->X, (int)M, c->ld, N, "X"},
+                        {c->B, (int)M, c->ld, K, "B start point"},
+                        {c->C, K, K, N, "C start point"}});
   if (st != DID_OK) return st;
 
   if (c->opt.init_scale) {

@@ -145,8 +145,8 @@ __global__ void __launch_bounds__(kDenseThreads) dense_kernel(DenseTileArgs t) {
 // sums are float32 pairs until the end.  The next chunk of B and C is loaded into
 // registers while this one is used.  Each product is the same chain of FMAs in k
 // order, so R comes out bit for bit the same.  Measured: 10000 x 100000,
-// K = 100 (exact objective) 11.9 -> 5.9 ms; 8165 x 18821, K = 100, a refresh and an
-// objective 3.8 -> 1.4 ms.
+// K = 100 (exact objective) 11.9 -> 5.9 ms; 8165 x 18821, K = 100, a refresh or an
+// objective 1.9 -> 0.95 ms.
 constexpr int kBig = 128;
 constexpr int kBigKc = 16;
 constexpr int kBigThreads = 256;

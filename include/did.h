@@ -122,7 +122,8 @@ typedef struct {
  * (K <= 128) only read R:
  * the changes of a sweep stay pending as vectors, and R is formed anew from X
  * after its last k (did_info then counts a periodic refresh that falls due,
- * which finds R formed from the current factors already).
+ * which finds R formed from the current factors already); so do those of
+ * DID_ORDER_DID (with columns up to about 8000 rows, a pass then serving several k).
  * Deferred write-back defers the
  * write of R for k to the pass for k+1 (one write per pair of k, three passes
  * over R per pair instead of four).  It needs two more M-vectors of shared

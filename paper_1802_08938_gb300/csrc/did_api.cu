@@ -73,6 +73,9 @@ struct did_ctx {
   bool defer = false;               // interleaved sweeps read R only and form it anew after each sweep
   did::DeferPlan dplan{};
   did::DeferBuffers dbuf{};
+  bool cfirst = false;              // the same for the C-first order
+  did::CfirstPlan cplan{};
+  did::CfirstBuffers cbuf{};
   int dense_grid = 0;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   int64_t sweep_launches = 0, prologue_launches = 0, dense_launches = 0;
@@ -440,8 +443,8 @@ did_status run_batched(did_ctx* c, int64_t max_sweeps, int stop_rule, double tol
   return DID_OK;
 }
 
-// Interleaved order by read-only sweeps: each sweep is the K passes of the
-// sweep kernel over a residual that it does not write, then R = X - B C on the
+// Read-only sweeps of the per-k orders: each sweep is the passes of the
+// sweep kernels over a residual that it does not write, then R = X - B C on the
 // tensor cores (with 1/2 ||R||^2 and the partials of R c_1^T), or by the float32
 // pass where those do not take K.  A periodic
 // refresh that falls due finds R formed from the current factors already.
@@ -460,8 +463,10 @@ did_status run_defer(did_ctx* c, int64_t max_sweeps, int stop_rule, double tol, 
   da.K = c->K;
   da.N = c->N;
   da.bf16 = c->bf16 ? 1 : 0;
+  unsigned* work = c->cfirst ? c->cbuf.work : c->dbuf.work;
+  const int nwork = c->cfirst ? 2 * c->K : c->K + 1;
   while (*done_total < max_sweeps) {
-    if (c->need_refresh || (tc && c->npart_first == 0)) {
+    if (c->need_refresh || (c->defer && tc && c->npart_first == 0)) {
       did_status st = refresh(c);
       if (st != DID_OK) return st;
     } else if (refresh_due(c)) {
@@ -477,21 +482,25 @@ did_status run_defer(did_ctx* c, int64_t max_sweeps, int stop_rule, double tol, 
     const int cap = c->tstamp ? (int)std::min<int64_t>((int64_t)n * c->K, c->tstamp_cap) : 0;
     c->tstamp_n = cap;
     DID_CUDA(c, cudaMemsetAsync(c->ctrl, 0, sizeof(Ctrl), c->stream));
-    DID_CUDA(c, cudaMemsetAsync(c->dbuf.work, 0, sizeof(unsigned) * (c->K + 1), c->stream));
+    DID_CUDA(c, cudaMemsetAsync(work, 0, sizeof(unsigned) * nwork, c->stream));
     DID_CUDA(c, cudaEventRecord(c->ev0, c->stream));
     for (int s = 0; s < n; ++s) {
       const int step0 = s * c->K;
-      DID_CUDA(c, did::launch_defer(c->dplan, c->dbuf, c->ld, c->N, c->K, c->npart_first, c->opt.debug_barrier_extra,
-                                    tmo, step0 < cap ? c->tstamp + 4 * (size_t)step0 : nullptr,
-                                    std::max(0, cap - step0), c->stream));
+      if (c->cfirst)
+        DID_CUDA(c, did::launch_cfirst(c->cplan, c->cbuf, c->ld, c->N, c->K, c->opt.debug_barrier_extra, tmo, c->stream));
+      else
+        DID_CUDA(c, did::launch_defer(c->dplan, c->dbuf, c->ld, c->N, c->K, c->npart_first, c->opt.debug_barrier_extra,
+                                      tmo, step0 < cap ? c->tstamp + 4 * (size_t)step0 : nullptr,
+                                      std::max(0, cap - step0), c->stream));
       if (tc) {
         DID_CUDA(c, did::launch_refresh_tc(c->X, c->R, c->B, c->C, (int)c->M, c->ld, c->N, c->K, c->tc_ws, c->tc_part,
-                                           c->P, c->CCp, &c->ctrl->err, tmo, c->stream, !c->bf16));
-        DID_CUDA(c, did::launch_defer_close(c->tc_part, G, 1, c->dbuf, c->K, c->trace_dev + s,
+                                           c->defer ? c->P : nullptr, c->defer ? c->CCp : nullptr, &c->ctrl->err,
+                                           tmo, c->stream, !c->bf16));
+        DID_CUDA(c, did::launch_defer_close(c->tc_part, G, 1, c->ctrl, work, nwork, c->trace_dev + s,
                                              stop_rule, tol, f_start, f0, s == 0, c->stream));
       } else {
         DID_CUDA(c, did::launch_dense(da, c->stream));
-        DID_CUDA(c, did::launch_defer_close(c->dense_part, c->dense_grid, 3, c->dbuf, c->K, c->trace_dev + s,
+        DID_CUDA(c, did::launch_defer_close(c->dense_part, c->dense_grid, 3, c->ctrl, work, nwork, c->trace_dev + s,
                                              stop_rule, tol, f_start, f0, s == 0, c->stream));
       }
     }
@@ -521,7 +530,7 @@ did_status run_defer(did_ctx* c, int64_t max_sweeps, int stop_rule, double tol, 
 }
 
 did_status run(did_ctx* c, int64_t max_sweeps, int stop_rule, double tol, int64_t* done_total) {
-  if (c->defer) return run_defer(c, max_sweeps, stop_rule, tol, done_total);
+  if (c->defer || c->cfirst) return run_defer(c, max_sweeps, stop_rule, tol, done_total);
   if (c->batched) return run_batched(c, max_sweeps, stop_rule, tol, done_total);
   *done_total = 0;
   while (*done_total < max_sweeps) {
@@ -608,11 +617,14 @@ static did_status create_impl(did_ctx* c, const float* X, uint64_t seed) {
                                           DID_FLAG_SIMT_REFRESH));
   c->resident = no_flags && c->opt.order != DID_ORDER_DID_BATCHED &&
                 did::plan_resident(c->ld, N, K, c->opt.grid_ctas, &c->rplan);
-  // Sweeps that only read R; the tensor-core refresh forms it after each, or for
+  // Sweeps that only read R (below also the C-first order's); the tensor-core refresh forms it after each, or for
   // other K the float32 pass (and the next sweep a first pass for c_1).
   c->defer = !c->resident && no_flags && c->opt.order == DID_ORDER_INTERLEAVED &&
              defer_pays(c) &&
              did::plan_defer(c->ld, N, K, c->bf16, c->opt.grid_ctas, &c->dplan);
+  c->cfirst = !c->resident && no_flags && c->opt.order == DID_ORDER_DID && c->opt.grid_ctas <= 0 &&
+              !(c->opt.flags & DID_FLAG_PHASE_TIMES) && defer_pays(c) &&
+              did::plan_cfirst(c->ld, N, K, c->bf16, &c->cplan);
   c->dense_grid = did::dense_grid();
   DID_CUDA(c, cudaEventCreate(&c->ev0));
   DID_CUDA(c, cudaEventCreate(&c->ev1));
@@ -646,6 +658,14 @@ static did_status create_impl(did_ctx* c, const float* X, uint64_t seed) {
     ALLOC(dbuf.Xp, did::defer_pair_bytes(K, c->dplan.grid));
     ALLOC(dbuf.Yp, did::defer_pair_bytes(K, c->dplan.grid));
     ALLOC(dbuf.work, (size_t)(K + 1) * sizeof(unsigned));
+  } else if (c->cfirst) {
+    const did::CfirstSizes z = did::cfirst_sizes(c->cplan, c->ld, N, K);
+    ALLOC(cbuf.Co, z.Co);
+    ALLOC(cbuf.T, z.T);
+    ALLOC(cbuf.P, z.P);
+    ALLOC(cbuf.Gp, z.Gp);
+    ALLOC(cbuf.Xp, z.Xp);
+    ALLOC(cbuf.work, (size_t)2 * K * sizeof(unsigned));
   } else if (c->plan.lazy && !c->resident) {
     ALLOC(Cold, (size_t)N * sizeof(float));
     ALLOC(XCp, 2 * U * sizeof(double));
@@ -675,6 +695,11 @@ static did_status create_impl(did_ctx* c, const float* X, uint64_t seed) {
   c->B = c->Y + (size_t)K * c->ld;
   DID_CUDA(c, cudaMemsetAsync(c->Y, 0, (size_t)c->ld * K * sizeof(float), c->stream));
   if (c->resident) DID_CUDA(c, cudaMemsetAsync(c->res_words, 0, c->rplan.words_bytes, c->stream));
+  c->cbuf.R = c->R;
+  c->cbuf.B = c->B;
+  c->cbuf.C = c->C;
+  c->cbuf.ctrl = c->ctrl;
+  c->cbuf.degen = c->degen;
   c->dbuf.R = c->R;
   c->dbuf.B = c->B;
   c->dbuf.C = c->C;
@@ -887,11 +912,11 @@ did_status did_get_info(did_ctx* c, did_info* info) {
   info->K = c->K;
   info->precision = c->opt.precision;
   info->order = c->opt.order;
-  info->grid_ctas = c->resident ? c->rplan.grid : c->defer ? c->dplan.grid : c->plan.grid;
-  info->group_threads = c->defer ? c->dplan.GS : c->plan.GS;
+  info->grid_ctas = c->cfirst ? c->cplan.grid : c->resident ? c->rplan.grid : c->defer ? c->dplan.grid : c->plan.grid;
+  info->group_threads = c->cfirst ? c->cplan.GS : c->defer ? c->dplan.GS : c->plan.GS;
   info->vecs_per_thread = c->defer ? c->dplan.NR : c->plan.NR;
-  info->column_units = c->defer ? c->dplan.nunits : c->plan.nunits;
-  info->dynamic_units = c->defer ? c->dplan.dynamic : c->plan.dynamic;
+  info->column_units = c->cfirst ? c->cplan.nunits : c->defer ? c->dplan.nunits : c->plan.nunits;
+  info->dynamic_units = c->cfirst ? c->cplan.dynamic : c->defer ? c->dplan.dynamic : c->plan.dynamic;
   info->ld = c->ld;
   info->sweeps_done = c->sweeps_done;
   unsigned long long d = 0;

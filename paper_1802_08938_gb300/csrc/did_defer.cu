@@ -20,10 +20,10 @@ namespace {
 // Closes a sweep: f = 1/2 ||R||^2 from the refresh's per-CTA sums (added in
 // order), the stopping rule, and the barrier and the unit counters cleared
 // for the next launch.  Nothing after a sweep that stopped or failed.
-__global__ void defer_close_kernel(const double* part, int n, int stride, Ctrl* ctrl, unsigned* work, int K, double* trace,
+__global__ void defer_close_kernel(const double* part, int n, int stride, Ctrl* ctrl, unsigned* work, int nwork, double* trace,
                                    int stop_rule, double tol, double f_prev, double f0, int first) {
   if (ctrl->stopped || ctrl->err) return;
-  for (int i = threadIdx.x; i <= K; i += blockDim.x) work[i] = 0u;
+  for (int i = threadIdx.x; i < nwork; i += blockDim.x) work[i] = 0u;
   if (threadIdx.x == 0) {
     double s = 0.0;
     for (int i = 0; i < n; ++i) s += part[(size_t)i * stride];
@@ -150,9 +150,9 @@ cudaError_t launch_defer(const DeferPlan& plan, const DeferBuffers& b, int ld, i
   return cudaLaunchCooperativeKernel(plan.func, dim3(plan.grid), dim3(kDeferThreads), params, plan.smem, s);
 }
 
-cudaError_t launch_defer_close(const double* part, int n, int stride, const DeferBuffers& b, int K, double* trace,
+cudaError_t launch_defer_close(const double* part, int n, int stride, Ctrl* ctrl, unsigned* work, int nwork, double* trace,
                                int stop_rule, double tol, double f_prev, double f0, bool first, cudaStream_t s) {
-  defer_close_kernel<<<1, 128, 0, s>>>(part, n, stride, b.ctrl, b.work, K, trace, stop_rule, tol, f_prev, f0,
+  defer_close_kernel<<<1, 128, 0, s>>>(part, n, stride, ctrl, work, nwork, trace, stop_rule, tol, f_prev, f0,
                                        first ? 1 : 0);
   return cudaGetLastError();
 }

@@ -268,6 +268,129 @@ __device__ __forceinline__ void sum_over_ctas(const df* part, int n, int G, df* 
   }
 }
 
+// The producer warp.  Passes `first` to `last` - 1 one after another: the chunks of the CTA's units in order, dealt to the
+// groups in turn (a unit is padded to whole rounds with empty chunks, so
+// every group sees every unit), then a round of end marks.  The lanes take a
+// block of up to S chunks, one each: a lane waits until its stage's last chunk
+// has been read, puts NCX values of each of the chunk's columns (rows(pass, i),
+// i < NCX; null: zeros) and the column index beside it, and issues the copy.
+struct Stream {
+  const void* R;
+  int64_t N;
+  uint32_t colbytes;
+  unsigned char* ring;
+  StageMeta* meta;
+  float* cxs;              // [S][cx_stride], column e, row i of a chunk at e * NCX + i
+  int cx_stride;
+  uint64_t *full, *empty;
+  int S, NG, G, cta;
+  Units units;
+  int nunits, dynamic;
+  unsigned* work;          // unit counter of pass k at work[k - first]
+  volatile int* quit;
+  int* err;
+  uint64_t timeout_ns;
+};
+template <int CW, int NCX, typename Rows>
+__device__ __forceinline__ void produce(const Stream& a, int first, int last, Rows rows) {
+  const int lane = threadIdx.x & 31;
+  const int S = a.S, NG = a.NG;
+  const int64_t N = a.N;
+  const uint32_t stagebytes = (uint32_t)CW * a.colbytes;
+  int* err = a.err;
+  const uint64_t tmo = a.timeout_ns;
+  const int BL = S < 32 ? S : 32;
+  unsigned base = 0;                          // chunks issued before this block
+  bool ok = true;
+  float c[CW * NCX];
+  auto put = [&](bool mine, int64_t j, int n, int u, int count) {   // count: lanes of the block
+    const unsigned q = base + (unsigned)lane;
+    const unsigned st = q % (unsigned)S, round = q / (unsigned)S;
+    bool todo = mine;
+    uint64_t t0 = 0;
+    for (unsigned i = 1; __any_sync(0xffffffffu, todo); ++i) {
+      if (todo && (round == 0 || mbar_try_wait(a.empty + st, (round - 1) & 1u))) {
+        todo = false;
+#pragma unroll
+        for (int e = 0; e < CW * NCX; ++e) a.cxs[st * a.cx_stride + e] = c[e];
+        a.meta[st].j = j;
+        a.meta[st].n = n;
+        a.meta[st].u = u;
+        if (n > 0) {
+          mbar_arrive_expect_tx(a.full + st, (uint32_t)n * a.colbytes);
+          bulk_load(a.ring + (size_t)st * stagebytes,
+                    reinterpret_cast<const unsigned char*>(a.R) + (size_t)j * a.colbytes, (uint32_t)n * a.colbytes,
+                    a.full + st);
+        } else {
+          mbar_arrive(a.full + st);
+        }
+      }
+      if ((i & 63u) == 0) {                   // bounded
+        const uint64_t tn = globaltimer_ns();
+        if (t0 == 0) t0 = tn;
+        if (*a.quit) ok = false;
+        if (tn - t0 > tmo || i > (1u << 28)) {
+          if (todo) atomicCAS(err, 0, kDevErrTimeout);
+          ok = false;
+        }
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+      }
+    }
+    if (ok) {
+      base += (unsigned)count;
+    } else {
+      // this block's copies that were issued land before the CTA exits (bounded)
+      if (mine && !todo) mbar_wait_bounded(a.full + st, round & 1u, err, tmo);
+      __syncwarp();
+    }
+  };
+  for (int k = first; k < last && ok; ++k) {
+    auto grab = [&]() -> unsigned { return lane == 0 ? atomicAdd(a.work + (k - first), 1u) : 0u; };   // lane 0 has it
+    // the first unit is the CTA's own (a CTA that runs ahead into this pass must
+    // not take two large ones); the others come from the counter, asked for
+    // a block before they are needed
+    int64_t u = a.cta;
+    while (u < a.nunits && ok) {
+      unsigned unext = 0u;
+      int64_t lo, hi;
+      unit_range(a.units, N, u, lo, hi);
+      const int64_t chunks = (hi - lo + CW - 1) / CW;
+      const int64_t total = (chunks > 0 ? (chunks + NG - 1) / NG : 1) * NG;
+      auto load_c = [&](int64_t i) {          // the rows on chunk i of the unit
+        const int64_t j = lo + i * CW;
+#pragma unroll
+        for (int r = 0; r < NCX; ++r) {
+          const float* cn = rows(k, r);
+#pragma unroll
+          for (int e = 0; e < CW; ++e) c[e * NCX + r] = cn && i < total && j + e < hi ? __ldcg(cn + j + e) : 0.f;
+        }
+      };
+      load_c(lane);
+      for (int64_t i0 = 0; i0 < total && ok; i0 += BL) {
+        const int count = (int)(total - i0 < BL ? total - i0 : BL);
+        if (a.dynamic && i0 + BL >= total) unext = grab();
+        const int64_t j = lo + (i0 + lane) * CW;
+        const int n = j < hi ? (int)(hi - j < CW ? hi - j : CW) : 0;
+        put(lane < count, j, n, (int)u, count);
+        if (i0 + BL < total) load_c(i0 + BL + lane);
+      }
+      u = a.dynamic ? (int64_t)a.G + (int64_t)__shfl_sync(0xffffffffu, unext, 0) : (int64_t)a.nunits;
+    }
+    for (int i0 = 0; i0 < NG && ok; i0 += BL) {
+#pragma unroll
+      for (int e = 0; e < CW * NCX; ++e) c[e] = 0.f;
+      const int count = NG - i0 < BL ? NG - i0 : BL;
+      put(lane < count, 0, -1, 0, count);
+    }
+  }
+  // earlier copies still in flight land before the CTA exits (bounded)
+  if (!ok && lane == 0) {
+    for (unsigned d = base > (unsigned)S ? base - (unsigned)S : 0u; d < base; ++d)
+      mbar_wait_bounded(a.full + d % (unsigned)S, (d / (unsigned)S) & 1u, err, tmo);
+  }
+}
+
 // ------------------------------------------------------------- the kernel
 template <int NR, int CW, bool BF16>
 __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
@@ -310,100 +433,11 @@ __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
 
   if (w == kWorkThreads / 32) {
     // ------------------------------------------------------------ producer
-    // Pass after pass: the chunks of the CTA's units in order, dealt to the
-    // groups in turn (a unit is padded to whole rounds with empty chunks, so
-    // every group sees every unit), then a round of end marks.  The lanes
-    // take a block of up to S chunks, one each: a lane waits until its stage's
-    // last chunk has been read, puts c_{k+1} of the chunk's columns and the
-    // column index beside it, and issues the copy.
-    const int BL = S < 32 ? S : 32;
-    unsigned base = 0;                        // chunks issued before this block
-    bool ok = true;
-    auto put = [&](bool mine, int64_t j, int n, int u, const float* c, int count) {   // count: lanes of the block
-      const unsigned q = base + (unsigned)lane;
-      const unsigned st = q % (unsigned)S, round = q / (unsigned)S;
-      bool todo = mine;
-      uint64_t t0 = 0;
-      for (unsigned i = 1; __any_sync(0xffffffffu, todo); ++i) {
-        if (todo && (round == 0 || mbar_try_wait(empty + st, (round - 1) & 1u))) {
-          todo = false;
-#pragma unroll
-          for (int e = 0; e < CW; ++e) cxs[st * kMaxCw + e] = c[e];
-          meta[st].j = j;
-          meta[st].n = n;
-          meta[st].u = u;
-          if (n > 0) {
-            mbar_arrive_expect_tx(full + st, (uint32_t)n * colbytes);
-            bulk_load(ring + (size_t)st * stagebytes,
-                      reinterpret_cast<const unsigned char*>(a.R) + (size_t)j * colbytes, (uint32_t)n * colbytes,
-                      full + st);
-          } else {
-            mbar_arrive(full + st);
-          }
-        }
-        if ((i & 63u) == 0) {                 // bounded
-          const uint64_t tn = globaltimer_ns();
-          if (t0 == 0) t0 = tn;
-          if (*quit) ok = false;
-          if (tn - t0 > tmo || i > (1u << 28)) {
-            if (todo) atomicCAS(err, 0, kDevErrTimeout);
-            ok = false;
-          }
-          ok = __all_sync(0xffffffffu, ok);
-          if (!ok) break;
-        }
-      }
-      if (ok) {
-        base += (unsigned)count;
-      } else {
-        // this block's copies that were issued land before the CTA exits (bounded)
-        if (mine && !todo) mbar_wait_bounded(full + st, round & 1u, err, tmo);
-        __syncwarp();
-      }
-    };
-    for (int k = a.npart_first > 0 ? 0 : -1; k < K && ok; ++k) {
-      const float* cn = k + 1 < K ? a.C + (int64_t)(k + 1) * N : nullptr;
-      auto grab = [&]() -> unsigned { return lane == 0 ? atomicAdd(a.work + k + 1, 1u) : 0u; };   // lane 0 has it
-      // the first unit is the CTA's own (a CTA that runs ahead into this pass must
-      // not take two large ones); the others come from the counter, asked for
-      // a block before they are needed
-      int64_t u = cta;
-      while (u < a.nunits && ok) {
-        unsigned unext = 0u;
-        int64_t lo, hi;
-        unit_range(a.units, N, u, lo, hi);
-        const int64_t chunks = (hi - lo + CW - 1) / CW;
-        const int64_t total = (chunks > 0 ? (chunks + NG - 1) / NG : 1) * NG;
-        float c[CW];
-        auto load_c = [&](int64_t i) {        // c_{k+1} on chunk i of the unit
-          const int64_t j = lo + i * CW;
-#pragma unroll
-          for (int e = 0; e < CW; ++e) c[e] = cn && i < total && j + e < hi ? __ldcg(cn + j + e) : 0.f;
-        };
-        load_c(lane);
-        for (int64_t i0 = 0; i0 < total && ok; i0 += BL) {
-          const int count = (int)(total - i0 < BL ? total - i0 : BL);
-          if (a.dynamic && i0 + BL >= total) unext = grab();
-          const int64_t j = lo + (i0 + lane) * CW;
-          const int n = j < hi ? (int)(hi - j < CW ? hi - j : CW) : 0;
-          put(lane < count, j, n, (int)u, c, count);
-          if (i0 + BL < total) load_c(i0 + BL + lane);
-        }
-        u = a.dynamic ? (int64_t)G + (int64_t)__shfl_sync(0xffffffffu, unext, 0) : (int64_t)a.nunits;
-      }
-      for (int i0 = 0; i0 < NG && ok; i0 += BL) {
-        float c[CW];
-#pragma unroll
-        for (int e = 0; e < CW; ++e) c[e] = 0.f;
-        const int count = NG - i0 < BL ? NG - i0 : BL;
-        put(lane < count, 0, -1, 0, c, count);
-      }
-    }
-    // earlier copies still in flight land before the CTA exits (bounded)
-    if (!ok && lane == 0) {
-      for (unsigned d = base > (unsigned)S ? base - (unsigned)S : 0u; d < base; ++d)
-        mbar_wait_bounded(full + d % (unsigned)S, (d / (unsigned)S) & 1u, err, tmo);
-    }
+    // (pass k takes c_{k+1} along)
+    Stream p{a.R, N, colbytes, ring, meta, cxs, kMaxCw, full, empty, S, NG, G, cta, a.units, a.nunits, a.dynamic,
+             a.work + (a.npart_first > 0 ? 1 : 0), quit, err, tmo};
+    produce<CW, 1>(p, a.npart_first > 0 ? 0 : -1, K,
+                   [&](int k, int) -> const float* { return k + 1 < K ? a.C + (int64_t)(k + 1) * N : nullptr; });
     return;
   }
 

@@ -381,9 +381,35 @@ bool plan_defer(int ld, int64_t N, int K, bool bf16, int grid_override, DeferPla
 size_t defer_pair_bytes(int K, int grid);
 cudaError_t launch_defer(const DeferPlan& plan, const DeferBuffers& b, int ld, int64_t N, int K, int npart_first,
                          int bar_extra, uint64_t timeout_ns, uint64_t* tstamp, int tstamp_cap, cudaStream_t s);
-// f_prev: objective before the sweep (trace[-1] instead when s > 0).
-cudaError_t launch_defer_close(const double* part, int n, int stride, const DeferBuffers& b, int K, double* trace,
+// f_prev: objective before the sweep (trace[-1] instead unless first); work:
+// nwork unit counters, zeroed.
+cudaError_t launch_defer_close(const double* part, int n, int stride, Ctrl* ctrl, unsigned* work, int nwork, double* trace,
                                int stop_rule, double tol, double f_prev, double f0, bool first, cudaStream_t s);
+
+// The same for the C-first order (did_cfirst_kernel.cuh): a pass over R serves
+// KB of the K dots (C step) or partials (B step).
+struct CfirstPlan {
+  int grid, GS, NG, CW, S, KB;
+  Units units;
+  int nunits, dynamic, npart;
+  size_t csmem, bsmem;
+  const void *cfunc, *bfunc;
+};
+struct CfirstSizes {
+  size_t Co, T, P, Gp, Xp;    // bytes of the buffers below
+};
+struct CfirstBuffers {
+  const void* R;
+  float *B, *C, *Co, *T, *P;
+  void *Gp, *Xp;
+  unsigned* work;     // [2 K], zero before the first launch
+  Ctrl* ctrl;
+  unsigned long long* degen;
+};
+bool plan_cfirst(int ld, int64_t N, int K, bool bf16, CfirstPlan* plan);   // false: shape not supported
+CfirstSizes cfirst_sizes(const CfirstPlan& p, int ld, int64_t N, int K);
+cudaError_t launch_cfirst(const CfirstPlan& plan, const CfirstBuffers& b, int ld, int64_t N, int K, int bar_extra,
+                          uint64_t timeout_ns, cudaStream_t s);
 
 // Multi-instance sweeps (serving): one cooperative launch runs several
 // instances, each on its own range of CTAs (SweepArgs::cta_begin/cta_count).

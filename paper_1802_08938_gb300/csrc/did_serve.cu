@@ -560,8 +560,8 @@ bool run_round(did_server* s, std::vector<Req*>& act) {
                                              d.part, d.b.P, d.b.CC0, &d.b.ctrl->err, kServeTimeoutNs, st, !s->bf16)
                     : did::launch_dense(da, st);
       if (e == cudaSuccess)
-        e = did::launch_defer_close(d.tc_ws ? d.part : s->d_part, d.tc_ws ? G : s->dense_grid, d.tc_ws ? 1 : 3, d.b,
-                                    r->rq.K, tr + q, r->rq.tol > 0.0 ? 1 : 0, r->rq.tol, r->trace.back(),
+        e = did::launch_defer_close(d.tc_ws ? d.part : s->d_part, d.tc_ws ? G : s->dense_grid, d.tc_ws ? 1 : 3,
+                                    d.b.ctrl, d.b.work, r->rq.K + 1, tr + q, r->rq.tol > 0.0 ? 1 : 0, r->rq.tol, r->trace.back(),
                                     r->trace.front(), q == 0, st);
     }
   }

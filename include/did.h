@@ -318,9 +318,9 @@ did_status did_generate_uniform(float* out_dev, int64_t n, uint64_t seed, int32_
  * (|f_{t-1} - f_t| / f_{t-1} < tol, or max_iter sweeps).  Requests whose
  * residual fits the SMs' shared memory are packed into cooperative launches, each
  * on its own range of CTAs; larger ones take the whole GPU in turn (as many of
- * their sweeps a round as fit in about 20 ms, at least one); the rest share one
- * launch of the multi-instance sweep kernel, with CTAs in proportion to
- * measured CTA-seconds per sweep.  The scratch of these forms (the pending
+ * their sweeps a round as fit in about 20 ms, at least one); the rest, and
+ * several mid-sized ones where that is faster, share one launch of the
+ * multi-instance sweep kernel, with CTAs in proportion to measured CTA-seconds per sweep.  The scratch of these forms (the pending
  * factors and the refresh's operands of the largest request) is the server's, outside the
  * budget; where it cannot be had every request takes the last form.
  * Between rounds, finished requests are retired (B, C copied to host memory

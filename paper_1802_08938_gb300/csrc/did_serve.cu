@@ -10,8 +10,9 @@
 //             whatever the number of CTAs is;
 //   DEFER     larger: read-only sweeps on the whole GPU, one request after another,
 //             each pass at HBM speed, which a share of the SMs does not reach;
-//   PACKED    otherwise (K too large for a short column): the multi-instance sweep kernel, each
-//             request on its own CTA range, proportional to its per-sweep work.
+//   PACKED    otherwise (K too large for a short column, or several mid-sized requests at
+//             once, pack_mid_sized): the multi-instance sweep kernel, each request on its own
+//             CTA range, proportional to its per-sweep work.
 // All three stop a request on the device by its own rule.  With every
 // request in the multi-instance kernel 24 requests of 20 sweeps took 488 ms;
 // see run_round for what they take now.  Between rounds finished requests are retired and new ones
@@ -44,6 +45,13 @@ constexpr uint64_t kServeTimeoutNs = 4000000000ull;
 constexpr double kPassFixedS = 12e-6;
 constexpr double kCtaBytesPerS = 40e9;
 constexpr double kRoundMinS = 5e-3;      // a launch of the multi-instance kernel lasts at least this long
+// Costs of a k of a larger request: read-only sweeps alone on the GPU, and the
+// multi-instance kernel (the fixed part once, then the read and the write of each request).
+constexpr double kDeferFixedS = 20e-6;
+constexpr double kDeferBytesPerS = 6.5e12;
+constexpr double kPackFixedS = 30e-6;
+constexpr double kPackBytesPerS32 = 5.0e12;
+constexpr double kPackBytesPerS16 = 4.0e12;
 constexpr double kDeferSliceS = 20e-3;   // a larger request's sweeps in one round take at most about this long
 // Phase stamps kept per instance (4 per k of its first sweep in a round):
 // the measured time of that sweep drives the next round's CTA shares.
@@ -482,14 +490,52 @@ std::vector<Bin> pack(const did_server* s, const std::vector<Req*>& act, std::ve
   return bins;
 }
 
+// DEFER requests of this round that take less of the GPU's time in the
+// multi-instance kernel: alone each pays about kDeferFixedS a k, whatever its
+// size is, and its refresh; together they pay one kPackFixedS a k, then the read
+// and the write of their residuals.  The smallest go first, as many as make the
+// sum shortest.  A request may change its form between rounds: R is current
+// after each.  Measured on 128 requests (64..4096 rows, 256..65536 columns, K 8
+// to 64, 64 at once, 300 sweeps each): float32 7.85 solves/s with all of
+// them alone, 9.08 so (8.2 with the rates of the model 0.6 and 1.6 times these);
+// bfloat16 9.1 and 11.8 (11.4, 11.7); in the multi-instance kernel 6.9 and 9.8.
+void pack_mid_sized(const did_server* s, const std::vector<Req*>& act, std::vector<int>* def, std::vector<int>* packed) {
+  auto bytes = [&](int i) { return (double)act[i]->ld * (double)act[i]->rq.N * (s->bf16 ? 2.0 : 4.0); };
+  auto alone = [&](int i) {
+    return act[i]->rq.K * (kDeferFixedS + bytes(i) / kDeferBytesPerS) + (s->bf16 ? 3.0 : 2.0) * bytes(i) / kDeferBytesPerS;
+  };
+  const double rate = s->bf16 ? kPackBytesPerS16 : kPackBytesPerS32;
+  double fixed = 0.0, moved = 0.0, rest = 0.0;
+  auto add = [&](int i) {
+    fixed = std::max(fixed, act[i]->rq.K * kPackFixedS);
+    moved += act[i]->rq.K * 2.0 * bytes(i) / rate;
+  };
+  std::sort(def->begin(), def->end(), [&](int a, int b) { return bytes(a) != bytes(b) ? bytes(a) < bytes(b) : a < b; });
+  for (int i : *packed) add(i);
+  for (int i : *def) rest += alone(i);
+  size_t take = 0;
+  double best = fixed + moved + rest;
+  for (size_t q = 0; q < def->size() && packed->size() + q < (size_t)s->grid; ++q) {
+    add((*def)[q]);
+    rest -= alone((*def)[q]);
+    if (fixed + moved + rest < best) {
+      best = fixed + moved + rest;
+      take = q + 1;
+    }
+  }
+  packed->insert(packed->end(), def->begin(), def->begin() + take);
+  def->erase(def->begin(), def->begin() + take);
+}
+
 // One round over the active requests; returns false on a CUDA error.
 // Measured: 24 requests (64..4096 rows, 256..65536 columns, K 8 to 64, float32)
 // of 20 sweeps each: 488 ms with every request in the multi-instance kernel,
-// 310 ms with the three forms.
+// 306 ms with the three forms.
 bool run_round(did_server* s, std::vector<Req*>& act) {
   const int n = (int)act.size();
   std::vector<int> res, def, packed;
   for (int i = 0; i < n; ++i) (act[i]->form == RESIDENT ? res : act[i]->form == DEFER ? def : packed).push_back(i);
+  pack_mid_sized(s, act, &def, &packed);
   std::vector<Bin> bins = pack(s, act, res);
   size_t scratch = 0;
   for (const Bin& b : bins) scratch = std::max(scratch, b.words);

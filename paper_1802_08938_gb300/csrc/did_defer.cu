@@ -3,10 +3,10 @@
 //
 // Measured on one GB300, a sweep with the refresh that ends it, against the
 // sweep kernel that writes R (a plain read of 4 GB runs at 7.2 TB/s):
-//   5000 x 200000, K = 50, float32       48.0 -> 30.7 ms (599 us a k: pass 545, 7.3 TB/s)
+//   5000 x 200000, K = 50, float32       48.0 -> 30.6 ms (585 us a k: pass 545, 7.3 TB/s)
 //   10000 x 100000, K = 100, bfloat16    75.1 -> 37.1 ms (365 us a k: pass 313, 6.4 TB/s)
-//   784 x 70000, K = 16, float32         1.52 -> 1.01 ms (58 us a k: pass 35)
-//   784 x 70000, K = 16, bfloat16        1.13 -> 0.77 ms (44 us a k: pass 23)
+//   784 x 70000, K = 16, float32         1.52 -> 0.90 ms (49 us a k: pass 31)
+//   784 x 70000, K = 16, bfloat16        1.13 -> 0.70 ms (39 us a k: pass 20)
 #include "did_defer_kernel.cuh"
 
 #include <algorithm>
@@ -17,17 +17,24 @@ using namespace defer_impl;
 
 namespace {
 
-// Closes a sweep: f = 1/2 ||R||^2 from the refresh's per-CTA sums (added in
-// order), the stopping rule, and the barrier and the unit counters cleared
+// Closes a sweep: f = 1/2 ||R||^2 from the refresh's per-CTA sums (a tree of
+// fixed shape), the stopping rule, and the barrier and the unit counters cleared
 // for the next launch.  Nothing after a sweep that stopped or failed.
+constexpr int kCloseThreads = 128;
 __global__ void defer_close_kernel(const double* part, int n, int stride, Ctrl* ctrl, unsigned* work, int nwork, double* trace,
                                    int stop_rule, double tol, double f_prev, double f0, int first) {
+  __shared__ double sum[kCloseThreads];
   if (ctrl->stopped || ctrl->err) return;
   for (int i = threadIdx.x; i < nwork; i += blockDim.x) work[i] = 0u;
+  double s = 0.0;
+  for (int i = threadIdx.x; i < n; i += kCloseThreads) s += part[(size_t)i * stride];
+  sum[threadIdx.x] = s;
+  for (int h = kCloseThreads / 2; h > 0; h >>= 1) {
+    __syncthreads();
+    if ((int)threadIdx.x < h) sum[threadIdx.x] += sum[threadIdx.x + h];
+  }
   if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int i = 0; i < n; ++i) s += part[(size_t)i * stride];
-    const double f = 0.5 * s, prev = first ? f_prev : trace[-1];
+    const double f = 0.5 * sum[0], prev = first ? f_prev : trace[-1];
     *trace = f;
     ctrl->bar = 0u;
     ctrl->sweeps += 1;
@@ -152,7 +159,7 @@ cudaError_t launch_defer(const DeferPlan& plan, const DeferBuffers& b, int ld, i
 
 cudaError_t launch_defer_close(const double* part, int n, int stride, Ctrl* ctrl, unsigned* work, int nwork, double* trace,
                                int stop_rule, double tol, double f_prev, double f0, bool first, cudaStream_t s) {
-  defer_close_kernel<<<1, 128, 0, s>>>(part, n, stride, ctrl, work, nwork, trace, stop_rule, tol, f_prev, f0,
+  defer_close_kernel<<<1, kCloseThreads, 0, s>>>(part, n, stride, ctrl, work, nwork, trace, stop_rule, tol, f_prev, f0,
                                        first ? 1 : 0);
   return cudaGetLastError();
 }

@@ -52,7 +52,8 @@ CPU_SAMPLE_COLS = {"planted_exp_5000x200000_k50": 1000, "image_like_784x70000_k1
 CPU_SAMPLE_SWEEPS = 3
 
 SWEEP_SOURCES = ["paper_1802_08938_gb300/csrc/did_sweep.cu", "paper_1802_08938_gb300/csrc/did_sweep_kernel.cuh",
-                 "paper_1802_08938_gb300/csrc/did_internal.cuh"]
+                 "paper_1802_08938_gb300/csrc/did_internal.cuh", "paper_1802_08938_gb300/csrc/did_defer.cu",
+                 "paper_1802_08938_gb300/csrc/did_defer_kernel.cuh", "paper_1802_08938_gb300/csrc/did_refresh_tc.cu"]
 
 
 def sweep_source_hash():
@@ -257,8 +258,8 @@ def workload_run(did, name, precision, sweeps, warmup, stream, tol=0.0, max_swee
     i1 = c.info()
     ms = e0.elapsed_time(e1)
     kms = i1["sweep_kernel_ms"] - i0["sweep_kernel_ms"]
-    passes = sweep_passes(K, i1["lazy_writeback"])
-    alg = done * float(passes) * M * N * s_bytes + (i1["prologue_launches"] - i0["prologue_launches"]) * M * N * s_bytes
+    per_sweep, form = sweep_bytes(M, N, K, s_bytes)
+    alg = done * per_sweep
     peak, _ = measured_peaks()
     f = c.objective()
     trace = c.trace()
@@ -266,7 +267,7 @@ def workload_run(did, name, precision, sweeps, warmup, stream, tol=0.0, max_swee
     return {"workload": name, "precision": precision, "sweeps": int(done), "warmup": warmup,
             "value": done / (ms / 1000.0), "unit": "sweeps/s", "ms_per_sweep": ms / max(1, done),
             "roofline_frac": alg / (kms / 1e3) / 1e9 / peak if kms > 0 else None,
-            "alg_bytes_per_sweep": float(passes) * M * N * s_bytes, "writeback": "deferred" if i1["lazy_writeback"] else "eager",
+            "alg_bytes_per_sweep": per_sweep, "writeback": form,
             "refreshes": int(i1["refreshes"] - i0["refreshes"]),
             "refresh_kind": ("tcgen05" if i1["tc_refreshes"] > i0["tc_refreshes"] else "SIMT") if i1["refreshes"] > i0["refreshes"] else None,
             "objective_fBC": f, "trace_last": float(trace[-1]),
@@ -321,7 +322,7 @@ def order_bench(did, X, M, N, K, w, seed, stream, order, steps, warmup, flags=0,
     f = c.objective()
     trace = c.trace()
     c.close()
-    out = {"order": order, "writeback": "eager" if flags & did.DID_FLAG_EAGER_WRITEBACK else "deferred",
+    out = {"order": order, "writeback": "eager" if flags & did.DID_FLAG_EAGER_WRITEBACK else "default",
            "inner": list(inner), "trace": [float(v) for v in trace],
            "value": steps / (ms / 1000.0), "unit": "sweeps/s", "ms_per_sweep": ms / steps,
            "objective_after": f, "sweeps": warmup + steps,
@@ -361,6 +362,34 @@ def sweep_passes(K, lazy):
     """Passes over R per sweep of the interleaved kernel: a read and a write per
     k, less one write for each deferred k (pairs (k, k+1) share a write)."""
     return 2 * K - (K // 2 if lazy else 0)
+
+
+def c_first_block(M, s_bytes):
+    """k served by one pass of the C-first order's read-only sweep."""
+    vr = 16 // s_bytes
+    ld = (M + 15) // 16 * 16
+    gs = 32
+    while gs < 512 and gs * 16 < ld:
+        gs *= 2
+    rows = vr * max(1, -(-(ld // vr) // gs))
+    return 4 if rows <= 16 else 2 if rows <= 32 else 1
+
+
+def sweep_bytes(M, N, K, s_bytes, order="interleaved", eager=False, lazy=1):
+    """(bytes a sweep moves, how) of the per-k orders.  By default sweeps only
+    read R -- K times, or 2 K / (k a pass serves) times in the C-first order --
+    and form it anew from X at their end (read X, write R; a float32 residual
+    with K > 64 takes one more pass for the first partials).  With one write per
+    k: sweep_passes, or 4 K in the C-first order.  A residual that fits the SMs'
+    shared memory is read and written once a call."""
+    mn = float(M) * N
+    if eager:
+        return (sweep_passes(K, 0) if order == "interleaved" else 4 * K) * mn * s_bytes, "eager"
+    if mn * 4 <= 30e6:
+        return 2 * mn * s_bytes, "resident"
+    if order == "interleaved":
+        return (K + (1 if s_bytes == 4 and K > 64 else 0)) * mn * s_bytes + mn * (4 + s_bytes), "read-only"
+    return 2 * -(-K // c_first_block(M, s_bytes)) * mn * s_bytes + mn * (4 + s_bytes), "read-only"
 
 
 def max_over_ranks(x, ws):
@@ -542,8 +571,9 @@ def main():
     launches = info1["sweep_launches"] - info0["sweep_launches"]
     prologues = info1["prologue_launches"] - info0["prologue_launches"]
     kms = info1["sweep_kernel_ms"] - info0["sweep_kernel_ms"]
-    passes = sweep_passes(K, info1["lazy_writeback"]) if args.order == "interleaved" else 2 * K
-    alg_bytes = args.steps * float(passes) * M * N * s_bytes + prologues * 1.0 * M * N * s_bytes
+    eager = bool(flags & did.DID_FLAG_EAGER_WRITEBACK)
+    per_sweep, form = sweep_bytes(M, N, K, s_bytes, args.order, eager)
+    alg_bytes = args.steps * per_sweep + (prologues * 1.0 * M * N * s_bytes if eager else 0.0)
     achieved = alg_bytes / (kms / 1000.0) / 1e9
     peak, peak_kind = measured_peaks()
     traffic = profiled_traffic(args.workload, args.precision)
@@ -555,7 +585,11 @@ def main():
     refresh = None
     nref = dense_launches + tc_launches
     if nref:
-        rms = (info1["dense_kernel_ms"] - info0["dense_kernel_ms"] + info1["tc_refresh_ms"] - info0["tc_refresh_ms"]) / nref
+        # on its own after the timed region: those that end read-only sweeps are part of their time
+        for _ in range(3):
+            ctx.refresh_residual()
+        i2 = ctx.info()
+        rms = (i2["dense_kernel_ms"] - info1["dense_kernel_ms"] + i2["tc_refresh_ms"] - info1["tc_refresh_ms"]) / 3
         rbytes = M * N * (4 + s_bytes)
         kind = ("tcgen05 BF16x3" if prec == did.DID_BF16R else "tcgen05 BF16x6") if tc_launches else "SIMT FP32"
         refresh = {"kind": kind, "launches": int(nref),
@@ -582,8 +616,7 @@ def main():
         i1 = c16.info()
         ms16 = e0.elapsed_time(e1)
         kms16 = i1["sweep_kernel_ms"] - i0["sweep_kernel_ms"]
-        ab16 = (args.steps * float(sweep_passes(K, i1["lazy_writeback"])) * M * N * 2
-                + (i1["prologue_launches"] - i0["prologue_launches"]) * M * N * 2.0)
+        ab16 = args.steps * sweep_bytes(M, N, K, 2)[0]
         f16 = c16.objective()
         c16.close()
         v16 = ws * args.steps / (ms16 / 1000.0)
@@ -676,15 +709,14 @@ def main():
     else:
         roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                     "frac": achieved / peak, "traffic": traffic if args.order == "interleaved" else None,
-                    "kernel": "sweep_kernel", "peak_kind": peak_kind,
-                    "alg_bytes_per_sweep": float(passes) * M * N * s_bytes,
-                    # the survey's per-sweep figure, one read and one write of R per k; the
-                    # deferred write-back moves fewer bytes, and frac above uses the bytes it moves
+                    "kernel": "sweep_kernel" if form == "eager" else "%s sweep and refresh" % form, "peak_kind": peak_kind,
+                    "alg_bytes_per_sweep": per_sweep,
+                    # one read and one write of R per k; the sweep moves fewer bytes, and frac above uses those
                     "alg_bytes_per_sweep_2KMNs": 2.0 * K * M * N * s_bytes,
                     "frac_on_2KMNs": (2.0 * K * M * N * s_bytes * args.steps / (kms / 1000.0) / 1e9) / peak,
-                    "bytes_note": ("frac counts the %d passes of R a sweep moves (%s write-back); on 2K = %d "
+                    "bytes_note": ("frac counts the bytes a sweep moves (%s form, %.4g passes of R); on 2K = %d "
                                    "passes the same kernel time gives frac_on_2KMNs"
-                                   % (passes, "deferred" if info1["lazy_writeback"] else "eager", 2 * K)),
+                                   % (form, per_sweep / (float(M) * N * s_bytes), 2 * K)),
                     "lazy_writeback": int(info1["lazy_writeback"]), "ring_stages": int(info1["ring_stages"]),
                     "kernel_ms_per_sweep": kms / max(1, args.steps)}
 
@@ -692,7 +724,8 @@ def main():
         eager32 = [o for o in orders if o["order"] == "interleaved" and o["writeback"] == "eager"]
         if eager32:
             bf16["ratio_vs_fp32_eager"] = bf16["value"] / eager32[0]["value"]
-        bf16["writeback"] = "deferred" if bf16.pop("lazy", 0) else "eager"
+        bf16.pop("lazy", 0)
+        bf16["writeback"] = sweep_bytes(M, N, K, 2)[1]
 
     if rank == 0:
         line = {

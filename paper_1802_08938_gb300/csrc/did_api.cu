@@ -597,10 +597,36 @@ did_status did_create(const float* X, int64_t M, int64_t N, int32_t K, uint64_t 
 // Whether read-only sweeps pay: the pending terms (2 K values a column) are
 // small beside a column, and a pass is longer than the phases around it (about 20 us
 // a k, where the sweep kernel takes 27 to 32 us for small passes: 1024 x 2414 in
-// bfloat16, 5 MB, measured 29.6 against 29.2 us a k; 784 x 70000, 110 MB, 44
+// bfloat16, 5 MB, measured 29.6 against 29.2 us a k; 784 x 70000, 110 MB, 39
 // against 70).
 static bool defer_pays(const did_ctx* c) {
   return c->ld >= 4 * c->K && (size_t)c->ld * c->N * (c->bf16 ? 2 : 4) >= ((size_t)16 << 20);
+}
+
+// Scratch of the read-only sweeps.
+static did_status form_scratch(did_ctx* c) {
+  const int64_t N = c->N;
+  const int K = c->K;
+  auto take = [&](auto& field, size_t bytes) {
+    void* p;
+    const did_status st = dev_alloc(c, &p, bytes);
+    field = reinterpret_cast<std::decay_t<decltype(field)>>(p);
+    return st == DID_OK;
+  };
+  bool ok;
+  if (c->defer) {
+    const size_t W = (size_t)c->dplan.GS / 32;
+    ok = take(c->dbuf.Bo, (size_t)c->ld * K * sizeof(float)) && take(c->dbuf.Co, (size_t)K * N * sizeof(float)) &&
+         take(c->dbuf.T, (size_t)N * W * sizeof(float)) && take(c->dbuf.corr, (size_t)N * 2 * sizeof(float)) &&
+         take(c->dbuf.Xp, did::defer_pair_bytes(K, c->dplan.grid)) &&
+         take(c->dbuf.Yp, did::defer_pair_bytes(K, c->dplan.grid)) &&
+         take(c->dbuf.work, (size_t)(K + 1) * sizeof(unsigned));
+  } else {
+    const did::CfirstSizes z = did::cfirst_sizes(c->cplan, c->ld, N, K);
+    ok = take(c->cbuf.Co, z.Co) && take(c->cbuf.T, z.T) && take(c->cbuf.P, z.P) && take(c->cbuf.Gp, z.Gp) &&
+         take(c->cbuf.Xp, z.Xp) && take(c->cbuf.work, (size_t)2 * K * sizeof(unsigned));
+  }
+  return ok ? DID_OK : DID_ENOMEM;
 }
 
 static did_status create_impl(did_ctx* c, const float* X, uint64_t seed) {
@@ -642,34 +668,14 @@ static did_status create_impl(did_ctx* c, const float* X, uint64_t seed) {
   ALLOC(Y, (size_t)c->ld * 2 * K * sizeof(float));
   ALLOC(C, (size_t)K * N * sizeof(float));
   // partial rows: the plan's, and the tensor-core refresh's two per CTA
-  const size_t U = (size_t)std::max(std::max(c->defer ? c->dplan.npart : c->plan.npart, G), 2 * did::refresh_tc_grid());
+  const size_t U = (size_t)std::max(std::max(std::max(c->defer ? c->dplan.npart : 0, c->plan.npart), G),
+                                    2 * did::refresh_tc_grid());
   ALLOC(P, U * c->ld * sizeof(float));
   ALLOC(CCp, U * sizeof(double));
   ALLOC(Sp, (size_t)2 * G * sizeof(double));
   ALLOC(OBJp, U * sizeof(double));
   ALLOC(bold, (size_t)c->ld * sizeof(float));
   if (c->resident) ALLOC(res_words, c->rplan.words_bytes);
-  if (c->defer) {
-    const size_t W = (size_t)c->dplan.GS / 32;
-    ALLOC(dbuf.Bo, (size_t)c->ld * K * sizeof(float));
-    ALLOC(dbuf.Co, (size_t)K * N * sizeof(float));
-    ALLOC(dbuf.T, (size_t)N * W * sizeof(float));
-    ALLOC(dbuf.corr, (size_t)N * 2 * sizeof(float));
-    ALLOC(dbuf.Xp, did::defer_pair_bytes(K, c->dplan.grid));
-    ALLOC(dbuf.Yp, did::defer_pair_bytes(K, c->dplan.grid));
-    ALLOC(dbuf.work, (size_t)(K + 1) * sizeof(unsigned));
-  } else if (c->cfirst) {
-    const did::CfirstSizes z = did::cfirst_sizes(c->cplan, c->ld, N, K);
-    ALLOC(cbuf.Co, z.Co);
-    ALLOC(cbuf.T, z.T);
-    ALLOC(cbuf.P, z.P);
-    ALLOC(cbuf.Gp, z.Gp);
-    ALLOC(cbuf.Xp, z.Xp);
-    ALLOC(cbuf.work, (size_t)2 * K * sizeof(unsigned));
-  } else if (c->plan.lazy && !c->resident) {
-    ALLOC(Cold, (size_t)N * sizeof(float));
-    ALLOC(XCp, 2 * U * sizeof(double));
-  }
   ALLOC(ctrl, sizeof(Ctrl));
   ALLOC(trace_dev, sizeof(double) * kMaxSweepsPerLaunch);
   ALLOC(degen, sizeof(unsigned long long));
@@ -690,6 +696,20 @@ static did_status create_impl(did_ctx* c, const float* X, uint64_t seed) {
     if (wsb == 0) return fail(c, DID_EINVAL, "the batched order supports K <= 64");
     st = dev_alloc(c, &bws, wsb);
     if (st != DID_OK) return st;
+  }
+  // Last: a form of sweep whose scratch does not fit beside the rest gives way to the kernel that writes R.
+  if (c->defer || c->cfirst) {
+    const size_t mark = c->dev_allocs.size(), bytes = c->device_bytes;
+    if (form_scratch(c) != DID_OK) {
+      for (; c->dev_allocs.size() > mark; c->dev_allocs.pop_back()) cudaFree(c->dev_allocs.back());
+      c->device_bytes = bytes;
+      c->last_error.clear();
+      c->defer = c->cfirst = false;
+    }
+  }
+  if (c->plan.lazy && !c->resident && !c->defer && !c->cfirst) {
+    ALLOC(Cold, (size_t)N * sizeof(float));
+    ALLOC(XCp, 2 * U * sizeof(double));
   }
 #undef ALLOC
   c->B = c->Y + (size_t)K * c->ld;

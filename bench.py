@@ -271,8 +271,9 @@ def workload_run(did, name, precision, sweeps, warmup, stream, tol=0.0, max_swee
             "refreshes": int(i1["refreshes"] - i0["refreshes"]),
             "refresh_kind": ("tcgen05" if i1["tc_refreshes"] > i0["tc_refreshes"] else "SIMT") if i1["refreshes"] > i0["refreshes"] else None,
             "objective_fBC": f, "trace_last": float(trace[-1]),
-            "gpu_launches": int((i1["sweep_launches"] - i0["sweep_launches"]) + (i1["dense_launches"] - i0["dense_launches"])
-                                + 3 * (i1["tc_refreshes"] - i0["tc_refreshes"]))}
+            "gpu_launches": sweep_launches(form, K, s_bytes, "interleaved", done, i1["sweep_launches"] - i0["sweep_launches"],
+                                           i1["tc_refreshes"] - i0["tc_refreshes"],
+                                           i1["dense_launches"] - i0["dense_launches"])}
 
 
 def precision_pair(did, name, sweeps, warmup, stream, tol=0.0, max_sweeps=None):
@@ -390,6 +391,16 @@ def sweep_bytes(M, N, K, s_bytes, order="interleaved", eager=False, lazy=1):
     if order == "interleaved":
         return (K + (1 if s_bytes == 4 and K > 64 else 0)) * mn * s_bytes + mn * (4 + s_bytes), "read-only"
     return 2 * -(-K // c_first_block(M, s_bytes)) * mn * s_bytes + mn * (4 + s_bytes), "read-only"
+
+
+def sweep_launches(form, K, s_bytes, order, sweeps, launches, tc, dense):
+    """Kernel launches of `sweeps` sweeps, from the counters.  A read-only sweep is
+    its kernel (two in the C-first order), the refresh (two operand splits and
+    the GEMM, or the float32 pass) and a closing kernel, and the counted
+    refreshes are those; else each tensor-core refresh is three launches."""
+    if form == "read-only":
+        return int(sweeps * ((1 if order == "interleaved" else 2) + (1 if s_bytes == 4 and K > 64 else 3) + 1))
+    return int(launches + dense + 3 * tc)
 
 
 def max_over_ranks(x, ws):
@@ -572,15 +583,16 @@ def main():
     prologues = info1["prologue_launches"] - info0["prologue_launches"]
     kms = info1["sweep_kernel_ms"] - info0["sweep_kernel_ms"]
     eager = bool(flags & did.DID_FLAG_EAGER_WRITEBACK)
-    per_sweep, form = sweep_bytes(M, N, K, s_bytes, args.order, eager)
+    per_sweep, form = ((3.0 * M * N * s_bytes, "batched") if args.order == "did_batched" else
+                       sweep_bytes(M, N, K, s_bytes, args.order, eager))
     alg_bytes = args.steps * per_sweep + (prologues * 1.0 * M * N * s_bytes if eager else 0.0)
     achieved = alg_bytes / (kms / 1000.0) / 1e9
     peak, peak_kind = measured_peaks()
     traffic = profiled_traffic(args.workload, args.precision)
     dense_launches = info1["dense_launches"] - info0["dense_launches"]
     tc_launches = info1["tc_refreshes"] - info0["tc_refreshes"]
-    # each tensor-core refresh is three launches: two operand splits and the GEMM
-    gpu_launches = launches + dense_launches + 3 * tc_launches   # the timed region of the line
+    gpu_launches = sweep_launches(form, K, s_bytes, args.order, args.steps,
+                                  launches, tc_launches, dense_launches)   # the timed region of the line
     other_launches = 0                                            # the other measurements' timed regions
     refresh = None
     nref = dense_launches + tc_launches
@@ -625,7 +637,8 @@ def main():
                 "tc_refreshes": int(i1["tc_refreshes"] - i0["tc_refreshes"]),
                 "objective_after": f16,
                 "note": "same workload and seed, R stored in bfloat16, tensor-core BF16x3 refresh"}
-        other_launches += args.steps + 3 * int(i1["tc_refreshes"] - i0["tc_refreshes"])
+        other_launches += sweep_launches(sweep_bytes(M, N, K, 2)[1], K, 2, "interleaved", args.steps, args.steps,
+                                         i1["tc_refreshes"] - i0["tc_refreshes"], 0)
 
     orders = None
     if not args.no_orders and prec == did.DID_FP32 and args.order == "interleaved":

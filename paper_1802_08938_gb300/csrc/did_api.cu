@@ -886,18 +886,26 @@ did_status did_set_factors(did_ctx* c, const float* B, const float* C) {
 did_status did_get_residual(did_ctx* c, float* R) {
   if (!c || !R) return DID_EINVAL;
   if (c->batched) DID_CUDA(c, did::batched_materialize(c->batched, (float*)c->R, c->Y, c->C, c->ld, c->N, c->K, c->stream));
-  if (!c->bf16) {
-    DID_CUDA(c, cudaMemcpy2DAsync(R, (size_t)c->M * sizeof(float), c->R, (size_t)c->ld * sizeof(float),
-                                  (size_t)c->M * sizeof(float), (size_t)c->N, cudaMemcpyDefault, c->stream));
+  cudaPointerAttributes attr{}, last{};
+  const cudaError_t e = cudaPointerGetAttributes(&attr, R);
+  bool by_kernel = e == cudaSuccess && (attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged);
+  if (by_kernel && !c->bf16) {
+    // float32: memory of this device, both ends known to be there; cudaMemcpy2DAsync takes the rest
+    int dev = 0;
+    DID_CUDA(c, cudaGetDevice(&dev));
+    by_kernel = c->M > did::kUnpadMinRows && attr.type == cudaMemoryTypeDevice && attr.device == dev &&
+                cudaPointerGetAttributes(&last, R + (size_t)c->M * c->N - 1) == cudaSuccess &&
+                last.type == cudaMemoryTypeDevice && last.device == dev && ((uintptr_t)R & 3) == 0;
+  }
+  cudaGetLastError();
+  if (by_kernel) {
+    DID_CUDA(c, did::launch_unpad(c->R, c->bf16, R, (int)c->M, c->ld, (int)c->M, c->N, c->stream));
     DID_CUDA(c, cudaStreamSynchronize(c->stream));
     return DID_OK;
   }
-  cudaPointerAttributes attr{};
-  cudaError_t e = cudaPointerGetAttributes(&attr, R);
-  cudaGetLastError();
-  const bool on_device = e == cudaSuccess && (attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged);
-  if (on_device) {
-    DID_CUDA(c, did::launch_bf16_to_f32(c->R, R, (int)c->M, c->ld, (int)c->M, c->N, c->stream));
+  if (!c->bf16) {
+    DID_CUDA(c, cudaMemcpy2DAsync(R, (size_t)c->M * sizeof(float), c->R, (size_t)c->ld * sizeof(float),
+                                  (size_t)c->M * sizeof(float), (size_t)c->N, cudaMemcpyDefault, c->stream));
     DID_CUDA(c, cudaStreamSynchronize(c->stream));
     return DID_OK;
   }
@@ -907,7 +915,7 @@ did_status did_get_residual(did_ctx* c, float* R) {
     cudaGetLastError();
     return fail(c, DID_ENOMEM, "temporary buffer of %zu bytes for the residual", bytes);
   }
-  cudaError_t e1 = did::launch_bf16_to_f32(c->R, tmp, (int)c->M, c->ld, (int)c->M, c->N, c->stream);
+  cudaError_t e1 = did::launch_unpad(c->R, true, tmp, (int)c->M, c->ld, (int)c->M, c->N, c->stream);
   cudaError_t e2 = e1 == cudaSuccess ? cudaMemcpyAsync(R, tmp, bytes, cudaMemcpyDefault, c->stream) : e1;
   cudaError_t e3 = cudaStreamSynchronize(c->stream);
   cudaFree(tmp);

@@ -481,7 +481,8 @@ cudaError_t launch_gen_planted_x_ld(float* X, int ldx, const float* B0, const fl
 cudaError_t launch_check_nonneg_finite(const float* X, int rows, int ld, int64_t cols,
                                        unsigned long long* bad, cudaStream_t s);
 cudaError_t launch_scale(float* p, int64_t n, float s, cudaStream_t st);
-cudaError_t launch_bf16_to_f32(const void* R, float* out, int rows, int ld_in, int ld_out,
-                               int64_t cols, cudaStream_t s);
+constexpr int kUnpadMinRows = 128;
+cudaError_t launch_unpad(const void* R, bool bf16, float* out, int rows, int ld_in, int ld_out, int64_t cols,
+                         cudaStream_t s);
 
 }  // namespace did

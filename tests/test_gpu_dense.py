@@ -33,3 +33,18 @@ def test_refresh_and_objective(did, M, N, K, precision):
     assert np.all(np.abs(R - Rd) <= bound + 1e-30)
     fd = 0.5 * float(np.sum(Rd ** 2))
     assert abs(f - fd) <= 1e-5 * fd and abs(f0 - fd) <= 1e-5 * fd
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("M,N", [(1, 1), (31, 4501), (33, 9003), (100, 7001), (128, 513), (129, 40), (257, 33), (1024, 300), (1025, 299), (8165, 70)])
+def test_residual_copies(did, M, N, precision):
+    """The residual to device memory (any 4-byte aligned address) and to the host: the same values."""
+    import torch
+    X, _, _ = W.planted(M, N, 1, seed=M + N, sigma=0.05)
+    with did.Context(np.ascontiguousarray(X.T), M, N, 1, seed=3, precision=precision) as ctx:
+        host = ctx.residual()
+        buf = torch.full((M * N + 2,), 7.0, device="cuda")
+        did.did_get_residual(ctx.h, buf[1:M * N + 1])
+    got = buf.cpu().numpy()
+    assert got[0] == 7.0 and got[-1] == 7.0
+    assert np.array_equal(got[1:-1].reshape(N, M), np.asarray(host).T)

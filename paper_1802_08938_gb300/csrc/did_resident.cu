@@ -531,6 +531,7 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
       const float* cx = crow(knext);
       if (send && K > 1) {
         if (ck == cx) {
+          __syncthreads();                         // the previous update has read cold
           for (int c = t; c < nc; c += kResThreads) cold[c] = ck[c];
           ck = cold;
           __syncthreads();

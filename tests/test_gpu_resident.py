@@ -60,6 +60,27 @@ def test_matches_oracle(did, M, N, K, order):
     assert np.max(np.abs(got["R"] - Rd)) <= 1e-4 * max(1.0, float(np.abs(X).max()))
 
 
+@pytest.mark.parametrize("M,N,K,sweeps", [(513, 9001, 5, 12), (513, 9001, 7, 12), (300, 9601, 3, 20), (1040, 4961, 3, 20)])
+def test_odd_k_sweeps_of_one_launch(did, M, N, K, sweeps):
+    """With odd K the last step of a sweep keeps its row of C in the buffer the
+    update before it reads: rows that some warps of a CTA have more of than
+    others (ld not a multiple of 512), and more than 32 columns a CTA."""
+    X, _, _ = W.planted(M, N, K, seed=M + K, sigma=0.05)
+    B0, C0 = W.init_factors(M, N, K, 5)
+    ref = O.factor(X, B0, C0, order="hals", max_iter=sweeps, stop="none")
+    got = run(did, X, B0, C0, (sweeps,))
+    assert -(-N // got["info"]["grid_ctas"]) > 32
+    assert rel(got["B"], ref["B"]) <= 1e-5 and rel(got["C"], ref["C"]) <= 1e-5
+    for _ in range(3):
+        again = run(did, X, B0, C0, (sweeps,))
+        for key in ("B", "C", "R", "trace"):
+            assert np.array_equal(got[key], again[key]), key
+    # each step of a sweep rounds an entry of R three times, by 2^-24 of |R| and of the product each
+    S = np.abs(got["B"]).astype(np.float64) @ got["C"].astype(np.float64)
+    Rd = X.astype(np.float64) - got["B"].astype(np.float64) @ got["C"].astype(np.float64)
+    assert np.all(np.abs(got["R"] - Rd) <= 3 * K * sweeps * 2.0 ** -24 * (np.abs(X) + S))
+
+
 @pytest.mark.parametrize("order", [0, 1])
 def test_bfloat16_residual_and_refresh(did, order):
     M, N, K = 700, 1501, 12

@@ -64,6 +64,7 @@ bool plan_cfirst(int ld, int64_t N, int K, bool bf16, CfirstPlan* plan) {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   CfirstPlan P{};
   P.grid = sms;
+  if (defer_rows(ld, P.grid) > kMaxRows) return false;
   P.GS = 32;
   while (P.GS < kWorkThreads && P.GS * 16 < ld) P.GS *= 2;
   const int NR = std::max(1, (nvec + P.GS - 1) / P.GS);

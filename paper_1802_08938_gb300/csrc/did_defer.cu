@@ -55,6 +55,7 @@ bool plan_defer(int ld, int64_t N, int K, bool bf16, int grid_override, DeferPla
   if (K > 128) return false;
   DeferPlan P{};
   P.grid = grid_override > 0 ? std::min(grid_override, sms) : sms;
+  if (defer_rows(ld, P.grid) > kMaxRows) return false;
   // Threads of a column group: as few as hold a column in 16 rows each, so
   // that a warp's reduction is shared by much of a column and b_k', the
   // partials and a chunk stay in registers; 512 beyond that.

@@ -162,6 +162,9 @@ struct DeferSmem {
 __host__ __device__ __forceinline__ size_t smax(size_t a, size_t b) { return a > b ? a : b; }
 __host__ __device__ __forceinline__ size_t al16(size_t x) { return (x + 15) & ~(size_t)15; }
 // Rows of a CTA's slice: a multiple of four, for 16-byte loads of the partial rows.
+// A thread adds the partial rows of one quad of them, so a slice holds at
+// most kMaxRows; the planners refuse longer ones (a grid of few CTAs).
+constexpr int kMaxRows = 4 * kWorkThreads;
 __host__ __device__ __forceinline__ int defer_rows(int ld, int grid) { return ((ld + grid - 1) / grid + 3) / 4 * 4; }
 __host__ __device__ __forceinline__ DeferSmem defer_smem(int ld, int K, int grid, int S, int CW, int elem) {
   DeferSmem L;

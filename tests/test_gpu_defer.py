@@ -103,3 +103,20 @@ def test_expired_wait_is_reported(did):
         assert e.value.status == did.DID_ETIMEOUT
         B, C = ctx.factors()
         assert np.isfinite(B).all() and (B >= 0).all() and np.isfinite(C).all() and (C >= 0).all()
+
+
+@pytest.mark.parametrize("M,N,K,grid", [(2048, 2105, 4, 1), (4096, 1101, 3, 2), (2064, 2100, 4, 1), (3000, 2000, 4, 1),
+                                        (5000, 1000, 4, 2), (9000, 600, 3, 4)])
+def test_few_ctas(did, M, N, K, grid):
+    """A grid given by the caller: slices of 2048 rows, the longest that phase A
+    of the read-only sweep adds up, and longer ones, which the kernel that
+    writes R takes."""
+    X, _, _ = W.planted(M, N, K, seed=M + N, sigma=0.05)
+    B0, C0 = W.init_factors(M, N, K, 5)
+    ref = O.factor(X, B0, C0, order="hals", max_iter=3, stop="none")
+    got = run(did, X, B0, C0, 3, grid_ctas=grid)
+    assert got["info"]["grid_ctas"] == grid
+    eB, eC = rel(got["B"], ref["B"]), rel(got["C"], ref["C"])
+    eF = float(np.max(np.abs(got["trace"] - ref["trace"]) / ref["trace"]))
+    print("read-only M=%d N=%d K=%d grid=%d: relB %.3g relC %.3g relf %.3g" % (M, N, K, grid, eB, eC, eF))
+    assert eB <= 1e-5 and eC <= 1e-5 and eF <= 1e-5

@@ -67,6 +67,14 @@ __host__ __device__ __forceinline__ CfSmem cf_smem(int ld, int K, int grid, int 
   return L;
 }
 
+// Whether an earlier launch stopped or failed (the C step of this sweep included):
+// nothing of this one runs then.  err may also be of this launch, set by a CTA
+// ahead of this one; the CTAs that began then leave at their next wait.  One
+// thread reads, so that a CTA's threads agree.
+__device__ __forceinline__ bool launch_ended(const Ctrl* ctrl) {
+  return __syncthreads_or(threadIdx.x == 0 && (ld_volatile(&ctrl->stopped) != 0 || ld_volatile(&ctrl->err) != 0)) != 0;
+}
+
 // What both kernels set up.
 struct Cta {
   unsigned char* ring;
@@ -103,7 +111,7 @@ __device__ __forceinline__ Cta cf_setup(unsigned char* smem, const CfSmem& L, in
 #define DID_CF_GRID_SYNC()                                                                                      \
   do {                                                                                                          \
     ++nbar;                                                                                                     \
-    if (!work_grid_sync(&a.ctrl->bar, nbar * (unsigned)G + (unsigned)a.bar_extra, err, tmo, sm.s_ok)) {          \
+    if (!work_grid_sync(&a.ctrl->bar, nbar * (unsigned)G + (unsigned)a.bar_extra, err, tmo, sm.s_ok, sm.quit)) { \
       if (t == 0) *sm.quit = 1;                                                                                 \
       return;                                                                                                   \
     }                                                                                                           \
@@ -113,7 +121,7 @@ __device__ __forceinline__ Cta cf_setup(unsigned char* smem, const CfSmem& L, in
 template <int NR, int CW, int KB, bool BF16>
 __global__ void __launch_bounds__(kThreads, 1) cstep_kernel(CfArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
-  if (a.ctrl->stopped) return;
+  if (launch_ended(a.ctrl)) return;
   typedef Vec<BF16> V;
   typedef typename V::raw raw;
   constexpr int VR = V::kRows, VH = VR / 2, ELEM = BF16 ? 2 : 4;
@@ -188,7 +196,10 @@ __global__ void __launch_bounds__(kThreads, 1) cstep_kernel(CfArgs a) {
         }
       }
     while (true) {
-      if (!stage_wait(sm.full + cst, cph, err, tmo)) break;       // the next grid barrier sees the error
+      if (!stage_wait(sm.full + cst, cph, err, tmo)) {
+        *sm.quit = 1;                              // the CTA leaves after this pass
+        break;
+      }
       const int64_t j = sm.meta[cst].j;
       const int n = sm.meta[cst].n;
       const unsigned st = cst;
@@ -253,6 +264,7 @@ __global__ void __launch_bounds__(kThreads, 1) cstep_kernel(CfArgs a) {
     } else {
       __threadfence_block();
       work_sync();
+      if (*sm.quit) return;
     }
     // own columns: c_k' for the block's k in turn
     for (int64_t j = jlo + t; j < jhi; j += kWorkThreads) {
@@ -315,7 +327,7 @@ __global__ void __launch_bounds__(kThreads, 1) cstep_kernel(CfArgs a) {
 template <int NR, int CW, int KB, bool BF16>
 __global__ void __launch_bounds__(kThreads, 1) bstep_kernel(CfArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
-  if (a.ctrl->stopped) return;
+  if (launch_ended(a.ctrl)) return;
   typedef Vec<BF16> V;
   typedef typename V::raw raw;
   constexpr int VR = V::kRows, VH = VR / 2, ELEM = BF16 ? 2 : 4;
@@ -410,7 +422,10 @@ __global__ void __launch_bounds__(kThreads, 1) bstep_kernel(CfArgs a) {
         }
       };
       while (true) {
-        if (!stage_wait(sm.full + cst, cph, err, tmo)) break;
+        if (!stage_wait(sm.full + cst, cph, err, tmo)) {
+          *sm.quit = 1;
+          break;
+        }
         const int n = sm.meta[cst].n, u = sm.meta[cst].u;
         const unsigned st = cst;
         cst += (unsigned)NG;

@@ -19,12 +19,19 @@ namespace {
 
 // Closes a sweep: f = 1/2 ||R||^2 from the refresh's per-CTA sums (a tree of
 // fixed shape), the stopping rule, and the barrier and the unit counters cleared
-// for the next launch.  Nothing after a sweep that stopped or failed.
+// for the next launch.  After a sweep that failed it stops the later ones of the
+// queue instead: their barrier and unit counters would begin where the
+// failed one left them.  Nothing after a sweep that stopped.
 constexpr int kCloseThreads = 128;
 __global__ void defer_close_kernel(const double* part, int n, int stride, Ctrl* ctrl, unsigned* work, int nwork, double* trace,
                                    int stop_rule, double tol, double f_prev, double f0, int first) {
   __shared__ double sum[kCloseThreads];
-  if (ctrl->stopped || ctrl->err) return;
+  if (ctrl->stopped) return;
+  if (ctrl->err) {
+    __syncthreads();
+    if (threadIdx.x == 0) ctrl->stopped = 1;
+    return;
+  }
   for (int i = threadIdx.x; i < nwork; i += blockDim.x) work[i] = 0u;
   double s = 0.0;
   for (int i = threadIdx.x; i < n; i += kCloseThreads) s += part[(size_t)i * stride];

@@ -202,10 +202,13 @@ __device__ __forceinline__ void side_arrive(int id) {
 __device__ __forceinline__ void side_wait(int id) { named_bar(id, kWorkThreads + kSideThreads); }
 
 // Grid barrier of the computing warps (see grid_sync): release add, acquire
-// poll without back-off; the limit is read every 64 polls.
+// poll without back-off; the limit is read every 64 polls.  A CTA one of whose
+// threads gave up waiting for a stage (*quit) does not arrive, so no CTA goes
+// on with its partial sums.
 __device__ __forceinline__ bool work_grid_sync(unsigned* bar, unsigned target, int* err, uint64_t timeout_ns,
-                                               int* s_ok) {
+                                               int* s_ok, volatile int* quit) {
   work_sync();
+  if (*quit) return false;
   if (threadIdx.x == 0) {
     int ok = 1;
     __threadfence();
@@ -230,16 +233,17 @@ __device__ __forceinline__ bool work_grid_sync(unsigned* bar, unsigned target, i
   return *s_ok != 0;
 }
 
-// Wait for phase `parity` of a stage, bounded by the limit (looked at every 64
-// polls: %globaltimer is slow to read).
+// Wait of a whole warp for phase `parity` of a stage, bounded by the limit
+// (looked at every 64 polls: %globaltimer is slow to read).  The lanes agree on the
+// result, as what follows shuffles among all of them.
 __device__ __forceinline__ bool stage_wait(uint64_t* b, uint32_t parity, int* err, uint64_t timeout_ns) {
-  if (mbar_try_wait(b, parity)) return true;
+  if (__all_sync(0xffffffffu, mbar_try_wait(b, parity))) return true;
   uint64_t t0 = 0;
-  for (unsigned i = 1; !mbar_try_wait(b, parity); ++i) {
+  for (unsigned i = 1; !__all_sync(0xffffffffu, mbar_try_wait(b, parity)); ++i) {
     if ((i & 63u) == 0) {
       const uint64_t t = globaltimer_ns();
       if (t0 == 0) t0 = t;
-      if (t - t0 > timeout_ns || i > (1u << 28)) {
+      if (__any_sync(0xffffffffu, t - t0 > timeout_ns || i > (1u << 28))) {
         atomicCAS(err, 0, kDevErrTimeout);
         return false;
       }
@@ -417,8 +421,8 @@ __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
   float* cxs = reinterpret_cast<float*>(smem + L.cx);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + L.bars);
   uint64_t* empty = full + S;
-  volatile int* quit = reinterpret_cast<volatile int*>(smem + L.misc);
-  int* s_ok = reinterpret_cast<int*>(smem + L.misc) + 1;
+  __shared__ volatile int quit;                   // -1: a computing thread gave up waiting for a stage; 1: the CTA leaves
+  int* s_ok = reinterpret_cast<int*>(smem + L.misc);
   df* cc0 = reinterpret_cast<df*>(smem + L.misc + 16);             // ||c_1||^2 of the refresh
   int* err = &a.ctrl->err;
   const uint64_t tmo = a.timeout_ns;
@@ -430,7 +434,7 @@ __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
     mbar_init(full + t, 1);
     mbar_init(empty + t, GS / 32);
   }
-  if (t == 0) *quit = 0;
+  if (t == 0) quit = 0;
   fence_mbar_init();
   __syncthreads();
 
@@ -438,7 +442,7 @@ __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
     // ------------------------------------------------------------ producer
     // (pass k takes c_{k+1} along)
     Stream p{a.R, N, colbytes, ring, meta, cxs, kMaxCw, full, empty, S, NG, G, cta, a.units, a.nunits, a.dynamic,
-             a.work + (a.npart_first > 0 ? 1 : 0), quit, err, tmo};
+             a.work + (a.npart_first > 0 ? 1 : 0), &quit, err, tmo};
     produce<CW, 1>(p, a.npart_first > 0 ? 0 : -1, K,
                    [&](int k, int) -> const float* { return k + 1 < K ? a.C + (int64_t)(k + 1) * N : nullptr; });
     return;
@@ -461,7 +465,7 @@ __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
     df* xwarp = xw + (size_t)(16 + ws) * 2 * (K + 1);
     for (int k = 0; k < K; ++k) {
       side_wait(2);
-      if (*quit) return;
+      if (quit > 0) return;
       const bool more = k + 1 < K;
       const float* cn_row = a.C + (int64_t)(more ? k + 1 : 0) * N;
       for (int e = lane; e < 2 * (K + 1); e += 32) xwarp[e] = df_zero();
@@ -518,14 +522,20 @@ __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
 
   // ------------------------------------------------------- computing warps
   unsigned nbar = 0;
-#define DID_DEFER_GRID_SYNC()                                                                                  \
+  // Leaving: the side warps are let on once more and see it.  Where they may be
+  // in phase B (busy), they finish it first, so that all of them see it at the same start.
+#define DID_DEFER_LEAVE(busy)   \
+  do {                          \
+    if (busy) side_wait(3);     \
+    if (t == 0) quit = 1;       \
+    side_arrive(2);             \
+    return;                     \
+  } while (0)
+#define DID_DEFER_GRID_SYNC(busy)                                                                              \
   do {                                                                                                         \
     ++nbar;                                                                                                    \
-    if (!work_grid_sync(&a.ctrl->bar, nbar * (unsigned)G + (unsigned)a.bar_extra, err, tmo, s_ok)) {            \
-      if (t == 0) *quit = 1;                                                                                   \
-      side_arrive(2);                                                                                          \
-      return;                                                                                                  \
-    }                                                                                                          \
+    if (!work_grid_sync(&a.ctrl->bar, nbar * (unsigned)G + (unsigned)a.bar_extra, err, tmo, s_ok, &quit))       \
+      DID_DEFER_LEAVE(busy);                                                                                   \
   } while (0)
 
   const int g = t / GS, lt = t - g * GS;          // column group, place in it
@@ -647,7 +657,7 @@ __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
         __stcg(reinterpret_cast<float2*>(a.Yp + (size_t)(2 * t + 1) * G + cta), make_float2(sn.h, sn.l));
       }
     }
-    DID_DEFER_GRID_SYNC();
+    DID_DEFER_GRID_SYNC(false);
     if (rec) a.tstamp[4 * k + 1] = globaltimer_ns();
 
     sum_over_ctas(a.Yp, 2 * k + 2, G, sums);
@@ -727,7 +737,10 @@ __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
         }
       };
       while (true) {
-        if (!stage_wait(full + cst, cph, err, tmo)) break;   // the next grid barrier sees the error
+        if (!stage_wait(full + cst, cph, err, tmo)) {
+          quit = -1;                               // the CTA leaves after this phase
+          break;
+        }
         const int64_t j = meta[cst].j;
         const int n = meta[cst].n, u = meta[cst].u;
         const unsigned st = cst;
@@ -825,10 +838,11 @@ __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
     }
     if (rec) a.tstamp[4 * k + 2] = globaltimer_ns();
     if (a.dynamic) {
-      DID_DEFER_GRID_SYNC();
+      DID_DEFER_GRID_SYNC(k >= 0);
     } else {
       __threadfence_block();
       work_sync();
+      if (quit) DID_DEFER_LEAVE(k >= 0);
     }
 
     // ------------------------------------------------------------ phase F
@@ -915,10 +929,11 @@ __global__ void __launch_bounds__(kDeferThreads, 1) defer_kernel(DeferArgs a) {
       for (int e = e0; e < e1; ++e) s = df_add(s, xw[(size_t)e * 2 * (K + 1) + src]);
       __stcg(reinterpret_cast<float2*>(a.Xp + (size_t)i * G + cta), make_float2(s.h, s.l));
     }
-    DID_DEFER_GRID_SYNC();
+    DID_DEFER_GRID_SYNC(false);
     if (rec) a.tstamp[4 * k + 3] = globaltimer_ns();
   }
 #undef DID_DEFER_GRID_SYNC
+#undef DID_DEFER_LEAVE
   if (stamps && K - 1 < a.tstamp_cap) a.tstamp[4 * (K - 1) + 3] = globaltimer_ns();
 }
 

@@ -25,7 +25,7 @@ constexpr int kDevErrTimeout = 1;     // a grid wait ran out of time
 struct Ctrl {
   unsigned bar;        // grid-barrier arrival counter
   int err;             // device error word
-  int stopped;         // 1 when the stopping rule held inside the launch
+  int stopped;         // 1 when the stopping rule held inside the launch (read-only sweeps: or one failed)
   int sweeps;          // sweeps completed by the launch
   unsigned work[2];    // column-unit counters of alternate passes
 };
@@ -356,7 +356,7 @@ cudaError_t launch_resident(const ResidentPlan& plan, const SweepArgs& args, voi
 // after it (launch_refresh_tc, with the partials of R c_1^T, or launch_dense
 // without them) and closes the sweep with launch_defer_close, which adds the
 // n sums of R^2 at part[stride * i] and applies the stopping rule; a launch
-// that finds Ctrl::stopped set does nothing.
+// that finds Ctrl::stopped set (the rule held, or a sweep failed) does nothing.
 struct DeferPlan {
   int grid, GS, NG, NR, CW, S;
   Units units;

@@ -120,3 +120,21 @@ def test_few_ctas(did, M, N, K, grid):
     eF = float(np.max(np.abs(got["trace"] - ref["trace"]) / ref["trace"]))
     print("read-only M=%d N=%d K=%d grid=%d: relB %.3g relC %.3g relf %.3g" % (M, N, K, grid, eB, eC, eF))
     assert eB <= 1e-5 and eC <= 1e-5 and eF <= 1e-5
+
+
+def test_expired_wait_ends_the_queued_sweeps(did):
+    """After an expired wait the sweeps queued behind it change nothing: B and C
+    are those that one sweep leaves, whatever the number asked for, and the
+    context goes on from them."""
+    M, N, K = 800, 12003, 3
+    X, _, _ = W.planted(M, N, K, seed=1, sigma=0.05)
+    left = []
+    for n in (1, 6, 6):
+        with did.Context(np.ascontiguousarray(X.T), M, N, K, seed=0, timeout_ns=10 ** 7, debug_barrier_extra=1) as ctx:
+            with pytest.raises(did.DIDError) as e:
+                ctx.sweep(n)
+            assert e.value.status == did.DID_ETIMEOUT
+            left.append((*ctx.factors(), ctx.trace(), ctx.info()["sweeps_done"]))
+    for B, C, trace, done in left[1:]:
+        assert np.array_equal(B, left[0][0]) and np.array_equal(C, left[0][1])
+        assert len(trace) == 1 and done == 0

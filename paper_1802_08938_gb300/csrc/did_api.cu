@@ -463,6 +463,7 @@ did_status run_defer(did_ctx* c, int64_t max_sweeps, int stop_rule, double tol, 
   da.K = c->K;
   da.N = c->N;
   da.bf16 = c->bf16 ? 1 : 0;
+  da.stop = &c->ctrl->stopped;
   unsigned* work = c->cfirst ? c->cbuf.work : c->dbuf.work;
   const int nwork = c->cfirst ? 2 * c->K : c->K + 1;
   while (*done_total < max_sweeps) {
@@ -495,7 +496,7 @@ did_status run_defer(did_ctx* c, int64_t max_sweeps, int stop_rule, double tol, 
       if (tc) {
         DID_CUDA(c, did::launch_refresh_tc(c->X, c->R, c->B, c->C, (int)c->M, c->ld, c->N, c->K, c->tc_ws, c->tc_part,
                                            c->defer ? c->P : nullptr, c->defer ? c->CCp : nullptr, &c->ctrl->err,
-                                           tmo, c->stream, !c->bf16));
+                                           tmo, c->stream, !c->bf16, &c->ctrl->stopped));
         DID_CUDA(c, did::launch_defer_close(c->tc_part, G, 1, c->ctrl, work, nwork, c->trace_dev + s,
                                              stop_rule, tol, f_start, f0, s == 0, c->stream));
       } else {

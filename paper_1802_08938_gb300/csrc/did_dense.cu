@@ -49,6 +49,8 @@ __global__ void __launch_bounds__(kDenseThreads) dense_kernel(DenseTileArgs t) {
   __shared__ __align__(16) float Cs[kKc][kTile];
   __shared__ double scratch[kDenseThreads / 32];
 
+  if (a.stop && *a.stop) return;                   // (set by an earlier launch)
+
   const int tr = threadIdx.x & 15, tc = threadIdx.x >> 4;
   const int mt = (a.M + kTile - 1) / kTile;
   const int64_t nt = (a.N + kTile - 1) / kTile;
@@ -165,6 +167,7 @@ __global__ void __launch_bounds__(kBigThreads, 2) dense_big_kernel(DenseArgs a) 
   __shared__ __align__(16) float Bs[2][kBigKc][kBig];
   __shared__ __align__(16) float Cs[2][kBigKc][kBig];
   __shared__ double scratch[kBigThreads / 32];
+  if (a.stop && *a.stop) return;
   const int t = threadIdx.x;
   const int tr = t & 15, tc = t >> 4;              // rows 4 tr.. and 64 + 4 tr.., columns 4 tc.. and 64 + 4 tc..
   const int mt = (a.ld + kBig - 1) / kBig;

@@ -430,6 +430,7 @@ struct DenseArgs {
   int64_t N;
   int mode;
   int bf16;
+  const int* stop;    // the launch does nothing when *stop is set (or null)
 };
 int dense_grid();
 cudaError_t launch_dense(const DenseArgs& a, cudaStream_t s);
@@ -444,7 +445,7 @@ size_t refresh_tc_workspace_bytes(int M, int ld, int64_t N, int K, bool f32);
 int refresh_tc_grid();
 cudaError_t launch_refresh_tc(const float* X, void* R, const float* B, const float* C, int M, int ld, int64_t N,
                               int K, void* workspace, double* part, float* P1, double* CC1, int* err,
-                              uint64_t timeout_ns, cudaStream_t s, bool f32);
+                              uint64_t timeout_ns, cudaStream_t s, bool f32, const int* stop = nullptr);
 
 // Batched DID (Algorithm 3 with one reduction per sweep) on the library's
 // tensor-core kernels (did_batched.cu); K <= 64.

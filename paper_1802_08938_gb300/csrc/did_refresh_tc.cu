@@ -74,8 +74,9 @@ struct TcArgs {
   const void* Bhl;           // [col tiles][terms][64 cols x Kp] tiled C factor
   double* part;              // [grid] sum of R^2 per CTA
   const float* c1;           // row 1 of C (N floats), or null: no partials
-  float* P1;                 // [2 grid][ld] partials of R c_1^T (row 2 cta + column half), zeroed by the host
+  float* P1;                 // [2 grid][ld] partials of R c_1^T (row 2 cta + column half), zeroed by prep_b_kernel
   double* CC1;               // [2 grid] partials of ||c_1||^2
+  const int* stop;           // the launch does nothing when *stop is set (or null)
   int* err;                  // error word
   int M, ld, Kp;
   int xbufs;                 // X tile buffers (2..kMaxXBuf)
@@ -134,6 +135,7 @@ __device__ __forceinline__ void rt_unit(const TcArgs& a, int64_t u, int& rb, int
 template <bool F32>
 __global__ void __launch_bounds__(kTcThreads, 1) refresh_tc_kernel(TcArgs a, const __grid_constant__ CUtensorMap tmX,
                                                                   const __grid_constant__ CUtensorMap tmR) {
+  if (a.stop && *a.stop) return;                  // (set by an earlier launch)
   constexpr int NT = F32 ? 3 : 2;                 // bfloat16 terms per operand
   // TMEM columns of one accumulator: range r holds the products p_i q_j with
   // i + j = r.  The tensor core's float32 accumulation truncates, so every
@@ -466,9 +468,15 @@ __device__ __forceinline__ void split_terms(float v, __nv_bfloat16* t) {
   }
 }
 
-// B factor (ld x K column-major float32) -> [row block][term][128 x Kp].
+// B factor (ld x K column-major float32) -> [row block][term][128 x Kp].  It
+// also clears the n1 partials of R c_1^T: a CTA of the pass adds only the rows
+// of its units.
 template <int NT>
-__global__ void prep_b_kernel(const float* B, int M, int ld, int K, int Kp, int row_blocks, __nv_bfloat16* out) {
+__global__ void prep_b_kernel(const float* B, int M, int ld, int K, int Kp, int row_blocks, __nv_bfloat16* out,
+                              float* P1, int64_t n1, const int* stop) {
+  if (stop && *stop) return;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n1 / 4; i += (int64_t)gridDim.x * blockDim.x)
+    reinterpret_cast<float4*>(P1)[i] = make_float4(0.f, 0.f, 0.f, 0.f);   // (ld is a multiple of 16)
   const int64_t n = (int64_t)row_blocks * kTileM * Kp;
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n;
        idx += (int64_t)gridDim.x * blockDim.x) {
@@ -486,7 +494,9 @@ __global__ void prep_b_kernel(const float* B, int M, int ld, int K, int Kp, int 
 
 // C factor (K x N row-major float32) -> [column tile][term][64 x Kp].
 template <int NT>
-__global__ void prep_c_kernel(const float* C, int64_t N, int K, int Kp, int64_t col_tiles, __nv_bfloat16* out) {
+__global__ void prep_c_kernel(const float* C, int64_t N, int K, int Kp, int64_t col_tiles, __nv_bfloat16* out,
+                              const int* stop) {
+  if (stop && *stop) return;
   const int64_t n = col_tiles * kTileN * Kp;
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n;
        idx += (int64_t)gridDim.x * blockDim.x) {
@@ -528,7 +538,7 @@ int refresh_tc_grid() { return sm_count_tc(); }
 template <bool F32>
 static cudaError_t launch_tc(const float* X, void* R, const float* B, const float* C, int M, int ld, int64_t N,
                              int K, void* workspace, double* part, float* P1, double* CC1, int* err,
-                             uint64_t timeout_ns, cudaStream_t s) {
+                             uint64_t timeout_ns, cudaStream_t s, const int* stop) {
   const int Kp = (K + 15) / 16 * 16;
   const int row_blocks = (ld + kTileM - 1) / kTileM;
   const int64_t col_tiles = (N + kTileN - 1) / kTileN;
@@ -536,8 +546,9 @@ static cudaError_t launch_tc(const float* X, void* R, const float* B, const floa
   __nv_bfloat16* Ahl = static_cast<__nv_bfloat16*>(workspace);
   __nv_bfloat16* Bhl = Ahl + (size_t)row_blocks * NT * kTileM * Kp;
   const int sms = sm_count_tc();
-  prep_b_kernel<NT><<<sms * 4, 256, 0, s>>>(B, M, ld, K, Kp, row_blocks, Ahl);
-  prep_c_kernel<NT><<<sms * 8, 256, 0, s>>>(C, N, K, Kp, col_tiles, Bhl);
+  prep_b_kernel<NT><<<sms * 4, 256, 0, s>>>(B, M, ld, K, Kp, row_blocks, Ahl, P1, P1 ? (int64_t)2 * sms * ld : 0,
+                                            stop);
+  prep_c_kernel<NT><<<sms * 8, 256, 0, s>>>(C, N, K, Kp, col_tiles, Bhl, stop);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   TcArgs a{};
@@ -549,6 +560,7 @@ static cudaError_t launch_tc(const float* X, void* R, const float* B, const floa
   a.c1 = P1 ? C : nullptr;   // row 1 of the row-major K x N factor
   a.P1 = P1;
   a.CC1 = CC1;
+  a.stop = stop;
   a.err = err;
   a.M = M;
   a.ld = ld;
@@ -619,22 +631,16 @@ static cudaError_t launch_tc(const float* X, void* R, const float* B, const floa
   const size_t smem = tc_smem(Kp, NT, a.xbufs, a.cbufs).total;
   e = cudaFuncSetAttribute(refresh_tc_kernel<F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  // the partial rows of R c_1^T start at zero: a CTA adds only the rows of its units
-  if (P1) {
-    e = cudaMemsetAsync(P1, 0, (size_t)2 * sms * ld * sizeof(float), s);
-    if (e != cudaSuccess) return e;
-  }
   refresh_tc_kernel<F32><<<sms, kTcThreads, smem, s>>>(a, tmX, tmR);
   return cudaGetLastError();
 }
 
 cudaError_t launch_refresh_tc(const float* X, void* R, const float* B, const float* C, int M, int ld, int64_t N, int K,
                               void* workspace, double* part, float* P1, double* CC1, int* err, uint64_t timeout_ns,
-                              cudaStream_t s, bool f32) {
+                              cudaStream_t s, bool f32, const int* stop) {
   if (!refresh_tc_supported(K, f32)) return cudaErrorInvalidValue;
-  return f32 ? launch_tc<true>(X, R, B, C, M, ld, N, K, workspace, part, P1, CC1, err, timeout_ns, s)
-             : launch_tc<false>(X, R, B, C, M, ld, N, K, workspace, part, P1, CC1, err, timeout_ns,
-                                               s);
+  return f32 ? launch_tc<true>(X, R, B, C, M, ld, N, K, workspace, part, P1, CC1, err, timeout_ns, s, stop)
+             : launch_tc<false>(X, R, B, C, M, ld, N, K, workspace, part, P1, CC1, err, timeout_ns, s, stop);
 }
 
 }  // namespace did

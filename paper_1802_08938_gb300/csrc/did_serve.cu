@@ -596,6 +596,7 @@ bool run_round(did_server* s, std::vector<Req*>& act) {
     da.K = r->rq.K;
     da.N = r->rq.N;
     da.bf16 = s->bf16 ? 1 : 0;
+    da.stop = &d.b.ctrl->stopped;
     if (e == cudaSuccess) e = cudaMemsetAsync(d.b.work, 0, sizeof(unsigned) * (r->rq.K + 1), st);
     for (int q = 0; q < nsw && e == cudaSuccess; ++q) {
       // (the partials of c_1 are in the scratch: another request may have used it since)
@@ -603,7 +604,8 @@ bool run_round(did_server* s, std::vector<Req*>& act) {
                             nullptr, 0, st);
       if (e == cudaSuccess)
         e = d.tc_ws ? did::launch_refresh_tc(r->X, r->R, r->B, r->C, (int)r->rq.M, r->ld, r->rq.N, r->rq.K, d.tc_ws,
-                                             d.part, d.b.P, d.b.CC0, &d.b.ctrl->err, kServeTimeoutNs, st, !s->bf16)
+                                             d.part, d.b.P, d.b.CC0, &d.b.ctrl->err, kServeTimeoutNs, st, !s->bf16,
+                                             &d.b.ctrl->stopped)
                     : did::launch_dense(da, st);
       if (e == cudaSuccess)
         e = did::launch_defer_close(d.tc_ws ? d.part : s->d_part, d.tc_ws ? G : s->dense_grid, d.tc_ws ? 1 : 3,

@@ -138,3 +138,29 @@ def test_expired_wait_ends_the_queued_sweeps(did):
     for B, C, trace, done in left[1:]:
         assert np.array_equal(B, left[0][0]) and np.array_equal(C, left[0][1])
         assert len(trace) == 1 and done == 0
+
+
+@pytest.mark.parametrize("order,K", [(0, 1), (1, 1), (0, 70)])
+def test_stop_ends_the_queued_sweeps(did, order, K):
+    """With a stopping rule a few sweeps are queued ahead.  Once it holds, the
+    passes that would form R again do nothing either: a call that stops after
+    its first sweep takes no longer than one sweep (three more passes over X and R
+    would triple it at K = 1), and the next call goes on from the same state."""
+    M, N = (1500, 40000) if K == 1 else (300, 40000)
+    X, _, _ = W.planted(M, N, K, seed=3, sigma=0.05)
+    Xc = np.ascontiguousarray(X.T)
+    with did.Context(Xc, M, N, K, seed=1, order=order) as a, did.Context(Xc, M, N, K, seed=1, order=order) as b:
+        ms = {}
+        for ctx, call in ((a, lambda: a.sweep(1)), (b, lambda: b.factor(4, 1.0))):
+            t = []
+            for _ in range(6):
+                t0 = ctx.info()["sweep_kernel_ms"]
+                call()
+                t.append(ctx.info()["sweep_kernel_ms"] - t0)
+            ms[ctx] = min(t)
+        assert a.info()["sweeps_done"] == 6 and b.info()["sweeps_done"] == 6
+        for x, y in zip((*a.factors(), a.trace(), a.residual()), (*b.factors(), b.trace(), b.residual())):
+            assert np.array_equal(x, y)
+        print("order %d K=%d: one sweep %.3f ms, stopped after one %.3f ms" % (order, K, ms[a], ms[b]))
+        if K == 1:
+            assert ms[b] <= 2.0 * ms[a]      # queued launches that return at once; 2.6 and 3.0 with the passes

@@ -51,6 +51,9 @@ CPU_SAMPLE_COLS = {"planted_exp_5000x200000_k50": 1000, "image_like_784x70000_k1
                    "salt_10000x500000_k100": 250, "planted_uniform_200x1000_k10": 1000}
 CPU_SAMPLE_SWEEPS = 3
 
+# did_info.sweep_form (DID_FORM_*)
+FORM_WRITING, FORM_RESIDENT, FORM_READ_ONLY, FORM_BATCHED = 0, 1, 2, 3
+
 SWEEP_SOURCES = ["paper_1802_08938_gb300/csrc/did_sweep.cu", "paper_1802_08938_gb300/csrc/did_sweep_kernel.cuh",
                  "paper_1802_08938_gb300/csrc/did_internal.cuh", "paper_1802_08938_gb300/csrc/did_defer.cu",
                  "paper_1802_08938_gb300/csrc/did_defer_kernel.cuh", "paper_1802_08938_gb300/csrc/did_refresh_tc.cu"]
@@ -258,8 +261,8 @@ def workload_run(did, name, precision, sweeps, warmup, stream, tol=0.0, max_swee
     i1 = c.info()
     ms = e0.elapsed_time(e1)
     kms = i1["sweep_kernel_ms"] - i0["sweep_kernel_ms"]
-    per_sweep, form = sweep_bytes(M, N, K, s_bytes)
-    alg = done * per_sweep
+    per_sweep, form = sweep_bytes(M, N, K, s_bytes, i1)
+    alg = done * per_sweep + (i1["prologue_launches"] - i0["prologue_launches"]) * M * N * s_bytes
     peak, _ = measured_peaks()
     f = c.objective()
     trace = c.trace()
@@ -323,11 +326,15 @@ def order_bench(did, X, M, N, K, w, seed, stream, order, steps, warmup, flags=0,
     f = c.objective()
     trace = c.trace()
     c.close()
-    out = {"order": order, "writeback": "eager" if flags & did.DID_FLAG_EAGER_WRITEBACK else "default",
+    form = sweep_bytes(M, N, K, 4, i1, order)[1]
+    out = {"order": order, "writeback": form,
            "inner": list(inner), "trace": [float(v) for v in trace],
            "value": steps / (ms / 1000.0), "unit": "sweeps/s", "ms_per_sweep": ms / steps,
            "objective_after": f, "sweeps": warmup + steps,
-           "sweep_ms": (i1["sweep_kernel_ms"] - i0["sweep_kernel_ms"]) / steps}
+           "sweep_ms": (i1["sweep_kernel_ms"] - i0["sweep_kernel_ms"]) / steps,
+           "gpu_launches": sweep_launches(form, K, 4, order, steps, i1["sweep_launches"] - i0["sweep_launches"],
+                                          i1["tc_refreshes"] - i0["tc_refreshes"],
+                                          i1["dense_launches"] - i0["dense_launches"])}
     if order == "did_batched":
         out["roofline"] = batched_roofline(M, N, K, out["sweep_ms"])
     return out
@@ -365,42 +372,38 @@ def sweep_passes(K, lazy):
     return 2 * K - (K // 2 if lazy else 0)
 
 
-def c_first_block(M, s_bytes):
-    """k served by one pass of the C-first order's read-only sweep."""
-    vr = 16 // s_bytes
-    ld = (M + 15) // 16 * 16
-    gs = 32
-    while gs < 512 and gs * 16 < ld:
-        gs *= 2
-    rows = vr * max(1, -(-(ld // vr) // gs))
-    return 4 if rows <= 16 else 2 if rows <= 32 else 1
-
-
-def sweep_bytes(M, N, K, s_bytes, order="interleaved", eager=False, lazy=1):
-    """(bytes a sweep moves, how) of the per-k orders.  By default sweeps only
-    read R -- K times, or 2 K / (k a pass serves) times in the C-first order --
-    and form it anew from X at their end (read X, write R; a float32 residual
-    with K > 64 takes one more pass for the first partials).  With one write per
-    k: sweep_passes, or 4 K in the C-first order.  A residual that fits the SMs'
-    shared memory is read and written once a call."""
+def sweep_bytes(M, N, K, s_bytes, info, order="interleaved"):
+    """(bytes a sweep moves, how), by the form that the context's sweeps run in.
+    Read-only: R is read K times, or 2 K / (k a pass serves) times in the C-first
+    order, and formed anew from X at the end (read X, write R; a float32
+    residual with K > 64 takes one more pass for the first partials).  Writing:
+    sweep_passes, or 4 K in the C-first order.  Resident: R is read and written
+    once a call.  Batched: three passes."""
     mn = float(M) * N
-    if eager:
-        return (sweep_passes(K, 0) if order == "interleaved" else 4 * K) * mn * s_bytes, "eager"
-    if mn * 4 <= 30e6:
+    form = info["sweep_form"]
+    if form == FORM_BATCHED:
+        return 3 * mn * s_bytes, "batched"
+    if form == FORM_RESIDENT:
         return 2 * mn * s_bytes, "resident"
+    if form == FORM_READ_ONLY:
+        passes = K if order == "interleaved" else 2 * -(-K // info["pass_blocks"])
+        if order == "interleaved" and s_bytes == 4 and K > 64:
+            passes += 1
+        return passes * mn * s_bytes + mn * (4 + s_bytes), "read-only"
     if order == "interleaved":
-        return (K + (1 if s_bytes == 4 and K > 64 else 0)) * mn * s_bytes + mn * (4 + s_bytes), "read-only"
-    return 2 * -(-K // c_first_block(M, s_bytes)) * mn * s_bytes + mn * (4 + s_bytes), "read-only"
+        return sweep_passes(K, info["lazy_writeback"]) * mn * s_bytes, "deferred" if info["lazy_writeback"] else "eager"
+    return 4 * K * mn * s_bytes, "eager"
 
 
 def sweep_launches(form, K, s_bytes, order, sweeps, launches, tc, dense):
     """Kernel launches of `sweeps` sweeps, from the counters.  A read-only sweep is
     its kernel (two in the C-first order), the refresh (two operand splits and
     the GEMM, or the float32 pass) and a closing kernel, and the counted
-    refreshes are those; else each tensor-core refresh is three launches."""
+    refreshes are those; else each tensor-core refresh is three launches.  A
+    batched sweep is eight kernels."""
     if form == "read-only":
         return int(sweeps * ((1 if order == "interleaved" else 2) + (1 if s_bytes == 4 and K > 64 else 3) + 1))
-    return int(launches + dense + 3 * tc)
+    return int((8 if form == "batched" else 1) * launches + dense + 3 * tc)
 
 
 def max_over_ranks(x, ws):
@@ -582,10 +585,8 @@ def main():
     launches = info1["sweep_launches"] - info0["sweep_launches"]
     prologues = info1["prologue_launches"] - info0["prologue_launches"]
     kms = info1["sweep_kernel_ms"] - info0["sweep_kernel_ms"]
-    eager = bool(flags & did.DID_FLAG_EAGER_WRITEBACK)
-    per_sweep, form = ((3.0 * M * N * s_bytes, "batched") if args.order == "did_batched" else
-                       sweep_bytes(M, N, K, s_bytes, args.order, eager))
-    alg_bytes = args.steps * per_sweep + (prologues * 1.0 * M * N * s_bytes if eager else 0.0)
+    per_sweep, form = sweep_bytes(M, N, K, s_bytes, info1, args.order)
+    alg_bytes = args.steps * per_sweep + prologues * 1.0 * M * N * s_bytes
     achieved = alg_bytes / (kms / 1000.0) / 1e9
     peak, peak_kind = measured_peaks()
     traffic = profiled_traffic(args.workload, args.precision)
@@ -628,16 +629,17 @@ def main():
         i1 = c16.info()
         ms16 = e0.elapsed_time(e1)
         kms16 = i1["sweep_kernel_ms"] - i0["sweep_kernel_ms"]
-        ab16 = args.steps * sweep_bytes(M, N, K, 2)[0]
+        per16, form16 = sweep_bytes(M, N, K, 2, i1)
+        ab16 = args.steps * per16 + (i1["prologue_launches"] - i0["prologue_launches"]) * M * N * 2.0
         f16 = c16.objective()
         c16.close()
         v16 = ws * args.steps / (ms16 / 1000.0)
-        bf16 = {"value": v16, "unit": "sweeps/s", "ratio_vs_fp32": v16 / value, "lazy": int(i1["lazy_writeback"]),
+        bf16 = {"value": v16, "unit": "sweeps/s", "ratio_vs_fp32": v16 / value, "writeback": form16,
                 "roofline_frac": ab16 / (kms16 / 1e3) / 1e9 / peak,
                 "tc_refreshes": int(i1["tc_refreshes"] - i0["tc_refreshes"]),
                 "objective_after": f16,
                 "note": "same workload and seed, R stored in bfloat16, tensor-core BF16x3 refresh"}
-        other_launches += sweep_launches(sweep_bytes(M, N, K, 2)[1], K, 2, "interleaved", args.steps, args.steps,
+        other_launches += sweep_launches(form16, K, 2, "interleaved", args.steps, args.steps,
                                          i1["tc_refreshes"] - i0["tc_refreshes"], 0)
 
     orders = None
@@ -655,8 +657,7 @@ def main():
             hit = [i for i, v in enumerate(o.pop("trace")) if v <= target]
             o["sweeps_to_plain_final"] = hit[0] if hit else None
             o["ms_to_plain_final"] = hit[0] * o["ms_per_sweep"] if hit else None
-        # the per-k orders launch one sweep kernel per sweep; the batched order 8 kernels per sweep
-        other_launches += 2 * args.steps + (3 * 8 * args.steps if batched_ok else 0)
+        other_launches += sum(o["gpu_launches"] for o in orders)
 
     e2e = None
     if not args.no_e2e:
@@ -722,7 +723,8 @@ def main():
     else:
         roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                     "frac": achieved / peak, "traffic": traffic if args.order == "interleaved" else None,
-                    "kernel": "sweep_kernel" if form == "eager" else "%s sweep and refresh" % form, "peak_kind": peak_kind,
+                    "kernel": {"resident": "resident sweep", "read-only": "read-only sweep and refresh"}.get(form, "sweep_kernel"),
+                    "peak_kind": peak_kind,
                     "alg_bytes_per_sweep": per_sweep,
                     # one read and one write of R per k; the sweep moves fewer bytes, and frac above uses those
                     "alg_bytes_per_sweep_2KMNs": 2.0 * K * M * N * s_bytes,
@@ -737,8 +739,6 @@ def main():
         eager32 = [o for o in orders if o["order"] == "interleaved" and o["writeback"] == "eager"]
         if eager32:
             bf16["ratio_vs_fp32_eager"] = bf16["value"] / eager32[0]["value"]
-        bf16.pop("lazy", 0)
-        bf16["writeback"] = sweep_bytes(M, N, K, 2)[1]
 
     if rank == 0:
         line = {

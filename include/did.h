@@ -142,6 +142,14 @@ typedef struct {
  * float32 one); the results are bitwise the same (for comparisons). */
 #define DID_FLAG_SINGLE_COLUMNS 32
 
+/* The form in which a context's sweeps run, chosen when it is created (see the
+ * flags above).
+ * DID_FORM_WRITING: the sweep kernel reads and writes R.
+ * DID_FORM_RESIDENT: R stays in the SMs' shared memory for a launch.
+ * DID_FORM_READ_ONLY: R is only read, and formed anew after each sweep.
+ * DID_FORM_BATCHED: the kernels of DID_ORDER_DID_BATCHED. */
+typedef enum { DID_FORM_WRITING = 0, DID_FORM_RESIDENT = 1, DID_FORM_READ_ONLY = 2, DID_FORM_BATCHED = 3 } did_form;
+
 typedef struct {
     int64_t M, N;
     int32_t K;
@@ -165,9 +173,12 @@ typedef struct {
     double dense_kernel_ms;
     int64_t tc_refreshes;    /* refreshes done on the tensor cores */
     double tc_refresh_ms;    /* their device time (operand split + the tensor-core pass) */
+    /* the plan of the sweep kernel, which runs in DID_FORM_WRITING */
     int32_t lazy_writeback;  /* 1: the sweep kernel defers the write of R in pairs of k */
     int32_t ring_stages;     /* shared-memory column stages per column group */
     int32_t column_pairs;    /* 1: a column group takes two columns per step of a c-pass */
+    int16_t sweep_form;      /* did_form */
+    int16_t pass_blocks;     /* DID_FORM_READ_ONLY: k that a pass over R serves, else 0 */
 } did_info;
 
 /* Fill *opt with the defaults: FP32, interleaved order, no refresh,

@@ -36,6 +36,7 @@ DID_FLAG_SIMT_REFRESH = 2
 DID_FLAG_EAGER_WRITEBACK = 8
 DID_FLAG_LAZY_WRITEBACK = 16
 DID_FLAG_SINGLE_COLUMNS = 32
+DID_FORM_WRITING, DID_FORM_RESIDENT, DID_FORM_READ_ONLY, DID_FORM_BATCHED = 0, 1, 2, 3
 
 
 class did_options(ctypes.Structure):
@@ -72,6 +73,7 @@ class did_info(ctypes.Structure):
         ("tc_refresh_ms", ctypes.c_double),
         ("lazy_writeback", ctypes.c_int32), ("ring_stages", ctypes.c_int32),
         ("column_pairs", ctypes.c_int32),
+        ("sweep_form", ctypes.c_int16), ("pass_blocks", ctypes.c_int16),
     ]
 
 

@@ -943,7 +943,7 @@ did_status did_get_info(did_ctx* c, did_info* info) {
   info->order = c->opt.order;
   info->grid_ctas = c->cfirst ? c->cplan.grid : c->resident ? c->rplan.grid : c->defer ? c->dplan.grid : c->plan.grid;
   info->group_threads = c->cfirst ? c->cplan.GS : c->defer ? c->dplan.GS : c->plan.GS;
-  info->vecs_per_thread = c->defer ? c->dplan.NR : c->plan.NR;
+  info->vecs_per_thread = c->cfirst ? c->cplan.NR : c->defer ? c->dplan.NR : c->plan.NR;
   info->column_units = c->cfirst ? c->cplan.nunits : c->defer ? c->dplan.nunits : c->plan.nunits;
   info->dynamic_units = c->cfirst ? c->cplan.dynamic : c->defer ? c->dplan.dynamic : c->plan.dynamic;
   info->ld = c->ld;
@@ -967,6 +967,9 @@ did_status did_get_info(did_ctx* c, did_info* info) {
   info->ring_stages = c->plan.D;
   info->column_pairs =
       c->opt.order == DID_ORDER_INTERLEAVED && !(c->opt.flags & DID_FLAG_SINGLE_COLUMNS) ? c->plan.pair : 0;
+  info->sweep_form = c->batched ? DID_FORM_BATCHED : c->resident ? DID_FORM_RESIDENT
+                     : c->defer || c->cfirst ? DID_FORM_READ_ONLY : DID_FORM_WRITING;
+  info->pass_blocks = c->cfirst ? c->cplan.KB : c->defer ? 1 : 0;
   return DID_OK;
 }
 

@@ -70,6 +70,7 @@ bool plan_cfirst(int ld, int64_t N, int K, bool bf16, CfirstPlan* plan) {
   const int NR = std::max(1, (nvec + P.GS - 1) / P.GS);
   if (NR > (bf16 ? 4 : 6)) return false;
   P.NG = kWorkThreads / P.GS;
+  P.NR = NR;
   P.KB = block_of(NR, bf16);
   const size_t budget = (size_t)optin - 1024;
   int CW = 0;

@@ -389,7 +389,7 @@ cudaError_t launch_defer_close(const double* part, int n, int stride, Ctrl* ctrl
 // The same for the C-first order (did_cfirst_kernel.cuh): a pass over R serves
 // KB of the K dots (C step) or partials (B step).
 struct CfirstPlan {
-  int grid, GS, NG, CW, S, KB;
+  int grid, GS, NG, NR, CW, S, KB;
   Units units;
   int nunits, dynamic, npart;
   size_t csmem, bsmem;

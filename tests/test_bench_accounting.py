@@ -60,6 +60,32 @@ def test_batched_flops_lead_term():
     assert 8 * K * M * N <= f <= 8 * K * M * N * 1.05
 
 
+@pytest.mark.parametrize("order,s_bytes,info,passes,how", [
+    ("interleaved", 4, dict(sweep_form=0, lazy_writeback=1, pass_blocks=0), 75, "deferred"),
+    ("interleaved", 4, dict(sweep_form=0, lazy_writeback=0, pass_blocks=0), 100, "eager"),
+    ("interleaved", 2, dict(sweep_form=1, lazy_writeback=0, pass_blocks=0), 2, "resident"),
+    ("interleaved", 4, dict(sweep_form=2, lazy_writeback=1, pass_blocks=1), 52, "read-only"),     # 50, X read, R written
+    ("interleaved", 2, dict(sweep_form=2, lazy_writeback=0, pass_blocks=1), 53, "read-only"),     # X is twice R's bytes
+    ("did", 4, dict(sweep_form=2, lazy_writeback=1, pass_blocks=4), 28, "read-only"),             # 2 x 13 passes
+    ("did", 4, dict(sweep_form=0, lazy_writeback=1, pass_blocks=0), 200, "eager"),
+    ("did_batched", 4, dict(sweep_form=3, lazy_writeback=1, pass_blocks=0), 3, "batched"),
+])
+def test_sweep_bytes_follow_the_form(order, s_bytes, info, passes, how):
+    """The bytes of a sweep follow the form that did_info reports, not the sizes."""
+    M, N, K = 5000, 200000, 50
+    assert bench.sweep_bytes(M, N, K, s_bytes, info, order) == (passes * M * N * s_bytes, how)
+
+
+def test_read_only_sweep_of_more_than_64_float32_blocks():
+    # no tensor-core refresh, so a pass more for R c_1^T, and a sweep is three launches instead of five
+    info = dict(sweep_form=2, lazy_writeback=0, pass_blocks=1)
+    assert bench.sweep_bytes(1000, 100000, 100, 4, info) == (103 * 1000 * 100000 * 4, "read-only")
+    assert bench.sweep_launches("read-only", 100, 4, "interleaved", 2, 2, 0, 0) == 6
+    assert bench.sweep_launches("read-only", 50, 4, "interleaved", 2, 2, 2, 0) == 10
+    assert bench.sweep_launches("read-only", 50, 4, "did", 2, 2, 2, 0) == 12
+    assert bench.sweep_launches("batched", 50, 4, "did_batched", 2, 2, 1, 0) == 19
+
+
 def test_peaks_are_the_measured_file():
     p = os.path.join(os.path.dirname(bench.__file__), "MEASURED_PEAKS.json")
     peak, kind = bench.measured_peaks()

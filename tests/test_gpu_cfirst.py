@@ -35,7 +35,7 @@ def run(did, X, B0, C0, sweeps, **kw):
 
 
 SHAPES = [(64, 150001, 7), (130, 70003, 4), (784, 12001, 5), (1030, 9001, 1), (2064, 4503, 9), (5003, 1999, 3),
-          (9000, 1051, 6), (12000, 801, 3), (600, 16001, 66)]
+          (9000, 1051, 6), (12000, 801, 3), (600, 16001, 66), (520, 20011, 128)]
 
 
 @pytest.mark.parametrize("M,N,K", SHAPES)
@@ -44,6 +44,9 @@ def test_float32_matches_oracle(did, M, N, K):
     B0, C0 = W.init_factors(M, N, K, 5)
     ref = O.factor(X, B0, C0, order="dbcd", max_iter=3, stop="none")
     got = run(did, X, B0, C0, 3)
+    rows = 4 * got["info"]["vecs_per_thread"]
+    assert got["info"]["sweep_form"] == did.DID_FORM_READ_ONLY
+    assert got["info"]["pass_blocks"] == (4 if rows <= 16 else 2)
     again = run(did, X, B0, C0, 3)
     eager = run(did, X, B0, C0, 3, flags=did.DID_FLAG_EAGER_WRITEBACK)
     eB, eC = rel(got["B"], ref["B"]), rel(got["C"], ref["C"])
@@ -65,7 +68,12 @@ def test_bfloat16_residual(did, M, N, K):
     B0, C0 = W.init_factors(M, N, K, 5)
     ref = O.factor(X, B0, C0, order="dbcd", max_iter=3, stop="none")
     got = run(did, X, B0, C0, 3, precision=did.DID_BF16R, refresh_every=2)
+    assert got["info"]["sweep_form"] == did.DID_FORM_READ_ONLY
     assert got["info"]["refreshes"] == 1
+    eB, eC = rel(got["B"], ref["B"]), rel(got["C"], ref["C"])
+    print("C-first read-only bfloat16 M=%d N=%d K=%d: relB %.3g relC %.3g" % (M, N, K, eB, eC))
+    # R is rounded by up to 2^-9 of an entry once a sweep; a contraction carries at most that share of |R| |b|
+    assert eB <= 3 * 2.0 ** -9 and eC <= 3 * 2.0 ** -9
     assert abs(got["f"] - ref["trace"][-1]) <= 1e-3 * ref["trace"][-1]
 
 

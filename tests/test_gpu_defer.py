@@ -38,8 +38,8 @@ def run(did, X, B0, C0, sweeps, **kw):
 
 
 SHAPES = [(64, 150001, 16), (130, 70003, 7), (784, 12001, 5), (1030, 9001, 2), (2064, 4503, 9), (5003, 1999, 3),
-          (9000, 1051, 1), (12000, 801, 4), (18001, 541, 2),
-          (600, 16001, 65), (1100, 9005, 101)]
+          (9000, 1051, 1), (12000, 801, 4), (14001, 641, 2), (16001, 601, 3), (17001, 541, 2),
+          (600, 16001, 65), (1100, 9005, 101), (520, 20011, 128)]
 
 
 @pytest.mark.parametrize("M,N,K", SHAPES)
@@ -48,6 +48,7 @@ def test_float32_matches_oracle(did, M, N, K):
     B0, C0 = W.init_factors(M, N, K, 5)
     ref = O.factor(X, B0, C0, order="hals", max_iter=3, stop="none")
     got = run(did, X, B0, C0, 3)
+    assert got["info"]["sweep_form"] == did.DID_FORM_READ_ONLY and got["info"]["pass_blocks"] == 1
     again = run(did, X, B0, C0, 3)
     eager = run(did, X, B0, C0, 3, flags=did.DID_FLAG_EAGER_WRITEBACK)
     eB, eC = rel(got["B"], ref["B"]), rel(got["C"], ref["C"])
@@ -64,13 +65,31 @@ def test_float32_matches_oracle(did, M, N, K):
     assert np.all(np.abs(got["R"] - Rd) <= 2.0 ** -17 * S + 2.0 ** -22 * np.abs(Rd) + 1e-6)
 
 
-@pytest.mark.parametrize("M,N,K", [(130, 70003, 7), (784, 12001, 20), (2064, 4503, 9), (9000, 1051, 70)])
+@pytest.mark.parametrize("M,N,K", [(18001, 541, 2), (600, 16001, 129), (120, 70003, 33)])
+def test_shapes_that_keep_the_kernel_that_writes_r(did, M, N, K):
+    """Columns of which the ring holds no three, more than 128 blocks, and
+    blocks too many for their column: the general kernel, without a flag."""
+    X, _, _ = W.planted(M, N, K, seed=M + N, sigma=0.05)
+    B0, C0 = W.init_factors(M, N, K, 5)
+    ref = O.factor(X, B0, C0, order="hals", max_iter=2, stop="none")
+    got = run(did, X, B0, C0, 2)
+    assert got["info"]["sweep_form"] == did.DID_FORM_WRITING and got["info"]["pass_blocks"] == 0
+    assert rel(got["B"], ref["B"]) <= 1e-5 and rel(got["C"], ref["C"]) <= 1e-5
+
+
+@pytest.mark.parametrize("M,N,K", [(130, 70003, 7), (784, 12001, 20), (2064, 4503, 9), (9000, 1051, 70), (16001, 601, 4),
+                                   (17001, 541, 3), (520, 20011, 128)])
 def test_bfloat16_residual(did, M, N, K):
     X, _, _ = W.planted(M, N, K, seed=M + N, sigma=0.05)
     B0, C0 = W.init_factors(M, N, K, 5)
     ref = O.factor(X, B0, C0, order="hals", max_iter=3, stop="none")
     got = run(did, X, B0, C0, 3, precision=did.DID_BF16R, refresh_every=2)
+    assert got["info"]["sweep_form"] == did.DID_FORM_READ_ONLY
     assert got["info"]["refreshes"] == 1
+    eB, eC = rel(got["B"], ref["B"]), rel(got["C"], ref["C"])
+    print("read-only bfloat16 M=%d N=%d K=%d: relB %.3g relC %.3g" % (M, N, K, eB, eC))
+    # R is rounded by up to 2^-9 of an entry once a sweep; a contraction carries at most that share of |R| |c|
+    assert eB <= 3 * 2.0 ** -9 and eC <= 3 * 2.0 ** -9
     assert abs(got["f"] - ref["trace"][-1]) <= 1e-3 * ref["trace"][-1]
 
 
@@ -82,6 +101,7 @@ def test_stopping_zero_norms_and_resume(did):
     ref = O.factor(X, B0, C0, order="hals", max_iter=60, tol=1e-2, stop="relchange")
     Xc = np.ascontiguousarray(X.T)
     with did.Context(Xc, M, N, K, B_init=np.ascontiguousarray(B0.T), C_init=C0) as ctx:
+        assert ctx.info()["sweep_form"] == did.DID_FORM_READ_ONLY
         iters, f = ctx.factor(60, 1e-2)
         B, C = ctx.factors()
         assert iters == ref["iters"] and ctx.info()["degenerate_events"] >= 1
@@ -116,6 +136,8 @@ def test_few_ctas(did, M, N, K, grid):
     ref = O.factor(X, B0, C0, order="hals", max_iter=3, stop="none")
     got = run(did, X, B0, C0, 3, grid_ctas=grid)
     assert got["info"]["grid_ctas"] == grid
+    rows = -(-((M + 15) // 16 * 16) // grid)
+    assert got["info"]["sweep_form"] == (did.DID_FORM_READ_ONLY if rows <= 2048 else did.DID_FORM_WRITING)
     eB, eC = rel(got["B"], ref["B"]), rel(got["C"], ref["C"])
     eF = float(np.max(np.abs(got["trace"] - ref["trace"]) / ref["trace"]))
     print("read-only M=%d N=%d K=%d grid=%d: relB %.3g relC %.3g relf %.3g" % (M, N, K, grid, eB, eC, eF))

@@ -45,7 +45,8 @@ def test_lazy_matches_oracle_and_eager(did, M, N, K):
     B0, C0 = W.init_factors(M, N, K, 5)
     sweeps = 20
     ref = O.factor(X, B0, C0, order="hals", max_iter=sweeps, stop="none")
-    lz = run(did, X, B0, C0, sweeps)
+    lz = run(did, X, B0, C0, sweeps, flags=did.DID_FLAG_LAZY_WRITEBACK)
+    assert lz["info"]["sweep_form"] == did.DID_FORM_WRITING
     eg = run(did, X, B0, C0, sweeps, flags=did.DID_FLAG_EAGER_WRITEBACK)
     assert lz["info"]["lazy_writeback"] == (1 if K >= 2 else lz["info"]["lazy_writeback"])
     assert eg["info"]["lazy_writeback"] == 0
@@ -54,6 +55,9 @@ def test_lazy_matches_oracle_and_eager(did, M, N, K):
     print("lazy M=%d N=%d K=%d stages=%d: relB %.3g relC %.3g max relf %.3g (eager relB %.3g)" % (
         M, N, K, lz["info"]["ring_stages"], eB, eC, eF, rel_fro(eg["B"], ref["B"])))
     assert eB <= 1e-4 and eC <= 1e-4 and eF <= 1e-5
+    assert eg["info"]["sweep_form"] == did.DID_FORM_WRITING
+    assert rel_fro(eg["B"], ref["B"]) <= 1e-4 and rel_fro(eg["C"], ref["C"]) <= 1e-4
+    assert float(np.max(np.abs(eg["trace"] - ref["trace"]) / ref["trace"])) <= 1e-5
     # every pending change reached R: the stored residual is X - B C
     Rd = X.astype(np.float64) - lz["B"].astype(np.float64) @ lz["C"].astype(np.float64)
     assert np.max(np.abs(lz["R"] - Rd)) <= 1e-4 * max(1.0, float(np.abs(X).max()))
@@ -65,8 +69,9 @@ def test_lazy_dynamic_units_and_refresh(did):
     B0, C0 = W.init_factors(M, N, K, 77)
     sweeps = 6
     ref = O.factor(X, B0, C0, order="hals", max_iter=sweeps, stop="none")
-    a = run(did, X, B0, C0, sweeps, refresh_every=4)
-    b = run(did, X, B0, C0, sweeps, refresh_every=4)
+    a = run(did, X, B0, C0, sweeps, refresh_every=4, flags=did.DID_FLAG_LAZY_WRITEBACK)
+    b = run(did, X, B0, C0, sweeps, refresh_every=4, flags=did.DID_FLAG_LAZY_WRITEBACK)
+    assert a["info"]["sweep_form"] == did.DID_FORM_WRITING
     assert a["info"]["lazy_writeback"] == 1 and a["info"]["dynamic_units"] == 1
     assert np.array_equal(a["B"], b["B"]) and np.array_equal(a["C"], b["C"])   # bitwise deterministic
     eF = float(np.max(np.abs(a["trace"] - ref["trace"]) / ref["trace"]))
@@ -83,7 +88,7 @@ def test_lazy_bf16_residual(did, K):
     sweeps = 15
     ref = O.factor(X, B0, C0, order="hals", max_iter=sweeps, stop="none")
     lz = run(did, X, B0, C0, sweeps, precision=did.DID_BF16R, refresh_every=5, flags=did.DID_FLAG_LAZY_WRITEBACK)
-    eg = run(did, X, B0, C0, sweeps, precision=did.DID_BF16R, refresh_every=5)
+    eg = run(did, X, B0, C0, sweeps, precision=did.DID_BF16R, refresh_every=5, flags=did.DID_FLAG_EAGER_WRITEBACK)
     f_ref = ref["trace"][-1]
     print("bf16 lazy K=%d: f rel %.3g (eager %.3g), lazy=%d" % (
         K, abs(lz["obj"] - f_ref) / f_ref, abs(eg["obj"] - f_ref) / f_ref, lz["info"]["lazy_writeback"]))
@@ -98,9 +103,9 @@ def test_lazy_stopping_and_resume(did):
     B0, C0 = W.init_factors(M, N, K, 8)
     ref = O.factor(X, B0, C0, order="hals", max_iter=500, tol=1e-2, stop="relchange")
     with did.Context(np.ascontiguousarray(X.T), M, N, K, B_init=np.ascontiguousarray(B0.T.astype(np.float32)),
-                     C_init=np.ascontiguousarray(C0.astype(np.float32))) as ctx:
+                     C_init=np.ascontiguousarray(C0.astype(np.float32)), flags=did.DID_FLAG_LAZY_WRITEBACK) as ctx:
         iters, f = ctx.factor(500, 1e-2)
-        assert ctx.info()["lazy_writeback"] == 1
+        assert ctx.info()["lazy_writeback"] == 1 and ctx.info()["sweep_form"] == did.DID_FORM_WRITING
     print("lazy stopping: GPU %d sweeps, oracle %d" % (iters, ref["iters"]))
     assert iters == ref["iters"]
 

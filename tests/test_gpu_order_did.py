@@ -1,7 +1,8 @@
 """The C-first block order of DBCD / DID (Algorithms 2 and 3) on the GPU.
 
 The GPU runs the C step (c_1..c_K with b fixed, equations up:c) and then the
-B step (b_1..b_K, each followed by E := E - delta b_i c_i) as column passes.
+B step (b_1..b_K, each followed by E := E - delta b_i c_i), in the form that the
+residual's size asks for and, with a flag, as column passes that write R.
 It is compared with the oracle's DBCD sweep with a kept residual, which the
 oracle pins to Algorithm 3 (W, V, delta b) to 1e-12.
 """
@@ -37,13 +38,14 @@ def run(did, X, B0, C0, sweeps, **kw):
         return B, C, ctx.trace(), ctx.residual()
 
 
+@pytest.mark.parametrize("flags", ["default", "eager"])
 @pytest.mark.parametrize("M,N,K", [(200, 1000, 10), (37, 53, 3), (784, 700, 16), (2001, 311, 5), (64, 3000, 8)])
-def test_c_first_order_matches_oracle(did, M, N, K):
+def test_c_first_order_matches_oracle(did, M, N, K, flags):
     X, _, _ = W.planted(M, N, K, seed=M + 3 * N, sigma=0.01)
     B0, C0 = W.init_factors(M, N, K, 2)
     sweeps = 20 if M * N < 1e6 else 10
     ref = O.factor(X, B0, C0, order="dbcd", max_iter=sweeps, stop="none")
-    B, C, t, R = run(did, X, B0, C0, sweeps)
+    B, C, t, R = run(did, X, B0, C0, sweeps, flags=did.DID_FLAG_EAGER_WRITEBACK if flags == "eager" else 0)
     eB, eC = rel_fro(B, ref["B"]), rel_fro(C, ref["C"])
     eF = abs(t[-1] - ref["trace"][-1]) / ref["trace"][-1]
     print("C-first M=%d N=%d K=%d: relB %.3g relC %.3g relf %.3g" % (M, N, K, eB, eC, eF))
@@ -53,14 +55,16 @@ def test_c_first_order_matches_oracle(did, M, N, K):
     assert np.max(np.abs(R - Rd)) <= 1e-4 * max(1.0, np.abs(X).max())
 
 
-def test_c_first_order_large_with_units(did):
+@pytest.mark.parametrize("flags", ["default", "eager"])
+def test_c_first_order_large_with_units(did, flags):
     """Enough columns for dynamic column units; deterministic across runs."""
     M, N, K = 500, 60000, 12
     X, _, _ = W.planted(M, N, K, seed=4, sigma=0.01)
     B0, C0 = W.init_factors(M, N, K, 4)
     ref = O.factor(X, B0, C0, order="dbcd", max_iter=4, stop="none")
-    B1, C1, t1, _ = run(did, X, B0, C0, 4)
-    B2, C2, t2, _ = run(did, X, B0, C0, 4)
+    kw = dict(flags=did.DID_FLAG_EAGER_WRITEBACK if flags == "eager" else 0)
+    B1, C1, t1, _ = run(did, X, B0, C0, 4, **kw)
+    B2, C2, t2, _ = run(did, X, B0, C0, 4, **kw)
     np.testing.assert_array_equal(B1, B2)
     np.testing.assert_array_equal(t1, t2)
     assert rel_fro(B1, ref["B"]) <= 1e-4 and rel_fro(C1, ref["C"]) <= 1e-4

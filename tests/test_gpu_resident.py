@@ -29,6 +29,7 @@ def run(did, X, B0, C0, sweeps, **kw):
     M, N = X.shape
     with did.Context(np.ascontiguousarray(X.T), M, N, B0.shape[1], B_init=np.ascontiguousarray(B0.T), C_init=C0,
                      **kw) as ctx:
+        assert ctx.info()["sweep_form"] == did.DID_FORM_RESIDENT
         for n in sweeps:
             ctx.sweep(n)
         B, C = ctx.factors()
@@ -36,7 +37,7 @@ def run(did, X, B0, C0, sweeps, **kw):
 
 
 # one CTA; K = 1; more CTAs than row slices; long columns, one a CTA; a ragged last CTA; near the capacity
-SHAPES = [(5, 7, 2), (40, 16, 1), (3, 3000, 1), (200, 1000, 10), (33, 2433, 7), (4099, 150, 5), (9000, 600, 3),
+SHAPES = [(5, 7, 2), (40, 16, 1), (3, 3000, 1), (200, 1000, 10), (33, 2433, 7), (4099, 150, 5), (9000, 450, 3),
           (1024, 2414, 25), (513, 9001, 4), (2500, 2401, 6)]
 
 

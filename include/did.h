@@ -331,9 +331,11 @@ did_status did_generate_uniform(float* out_dev, int64_t n, uint64_t seed, int32_
  * on its own range of CTAs; larger ones take the whole GPU in turn (as many of
  * their sweeps a round as fit in about 20 ms, at least one); the rest, and
  * several mid-sized ones where that is faster, share one launch of the
- * multi-instance sweep kernel, with CTAs in proportion to measured CTA-seconds per sweep.  The scratch of these forms (the pending
- * factors and the refresh's operands of the largest request) is the server's, outside the
- * budget; where it cannot be had every request takes the last form.
+ * multi-instance sweep kernel, with CTAs in proportion to measured CTA-seconds
+ * per sweep.  The scratch of the first two forms (exchange words, or the pending
+ * factors and the refresh's operands of the largest request) is the server's and
+ * counts in the budget; it gives way to a request that is admitted, and a request
+ * whose form's scratch does not fit takes the last form.
  * Between rounds, finished requests are retired (B, C copied to host memory
  * owned by the server, device memory freed) and waiting ones admitted, so
  * requests arriving while others run join at the next round.  The start
@@ -369,7 +371,7 @@ typedef struct {
     int64_t submitted, completed, failed;
     double solves_per_s;     /* completed / (last completion - first submission) */
     double p50_ms, p99_ms;   /* latency t_done - t_submit of completed requests */
-    size_t peak_bytes;       /* largest device memory held for requests at once */
+    size_t peak_bytes;       /* largest device memory held for requests and their scratch at once */
     int32_t peak_active;     /* largest number of requests in one round */
     int64_t rounds;
     double busy_s;           /* device time of the rounds (CUDA events) */

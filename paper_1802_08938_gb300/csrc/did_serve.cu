@@ -17,7 +17,9 @@
 // request in the multi-instance kernel 24 requests of 20 sweeps took 488 ms;
 // see run_round for what they take now.  Between rounds finished requests are retired and new ones
 // admitted.  All device memory of a request is one stream-ordered allocation;
-// the scratch of the forms is the server's (one request or launch uses it at a time).
+// the scratch of the forms is the server's (one request or launch uses it at a
+// time), within the budget: it is given back where a request is admitted in
+// its place, and a request whose form's scratch does not fit runs PACKED.
 #include "did_internal.cuh"
 
 #include <math.h>
@@ -159,14 +161,43 @@ size_t request_bytes(const did_server* s, int64_t M, int64_t N, int K, int ld) {
 
 void choose_form(const did_server* s, Req* r);
 
+void free_scratch(did_server* s) {
+  if (s->scratch) cudaFreeAsync(s->scratch, s->stream);
+  s->scratch = nullptr;
+  s->scratch_bytes = 0;
+}
+
+// The server's scratch, at least `bytes`; false if the budget (which it shares
+// with the requests) or the device has no room for it.
+bool need_scratch(did_server* s, size_t bytes) {
+  if (bytes <= s->scratch_bytes) return true;
+  if (s->used + bytes > s->budget) return false;
+  free_scratch(s);
+  if (cudaMallocAsync(&s->scratch, bytes, s->stream) != cudaSuccess) {
+    cudaGetLastError();
+    s->scratch = nullptr;
+    return false;
+  }
+  s->scratch_bytes = bytes;
+  return true;
+}
+
 // Allocate, generate or copy X, draw the start point and form R = X - B C.
 did_status admit(did_server* s, Req* r) {
   const int64_t M = r->rq.M, N = r->rq.N;
   const int K = r->rq.K;
   const int ld = r->ld;
   cudaStream_t st = s->stream;
-  if (cudaMallocAsync(&r->block, r->bytes, st) != cudaSuccess) {
+  cudaError_t got = cudaMallocAsync(&r->block, r->bytes, st);
+  if (got != cudaSuccess && s->scratch) {     // the scratch gives way to a request
     cudaGetLastError();
+    free_scratch(s);
+    got = cudaStreamSynchronize(st);
+    if (got == cudaSuccess) got = cudaMallocAsync(&r->block, r->bytes, st);
+  }
+  if (got != cudaSuccess) {
+    cudaGetLastError();
+    r->block = nullptr;
     return DID_ENOMEM;
   }
   unsigned char* p = static_cast<unsigned char*>(r->block);
@@ -297,21 +328,6 @@ void choose_form(const did_server* s, Req* r) {
   } else if (r->ld >= 4 * K && did::plan_defer(r->ld, N, K, s->bf16, 0, &r->dplan)) {
     r->form = DEFER;
   }
-}
-
-// The server's scratch, at least `bytes`; false if the memory is not there.
-bool need_scratch(did_server* s, size_t bytes) {
-  if (bytes <= s->scratch_bytes) return true;
-  if (s->scratch) cudaFreeAsync(s->scratch, s->stream);
-  s->scratch = nullptr;
-  s->scratch_bytes = 0;
-  if (cudaMallocAsync(&s->scratch, bytes, s->stream) != cudaSuccess) {
-    cudaGetLastError();
-    s->scratch = nullptr;
-    return false;
-  }
-  s->scratch_bytes = bytes;
-  return true;
 }
 
 // Buffers of a read-only sweep of r in the scratch (or, with base null, their size).
@@ -537,10 +553,28 @@ bool run_round(did_server* s, std::vector<Req*>& act) {
   for (int i = 0; i < n; ++i) (act[i]->form == RESIDENT ? res : act[i]->form == DEFER ? def : packed).push_back(i);
   pack_mid_sized(s, act, &def, &packed);
   std::vector<Bin> bins = pack(s, act, res);
+  // Requests whose form's scratch has no room in the budget beside the requests run PACKED.
+  const size_t room = s->budget - s->used;
   size_t scratch = 0;
-  for (const Bin& b : bins) scratch = std::max(scratch, b.words);
-  for (int i : def) scratch = std::max(scratch, defer_scratch(s, act[i], nullptr).bytes);
-  if (!need_scratch(s, scratch)) {       // no room beside the requests: all in the multi-instance kernel
+  for (size_t q = 0; q < bins.size();) {
+    if (bins[q].words > room) {
+      packed.insert(packed.end(), bins[q].slots.begin(), bins[q].slots.end());
+      bins.erase(bins.begin() + q);
+    } else {
+      scratch = std::max(scratch, bins[q++].words);
+    }
+  }
+  for (size_t q = 0; q < def.size();) {
+    const size_t need = defer_scratch(s, act[def[q]], nullptr).bytes;
+    if (need > room) {
+      packed.push_back(def[q]);
+      def.erase(def.begin() + q);
+    } else {
+      scratch = std::max(scratch, need);
+      ++q;
+    }
+  }
+  if (!need_scratch(s, scratch)) {       // no such memory on the device: all of them
     packed.resize(n);
     for (int i = 0; i < n; ++i) packed[i] = i;
     bins.clear();
@@ -654,7 +688,8 @@ void worker_main(did_server* s) {
       s->queue.pop_front();
       s->used += r->bytes;
       r->reserved = true;
-      s->peak = std::max(s->peak, s->used);
+      if (s->used + s->scratch_bytes > s->budget) free_scratch(s);   // a round asks for what then fits
+      s->peak = std::max(s->peak, s->used + s->scratch_bytes);
       r->t_start = now_s(s->t0);
       lk.unlock();
       const did_status st = admit(s, r);
@@ -680,6 +715,7 @@ void worker_main(did_server* s) {
     lk.unlock();
     const bool ok = run_round(s, act);
     lk.lock();
+    s->peak = std::max(s->peak, s->used + s->scratch_bytes);
     const double t = now_s(s->t0);
     std::vector<Req*> still;
     for (int i = 0; i < (int)act.size(); ++i) {
@@ -900,7 +936,7 @@ void did_server_destroy(did_server* s) {
     s->cv_work.notify_all();
   }
   if (s->worker.joinable()) s->worker.join();
-  if (s->scratch) cudaFreeAsync(s->scratch, s->stream);
+  free_scratch(s);
   if (s->stream) cudaStreamSynchronize(s->stream);
   cudaFree(s->d_res);
   cudaFreeHost(s->h_res);

@@ -144,7 +144,8 @@ __global__ void __launch_bounds__(kDenseThreads) dense_kernel(DenseTileArgs t) {
 // a thread 32 packed FMAs (f32x2) and four 16-byte loads from shared memory,
 // where the 4 x 4 tile above pays five loads for 16 FMAs, and its float64 sums
 // (float64 adds issue at 1/64 the rate) took a third of the time; here the
-// sums are float32 pairs until the end.  The next chunk of B and C is loaded into
+// sums (each of four squares in float32, as there) are float32 pairs of about
+// 48 bits until the end.  The next chunk of B and C is loaded into
 // registers while this one is used.  Each product is the same chain of FMAs in k
 // order, so R comes out bit for bit the same.  Measured: 10000 x 100000,
 // K = 100 (exact objective) 11.9 -> 5.9 ms; 8165 x 18821, K = 100, a refresh or an
@@ -163,6 +164,7 @@ struct Pair2 {
   }
 };
 
+template <int MODE>
 __global__ void __launch_bounds__(kBigThreads, 2) dense_big_kernel(DenseArgs a) {
   __shared__ __align__(16) float Bs[2][kBigKc][kBig];
   __shared__ __align__(16) float Cs[2][kBigKc][kBig];
@@ -240,9 +242,9 @@ __global__ void __launch_bounds__(kBigThreads, 2) dense_big_kernel(DenseArgs a) 
     for (int c = 0; c < 8; ++c) {
       const int64_t col = col0 + (c < 4 ? 4 * tc + c : 64 + 4 * tc + c - 4);
       if (col >= a.N) continue;
-      float l0 = 0.f, l1 = 0.f, l2 = 0.f;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
+        float l0 = 0.f, l1 = 0.f, l2 = 0.f;
         const int row = row0 + 64 * h + 4 * tr;
         if (row >= a.ld) continue;                  // (ld is a multiple of four)
         const size_t off = (size_t)col * a.ld + row;
@@ -253,14 +255,14 @@ __global__ void __launch_bounds__(kBigThreads, 2) dense_big_kernel(DenseArgs a) 
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           r[e] = xs[e] - p[e];
-          if (a.mode == 2) {
+          if (MODE == 2) {
             l1 = fmaf(xs[e], p[e], l1);
             l2 = fmaf(p[e], p[e], l2);
           } else {
             l0 = fmaf(r[e], r[e], l0);
           }
         }
-        if (a.mode == 0) {
+        if (MODE == 0) {
           if (a.bf16) {
             __nv_bfloat162 lo = __floats2bfloat162_rn(r[0], r[1]), hi = __floats2bfloat162_rn(r[2], r[3]);
             uint2 v;
@@ -271,10 +273,13 @@ __global__ void __launch_bounds__(kBigThreads, 2) dense_big_kernel(DenseArgs a) 
             *reinterpret_cast<float4*>(reinterpret_cast<float*>(a.R) + off) = make_float4(r[0], r[1], r[2], r[3]);
           }
         }
+        if (MODE == 2) {
+          s1.add(l1);
+          s2.add(l2);
+        } else {
+          s0.add(l0);
+        }
       }
-      s0.add(l0);
-      s1.add(l1);
-      s2.add(l2);
     }
   }
   const double d0 = block_sum_f64((double)s0.h + (double)s0.l, scratch);
@@ -408,7 +413,12 @@ cudaError_t launch_dense(const DenseArgs& a, cudaStream_t s) {
   // ld; below that the small ones keep more CTAs busy.
   const int64_t big = (int64_t)((a.ld + kBig - 1) / kBig) * ((a.N + kBig - 1) / kBig);
   if (big >= dense_grid() / 4 && (a.ld + kBig - 1) / kBig * kBig * 3 <= a.ld * 4) {
-    dense_big_kernel<<<dense_grid(), kBigThreads, 0, s>>>(a);
+    if (a.mode == 0)
+      dense_big_kernel<0><<<dense_grid(), kBigThreads, 0, s>>>(a);
+    else if (a.mode == 1)
+      dense_big_kernel<1><<<dense_grid(), kBigThreads, 0, s>>>(a);
+    else
+      dense_big_kernel<2><<<dense_grid(), kBigThreads, 0, s>>>(a);
     return cudaGetLastError();
   }
   DenseTileArgs t{};

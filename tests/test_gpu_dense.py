@@ -48,3 +48,21 @@ def test_residual_copies(did, M, N, precision):
     got = buf.cpu().numpy()
     assert got[0] == 7.0 and got[-1] == 7.0
     assert np.array_equal(got[1:-1].reshape(N, M), np.asarray(host).T)
+
+
+@pytest.mark.parametrize("M,N", [(1024, 4001), (700, 6007)])
+def test_objective_sums_four_squares_in_float32(did, M, N):
+    """Rows 10^4 times the others where a thread of the 128 x 128 tile has its
+    first: only the three squares added to a large one in float32 may be lost
+    in it (1.2e-8 of f), not all seven of the thread's rows (2.9e-8)."""
+    rng = np.random.default_rng(M)
+    Xt = rng.random((N, M)).astype(np.float32)
+    rows = np.arange(M)
+    large = (rows % 128 < 64) & (rows % 4 == 0)
+    Xt[:, large] = (1e4 * (0.8 + 0.2 * rng.random((N, int(large.sum()))))).astype(np.float32)
+    with did.Context(Xt, M, N, 1, B_init=np.zeros((1, M), np.float32), C_init=np.zeros((1, N), np.float32),
+                     flags=did.DID_FLAG_SIMT_REFRESH) as ctx:
+        f0, f = ctx.trace()[0], ctx.objective()
+    fd = 0.5 * float(np.sum(Xt.astype(np.float64) ** 2))
+    print("M=%d N=%d: %.3g %.3g" % (M, N, abs(f - fd) / fd, abs(f0 - fd) / fd))
+    assert abs(f - fd) <= 2e-8 * fd and abs(f0 - fd) <= 2e-8 * fd

@@ -56,6 +56,13 @@ __device__ __forceinline__ pf pf_fma(float x, float y, pf acc) {
   const float p = __fmul_rn(x, y);
   return pf_add(acc, pf{p, __fmaf_rn(x, y, -p)});
 }
+// acc + v, the compensation collected without renormalising (running sums).
+__device__ __forceinline__ void pf_acc(pf& a, float v) {
+  const float s = __fadd_rn(a.h, v);
+  const float t = __fsub_rn(s, a.h);
+  a.l = __fadd_rn(a.l, __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(v, t)));
+  a.h = s;
+}
 __device__ __forceinline__ pf pf_shfl(pf a, int m) {
   return pf{__shfl_xor_sync(0xffffffffu, a.h, m), __shfl_xor_sync(0xffffffffu, a.l, m)};
 }
@@ -383,7 +390,8 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
     for (int r = parts > 1 ? t - part * ld : t; r < ld; r += kResThreads) {
       const float x = bo[r], y = -bn[r];
       float* Rr = R + (size_t)clo * ld + r;
-      float p = 0.f, q = 0.f;
+      float p = 0.f;
+      pf q = pf{0.f, 0.f};                         // squares, four at a time
       int c = clo;
       for (; c + 4 <= chi; c += 4) {
         const float4 c0 = *reinterpret_cast<const float4*>(cold + c), c1 = *reinterpret_cast<const float4*>(cnew + c);
@@ -402,20 +410,20 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
         p = fmaf(v1, c2.y, p);
         p = fmaf(v2, c2.z, p);
         p = fmaf(v3, c2.w, p);
-        if (obj) q = fmaf(v0, v0, fmaf(v1, v1, fmaf(v2, v2, fmaf(v3, v3, q))));
+        if (obj) pf_acc(q, fmaf(v0, v0, fmaf(v1, v1, fmaf(v2, v2, v3 * v3))));
       }
       for (; c < chi; ++c, Rr += ld) {
         const float v = fmaf(x, cold[c], fmaf(y, cnew[c], *Rr));
         *Rr = v;
         p = fmaf(v, cx[c], p);
-        if (obj) q = fmaf(v, v, q);
+        if (obj) pf_acc(q, v * v);
       }
       if (parts > 1) {
         if (part < parts) ps[t] = p;               // ps[part * ld + r]
       } else if (send) {
         st_word(mine + r, p, s);
       }
-      if (obj) r2 = pf_add(r2, pf{q, 0.f});
+      if (obj) r2 = pf_add(r2, q);
     }
     if (parts > 1 && send) {
       __syncthreads();
@@ -491,7 +499,6 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
 
   const bool inter = a.order != DID_ORDER_DID;
   if (!dead && inter) send_first(step + 1);
-  int done = 0;
   for (int s = 0; s < a.n_sweeps && !dead; ++s) {
     pf r2 = pf{0.f, 0.f};
     if (!inter) {
@@ -611,7 +618,6 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
       }
       f_prev = f;
     }
-    ++done;
     if (stop) {
       if (cta == 0 && t == 0) a.ctrl->stopped = 1;
       break;
@@ -631,7 +637,6 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
     const int k = i / nrows, r = i - k * nrows;
     a.B[(size_t)k * ld + r0 + r] = brow[k * rpc + r];
   }
-  (void)done;
 }
 
 __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs a) {

@@ -122,3 +122,25 @@ def test_static_call_takes_it(did):
         did.did_sweep_static(R, ld, B, C, M, N, K, n)
     assert rel(B[:, :M].cpu().numpy().T, ref["B"]) <= 1e-5 and rel(C.cpu().numpy(), ref["C"]) <= 1e-5
     assert float(R[:, M:].abs().max()) == 0.0
+
+
+@pytest.mark.parametrize("M,N", [(200, 30001), (530, 9001), (16, 100003)])
+def test_objective_of_large_and_small_columns(did, M, N):
+    """1/2 ||R||^2 where the first column of each CTA's range is far larger than
+    the others: squares are added four columns at a time in float32 and then as
+    pairs.  (One float32 chain over a CTA's columns was 2.4e-8 to 1.1e-7 off.)"""
+    rng = np.random.default_rng(M)
+    Xt = rng.random((N, M)).astype(np.float32)
+    with did.Context(Xt, M, N, 1, seed=1) as ctx:
+        nc = -(-N // ctx.info()["grid_ctas"])
+    Xt[::nc] = (1e4 * (0.9 + 0.1 * rng.random(Xt[::nc].shape))).astype(np.float32)
+    with did.Context(Xt, M, N, 1, B_init=np.full((1, M), 1e-3, np.float32), C_init=np.full((1, N), 1e-3, np.float32),
+                     grid_ctas=0) as ctx:
+        assert ctx.info()["sweep_form"] == did.DID_FORM_RESIDENT and -(-N // ctx.info()["grid_ctas"]) == nc
+        ctx.sweep(1)
+        f, R = ctx.trace()[-1], ctx.residual().astype(np.float64)
+    fd = 0.5 * float(np.sum(R * R))
+    print("M=%d N=%d nc=%d: %.3g" % (M, N, nc, abs(f - fd) / fd))
+    # four roundings of up to 2^-24 of a thread's four squares, of random sign: over some 10^4 groups of
+    # large entries that is about 2^-24 / 100
+    assert abs(f - fd) <= 1e-8 * fd

@@ -186,3 +186,50 @@ def test_stop_ends_the_queued_sweeps(did, order, K):
         print("order %d K=%d: one sweep %.3f ms, stopped after one %.3f ms" % (order, K, ms[a], ms[b]))
         if K == 1:
             assert ms[b] <= 2.0 * ms[a]      # queued launches that return at once; 2.6 and 3.0 with the passes
+
+
+@pytest.mark.parametrize("order", [0, 1])
+@pytest.mark.parametrize("precision,share", [(0, 2.0 ** -42), (1, 2.0 ** -32)])
+def test_exact_fit_settles_at_the_refresh_error(did, order, precision, share):
+    """A noise-free rank-one matrix.  R is formed anew in each sweep, so f settles
+    where the refresh's error leaves it: 2^-21 of |B||C| an entry (2^-16 for a
+    bfloat16 residual), squared and halved."""
+    M, N = 800, 12003
+    X, _, _ = W.planted(M, N, 1, seed=3, sigma=0.0)
+    xx = float(np.sum(X.astype(np.float64) ** 2))
+    with did.Context(np.ascontiguousarray(X.T), M, N, 1, seed=1, order=order, precision=precision) as ctx:
+        assert ctx.info()["sweep_form"] == did.DID_FORM_READ_ONLY
+        ctx.sweep(60)
+        f, trace = ctx.objective(), ctx.trace()
+    print("exact fit order %d precision %d: f %.3g, trace %.3g of ||X||^2" % (order, precision, f / xx, trace[-1] / xx))
+    assert f <= 0.5 * share * xx and trace[-1] <= 0.5 * share * xx
+
+
+def test_no_room_for_the_scratch(did):
+    """Where the pending factors (102 MB) do not fit on the device beside X, R and
+    C, the context takes the kernel that writes R."""
+    torch = pytest.importorskip("torch")
+    M, N, K = 520, 200003, 128
+    X = torch.empty((N, M), device="cuda")
+    did.did_generate_planted(X, M, N, K, 5, sigma=0.05)
+
+    def factors(**kw):
+        with did.Context(X, M, N, K, seed=2, **kw) as ctx:
+            ctx.sweep(1)
+            i = ctx.info()
+            return (*ctx.factors(), i["sweep_form"], i["device_bytes"])
+
+    with_room = factors()
+    writing = factors(flags=did.DID_FLAG_LAZY_WRITEBACK)     # what a float32 residual runs without a flag then
+    assert with_room[2] == did.DID_FORM_READ_ONLY and with_room[3] - writing[3] >= 100 << 20
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    ballast = torch.empty(free - writing[3] - (60 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        got = factors()
+    finally:
+        del ballast
+        torch.cuda.empty_cache()
+    assert got[2] == did.DID_FORM_WRITING and got[3] < with_room[3]
+    assert np.array_equal(got[0], writing[0]) and np.array_equal(got[1], writing[1])

@@ -73,6 +73,7 @@
 // Every mbarrier wait is bounded; on expiry the kernel records the error,
 // stops issuing work, waits (bounded) for its copies and MMAs, frees its
 // tensor memory and returns; the host reads the error word after the sweeps.
+#include "did_pair.cuh"
 #include "did_tc.cuh"
 
 #include <stdio.h>
@@ -1316,24 +1317,8 @@ cudaError_t set_update_b_smem(int K) {
 // float32 pairs across threads in a fixed tree, eight entries a time (float64
 // shuffles, which issue at 1/64 the rate, took most of the former 79 us).
 constexpr int kYYThreads = 256;
-struct YYPair {
-  float h, l;
-};
-__device__ __forceinline__ YYPair yy_add(YYPair a, YYPair b) {
-  const float s = __fadd_rn(a.h, b.h);
-  const float t = __fsub_rn(s, a.h);
-  float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t));
-  e = __fadd_rn(e, __fadd_rn(a.l, b.l));
-  YYPair r;
-  r.h = __fadd_rn(s, e);
-  r.l = __fsub_rn(e, __fsub_rn(r.h, s));
-  return r;
-}
-__device__ __forceinline__ YYPair yy_shfl(YYPair a, int m) {
-  return YYPair{__shfl_xor_sync(0xffffffffu, a.h, m), __shfl_xor_sync(0xffffffffu, a.l, m)};
-}
 __global__ void __launch_bounds__(kYYThreads) yy_kernel(const float* __restrict__ Y, int ld, int K2, float* YY) {
-  __shared__ YYPair red[kYYThreads / 32][16];
+  __shared__ df red[kYYThreads / 32][16];
   const int a = blockIdx.x, b0 = blockIdx.y * 16;
   float s[16];
 #pragma unroll
@@ -1347,26 +1332,26 @@ __global__ void __launch_bounds__(kYYThreads) yy_kernel(const float* __restrict_
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
 #pragma unroll
   for (int g = 0; g < 2; ++g) {
-    YYPair v[8];
+    df v[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = YYPair{s[8 * g + q], 0.f};
+    for (int q = 0; q < 8; ++q) v[q] = df{s[8 * g + q], 0.f};
 #pragma unroll
     for (int m = 4; m >= 1; m >>= 1) {
       const bool up = (l & m) != 0;
 #pragma unroll
       for (int q = 0; q < m; ++q) {
-        const YYPair send = up ? v[q] : v[q + m], keep = up ? v[q + m] : v[q];
-        v[q] = yy_add(keep, yy_shfl(send, m));
+        const df send = up ? v[q] : v[q + m], keep = up ? v[q + m] : v[q];
+        v[q] = df_add(keep, df_shfl_xor(send, m));
       }
     }
-    v[0] = yy_add(v[0], yy_shfl(v[0], 8));
-    v[0] = yy_add(v[0], yy_shfl(v[0], 16));
+    v[0] = df_add(v[0], df_shfl_xor(v[0], 8));
+    v[0] = df_add(v[0], df_shfl_xor(v[0], 16));
     if (l < 8) red[w][8 * g + l] = v[0];           // lane l has entry l of the eight
   }
   __syncthreads();
   if (threadIdx.x < 16 && b0 + (int)threadIdx.x < K2) {
-    YYPair t = red[0][threadIdx.x];
-    for (int i = 1; i < kYYThreads / 32; ++i) t = yy_add(t, red[i][threadIdx.x]);
+    df t = red[0][threadIdx.x];
+    for (int i = 1; i < kYYThreads / 32; ++i) t = df_add(t, red[i][threadIdx.x]);
     YY[(size_t)a + (size_t)(b0 + threadIdx.x) * K2] = t.h;
   }
 }

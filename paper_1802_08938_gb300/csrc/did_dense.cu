@@ -14,6 +14,7 @@
 // blockIdx.x, blockIdx.x + grid, ... so the per-CTA partial sums, added by
 // the host in CTA order, are deterministic.
 #include "did_internal.cuh"
+#include "did_pair.cuh"
 
 #include <math.h>
 
@@ -154,16 +155,6 @@ constexpr int kBig = 128;
 constexpr int kBigKc = 16;
 constexpr int kBigThreads = 256;
 
-struct Pair2 {
-  float h, l;
-  __device__ __forceinline__ void add(float v) {
-    const float s = __fadd_rn(h, v);
-    const float t = __fsub_rn(s, h);
-    l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, t)), __fsub_rn(v, t)));
-    h = s;
-  }
-};
-
 template <int MODE>
 __global__ void __launch_bounds__(kBigThreads, 2) dense_big_kernel(DenseArgs a) {
   __shared__ __align__(16) float Bs[2][kBigKc][kBig];
@@ -178,7 +169,7 @@ __global__ void __launch_bounds__(kBigThreads, 2) dense_big_kernel(DenseArgs a) 
   const int chunks = (a.K + kBigKc - 1) / kBigKc;
   const int lk = t >> 5, lx = (t & 31) * 4;        // loader: rows lk and lk + 8 of a chunk, four values from lx
   const bool c_vec = (a.N & 3) == 0;
-  Pair2 s0{0.f, 0.f}, s1 = s0, s2 = s0;
+  df s0 = df_zero(), s1 = s0, s2 = s0;
 
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int row0 = (int)(tile % mt) * kBig;
@@ -274,10 +265,10 @@ __global__ void __launch_bounds__(kBigThreads, 2) dense_big_kernel(DenseArgs a) 
           }
         }
         if (MODE == 2) {
-          s1.add(l1);
-          s2.add(l2);
+          df_acc(s1, l1);
+          df_acc(s2, l2);
         } else {
-          s0.add(l0);
+          df_acc(s0, l0);
         }
       }
     }

@@ -341,10 +341,11 @@ struct ResidentPlan {
   size_t smem, words_bytes;
 };
 bool plan_resident(int ld, int64_t N, int K, int grid_override, ResidentPlan* plan);   // false: does not fit
-// Several instances in one launch (serving): a plan on at most `grid` CTAs each,
+// Several instances in one launch (serving): a plan on at most `grid` CTAs of `budget` bytes each,
 // their arguments (resident_args_bytes() apart; SweepArgs::cta_begin says
 // where their CTAs start, and their words are zero), one launch.
-bool plan_resident_on(int ld, int64_t N, int K, int grid, ResidentPlan* plan);
+bool plan_resident_on(size_t budget, int ld, int64_t N, int K, int grid, ResidentPlan* plan);
+size_t resident_multi_budget();   // shared memory of a CTA on the current device (0: not available)
 size_t resident_args_bytes();
 void fill_resident_args(void* dst, const ResidentPlan& plan, const SweepArgs& args, void* words, bool bf16);
 cudaError_t launch_resident_multi(const void* d_args, int ninst, int grid, size_t smem, cudaStream_t s);

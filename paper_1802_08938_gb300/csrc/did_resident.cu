@@ -28,6 +28,7 @@
 //
 // Every wait is bounded; on expiry the error word is set and all CTAs leave.
 #include "did_internal.cuh"
+#include "did_pair.cuh"
 
 #include <algorithm>
 
@@ -37,48 +38,6 @@ namespace {
 
 constexpr int kResThreads = 512;
 constexpr int kResWarps = kResThreads / 32;
-
-// Pairs of float32 (value and remainder) for the scalars.
-struct pf {
-  float h, l;
-};
-__device__ __forceinline__ pf pf_add(pf a, pf b) {
-  const float s = __fadd_rn(a.h, b.h);
-  const float t = __fsub_rn(s, a.h);
-  float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t));
-  e = __fadd_rn(e, __fadd_rn(a.l, b.l));
-  pf r;
-  r.h = __fadd_rn(s, e);
-  r.l = __fsub_rn(e, __fsub_rn(r.h, s));
-  return r;
-}
-__device__ __forceinline__ pf pf_fma(float x, float y, pf acc) {
-  const float p = __fmul_rn(x, y);
-  return pf_add(acc, pf{p, __fmaf_rn(x, y, -p)});
-}
-// acc + v, the compensation collected without renormalising (running sums).
-__device__ __forceinline__ void pf_acc(pf& a, float v) {
-  const float s = __fadd_rn(a.h, v);
-  const float t = __fsub_rn(s, a.h);
-  a.l = __fadd_rn(a.l, __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(v, t)));
-  a.h = s;
-}
-__device__ __forceinline__ pf pf_shfl(pf a, int m) {
-  return pf{__shfl_xor_sync(0xffffffffu, a.h, m), __shfl_xor_sync(0xffffffffu, a.l, m)};
-}
-__device__ __forceinline__ pf pf_warp_sum(pf a) {
-#pragma unroll
-  for (int m = 16; m >= 1; m >>= 1) a = pf_add(a, pf_shfl(a, m));
-  return a;
-}
-// a / b to about 45 bits: a float32 quotient and its correction.
-__device__ __forceinline__ pf pf_div(pf a, pf b) {
-  const float q = __fdiv_rn(a.h, b.h);
-  const float p = __fmul_rn(q, b.h);
-  const float e = __fmaf_rn(q, b.h, -p);
-  const float r = __fadd_rn(__fsub_rn(a.h, p), __fsub_rn(a.l, __fmaf_rn(q, b.l, e)));
-  return pf_add(pf{q, 0.f}, pf{__fdiv_rn(r, b.h), 0.f});
-}
 
 struct ResArgs {
   void* R;             // ld x N residual in global memory (float or bfloat16), read at the start, written at the end
@@ -177,7 +136,7 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
   float* vals = reinterpret_cast<float*>(smem + L.vals);
   float* ps = reinterpret_cast<float*>(smem + L.ps);
   float* brow = reinterpret_cast<float*>(smem + L.brow);
-  pf* red = reinterpret_cast<pf*>(smem + L.red);
+  df* red = reinterpret_cast<df*>(smem + L.red);
   volatile int* bad = reinterpret_cast<volatile int*>(smem + L.misc);
   int* err = &a.ctrl->err;
   const uint64_t tmo = a.timeout_ns;
@@ -219,9 +178,9 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
   };
   // ||c||^2 of a row on the own columns, sent for step `s` (one warp).
   auto send_cc = [&](const float* row, unsigned s) {
-    pf cc = pf{0.f, 0.f};
-    for (int c = lane; c < nc; c += 32) cc = pf_fma(row[c], row[c], cc);
-    cc = pf_warp_sum(cc);
+    df cc = df{0.f, 0.f};
+    for (int c = lane; c < nc; c += 32) cc = df_fma(row[c], row[c], cc);
+    cc = df_warp_sum(cc);
     if (lane == 0) {
       st_word(mine + ld + 2 * (s & 1), cc.h, s);
       st_word(mine + ld + 1 + 2 * (s & 1), cc.l, s);
@@ -229,8 +188,8 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
   };
   // Sum of the CTAs' words `at` and `at + 1` (a pair each) of step s, by one
   // warp; false if the wait ran out.
-  auto take_pair = [&](int at, unsigned s, pf& out) -> bool {
-    pf q = pf{0.f, 0.f};
+  auto take_pair = [&](int at, unsigned s, df& out) -> bool {
+    df q = df{0.f, 0.f};
     bool ok = true;
     for (int g = lane; g < G; g += 32) {
       uint2 x, y;
@@ -242,26 +201,26 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
         if (poll.expired(err, tmo)) { ok = false; break; }
       }
       if (!ok) break;
-      q = pf_add(q, pf{__uint_as_float(x.x), __uint_as_float(y.x)});
+      q = df_add(q, df{__uint_as_float(x.x), __uint_as_float(y.x)});
     }
     ok = __all_sync(0xffffffffu, ok);
-    out = pf_warp_sum(q);
+    out = df_warp_sum(q);
     return ok;
   };
   // Block sums of two pairs, in every thread (two barriers apart from the next use).
-  auto block_pairs = [&](pf& x, pf& y) {
+  auto block_pairs = [&](df& x, df& y) {
     // even lanes sum x, odd lanes y: one chain of additions instead of two
-    const pf send = (lane & 1) ? x : y, keep = (lane & 1) ? y : x;
-    pf v = pf_add(keep, pf_shfl(send, 1));
+    const df send = (lane & 1) ? x : y, keep = (lane & 1) ? y : x;
+    df v = df_add(keep, df_shfl_xor(send, 1));
 #pragma unroll
-    for (int m = 2; m <= 16; m <<= 1) v = pf_add(v, pf_shfl(v, m));
+    for (int m = 2; m <= 16; m <<= 1) v = df_add(v, df_shfl_xor(v, m));
     if (lane < 2) red[2 * w + lane] = v;
     __syncthreads();
     v = red[lane];                                 // warp lane / 2, x or y
 #pragma unroll
-    for (int m = 2; m <= 16; m <<= 1) v = pf_add(v, pf_shfl(v, m));
-    x = pf{__shfl_sync(0xffffffffu, v.h, 0), __shfl_sync(0xffffffffu, v.l, 0)};
-    y = pf{__shfl_sync(0xffffffffu, v.h, 1), __shfl_sync(0xffffffffu, v.l, 1)};
+    for (int m = 2; m <= 16; m <<= 1) v = df_add(v, df_shfl_xor(v, m));
+    x = df{__shfl_sync(0xffffffffu, v.h, 0), __shfl_sync(0xffffffffu, v.l, 0)};
+    y = df{__shfl_sync(0xffffffffu, v.h, 1), __shfl_sync(0xffffffffu, v.l, 1)};
   };
   // Partials of R c_1^T over the own columns, sent as step s (first step of a
   // launch or of a B step; later ones come with the update).
@@ -323,7 +282,7 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
       }
       if (!ok) break;
     }
-    pf cc = pf{0.f, 0.f};
+    df cc = df{0.f, 0.f};
     if (w == kResWarps - 1 && nrows > 0) {
       if (!take_pair(ld + 2 * (int)(s & 1), s, cc)) ok = false;
       if (lane == 0) red[2 * kResWarps] = cc;
@@ -334,14 +293,14 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
     cc = red[2 * kResWarps];
     const bool live = cc.h > 0.f;
     for (int r = w; r < nrows; r += kResWarps) {
-      pf q = pf{0.f, 0.f};
-      for (int g = lane; g < G; g += 32) q = pf_add(q, pf{vals[g * per + r], 0.f});
-      q = pf_warp_sum(q);
+      df q = df{0.f, 0.f};
+      for (int g = lane; g < G; g += 32) q = df_add(q, df{vals[g * per + r], 0.f});
+      q = df_warp_sum(q);
       if (lane == 0) {
         const float b_old = brow[k * rpc + r];
         float b_new = b_old;
         if (live) {
-          const pf v = pf_add(pf{b_old, 0.f}, pf_div(q, cc));
+          const df v = df_add(df{b_old, 0.f}, df_div(q, cc));
           b_new = v.h > 0.f ? v.h : 0.f;
         }
         brow[k * rpc + r] = b_new;
@@ -380,7 +339,7 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
   };
   // R += bo c_old - bn c_new on the own columns (cold, cnew) and, in the same
   // loop, the partials for the row cx of C (sent as step s) and, with obj, ||R||^2.
-  auto update = [&](const float* cx, unsigned s, bool send, bool obj, pf& r2) {
+  auto update = [&](const float* cx, unsigned s, bool send, bool obj, df& r2) {
     // a thread per row; where the rows leave threads over, several parts of
     // the columns (up to 512 / ld, at least 8 columns each) a row
     const int parts = min(kResThreads / ld, nc / 8);
@@ -391,7 +350,7 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
       const float x = bo[r], y = -bn[r];
       float* Rr = R + (size_t)clo * ld + r;
       float p = 0.f;
-      pf q = pf{0.f, 0.f};                         // squares, four at a time
+      df q = df{0.f, 0.f};                         // squares, four at a time
       int c = clo;
       for (; c + 4 <= chi; c += 4) {
         const float4 c0 = *reinterpret_cast<const float4*>(cold + c), c1 = *reinterpret_cast<const float4*>(cnew + c);
@@ -410,20 +369,20 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
         p = fmaf(v1, c2.y, p);
         p = fmaf(v2, c2.z, p);
         p = fmaf(v3, c2.w, p);
-        if (obj) pf_acc(q, fmaf(v0, v0, fmaf(v1, v1, fmaf(v2, v2, v3 * v3))));
+        if (obj) df_acc(q, fmaf(v0, v0, fmaf(v1, v1, fmaf(v2, v2, v3 * v3))));
       }
       for (; c < chi; ++c, Rr += ld) {
         const float v = fmaf(x, cold[c], fmaf(y, cnew[c], *Rr));
         *Rr = v;
         p = fmaf(v, cx[c], p);
-        if (obj) pf_acc(q, v * v);
+        if (obj) df_acc(q, v * v);
       }
       if (parts > 1) {
         if (part < parts) ps[t] = p;               // ps[part * ld + r]
       } else if (send) {
         st_word(mine + r, p, s);
       }
-      if (obj) r2 = pf_add(r2, q);
+      if (obj) r2 = df_add(r2, q);
     }
     if (parts > 1 && send) {
       __syncthreads();
@@ -436,10 +395,10 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
   };
   // c_k on the own columns from bn: a warp takes a column, or two where there
   // are more than warps.
-  auto columns = [&](int k, const float* ck, pf bb, pf bob) {
+  auto columns = [&](int k, const float* ck, df bb, df bob) {
     const bool cdeg = !(bb.h > 0.f);
-    const float inv_bb = cdeg ? 0.f : pf_div(pf{1.f, 0.f}, bb).h;
-    const float alpha = cdeg ? 0.f : pf_div(bob, bb).h;
+    const float inv_bb = cdeg ? 0.f : df_div(df{1.f, 0.f}, bb).h;
+    const float alpha = cdeg ? 0.f : df_div(bob, bb).h;
     if (cdeg && cta == 0 && t == 0) atomicAdd(a.degen, 1ull);
     const float4* b4 = reinterpret_cast<const float4*>(bn);
     auto finish = [&](int c, float dot) {
@@ -500,17 +459,17 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
   const bool inter = a.order != DID_ORDER_DID;
   if (!dead && inter) send_first(step + 1);
   for (int s = 0; s < a.n_sweeps && !dead; ++s) {
-    pf r2 = pf{0.f, 0.f};
+    df r2 = df{0.f, 0.f};
     if (!inter) {
       // C step: b fixed, columns local.  B is current in global memory (the
       // launch's start, or the grid barrier after the last B step).
       for (int k = 0; k < K; ++k) {
-        pf bb = pf{0.f, 0.f}, dummy = bb;
+        df bb = df{0.f, 0.f}, dummy = bb;
         __syncthreads();                           // bn, bo, cold, cnew are free
         for (int r = t; r < ld; r += kResThreads) {
           const float v = __ldcg(a.B + (size_t)k * ld + r);
           bn[r] = bo[r] = v;
-          bb = pf_fma(v, v, bb);
+          bb = df_fma(v, v, bb);
         }
         load_row(k);
         block_pairs(bb, dummy);
@@ -551,10 +510,10 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
       if (rec) a.tstamp[4 * at + 1] = globaltimer_ns();
       if (inter) {
         // (a thread reads only the rows it stored, so this needs no barrier)
-        pf bb = pf{0.f, 0.f}, bob = bb;
+        df bb = df{0.f, 0.f}, bob = bb;
         for (int r = t; r < ld; r += kResThreads) {
-          bb = pf_fma(bn[r], bn[r], bb);
-          bob = pf_fma(bn[r], bo[r], bob);
+          bb = df_fma(bn[r], bn[r], bb);
+          bob = df_fma(bn[r], bo[r], bob);
         }
         block_pairs(bb, bob);                      // its barrier publishes bn, bo, bad
         if (bad[1]) { dead = true; break; }
@@ -578,7 +537,7 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
     }
     if (dead) break;
     // objective: the CTAs' sums, in order, in every CTA that needs the value
-    pf z = pf{0.f, 0.f};
+    df z = df{0.f, 0.f};
     __syncthreads();
     block_pairs(r2, z);
     if (t == 0) {
@@ -588,7 +547,7 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
     bool stop = false;
     const bool need = a.stop_rule != 0 || cta == 0;
     if (need && w == 0) {
-      pf f2;
+      df f2;
       const bool ok = take_pair(ld + 4 + 2 * (s & 1), step, f2);
       if (!ok) bad[2] = 1;
       if (lane == 0) red[2 * kResWarps + 1] = f2;
@@ -605,7 +564,7 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
     __syncthreads();
     if (bad[2]) { dead = true; break; }
     if (need) {
-      const pf f2 = red[2 * kResWarps + 1];
+      const df f2 = red[2 * kResWarps + 1];
       const double f = 0.5 * ((double)f2.h + (double)f2.l);
       if (cta == 0 && t == 0) {
         a.trace[s] = f;
@@ -742,8 +701,9 @@ bool plan_resident(int ld, int64_t N, int K, int grid_override, ResidentPlan* pl
 }
 
 // Within a launch of several instances the CTAs are shared out by the caller.
-bool plan_resident_on(int ld, int64_t N, int K, int grid, ResidentPlan* plan) {
-  static const size_t budget = res_budget((const void*)resident_multi_kernel);
+size_t resident_multi_budget() { return res_budget((const void*)resident_multi_kernel); }
+
+bool plan_resident_on(size_t budget, int ld, int64_t N, int K, int grid, ResidentPlan* plan) {
   return grid > 0 && plan_on(ld, N, K, grid, budget, plan);
 }
 
@@ -765,7 +725,7 @@ void fill_resident_args(void* dst, const ResidentPlan& plan, const SweepArgs& s,
 cudaError_t launch_resident_multi(const void* d_args, int ninst, int grid, size_t smem, cudaStream_t st) {
   const ResArgs* inst = static_cast<const ResArgs*>(d_args);
   const cudaError_t e = cudaFuncSetAttribute(resident_multi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)res_budget((const void*)resident_multi_kernel));
+                                             (int)resident_multi_budget());
   if (e != cudaSuccess) return e;
   void* params[] = {(void*)&inst, (void*)&ninst};
   return cudaLaunchCooperativeKernel((const void*)resident_multi_kernel, dim3(grid), dim3(kResThreads), params, smem, st);

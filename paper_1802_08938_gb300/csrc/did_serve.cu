@@ -103,6 +103,7 @@ struct did_server {
   bool own_stream = false;
   int grid = 0;
   size_t smem_budget = 0;
+  size_t res_budget = 0;             // shared memory of a CTA of the resident kernel on this device
   std::chrono::steady_clock::time_point t0;
 
   std::mutex mu;
@@ -317,14 +318,14 @@ void choose_form(const did_server* s, Req* r) {
   const int K = r->rq.K;
   did::ResidentPlan p{};
   r->form = PACKED;
-  if (did::plan_resident_on(r->ld, N, K, s->grid, &p)) {
+  if (did::plan_resident_on(s->res_budget, r->ld, N, K, s->grid, &p)) {
     int lo = 1, hi = s->grid;
     while (lo < hi) {
       const int mid = (lo + hi) / 2;
-      if (did::plan_resident_on(r->ld, N, K, mid, &p)) hi = mid; else lo = mid + 1;
+      if (did::plan_resident_on(s->res_budget, r->ld, N, K, mid, &p)) hi = mid; else lo = mid + 1;
     }
     r->form = RESIDENT;
-    r->ctas = did::plan_resident_on(r->ld, N, K, lo, &p) ? lo : s->grid;
+    r->ctas = did::plan_resident_on(s->res_budget, r->ld, N, K, lo, &p) ? lo : s->grid;
   } else if (r->ld >= 4 * K && did::plan_defer(r->ld, N, K, s->bf16, 0, &r->dplan)) {
     r->form = DEFER;
   }
@@ -497,7 +498,8 @@ std::vector<Bin> pack(const did_server* s, const std::vector<Req*>& act, std::ve
     for (int q = 0; q < n; ++q) {
       const Req* r = act[b.slots[q]];
       did::ResidentPlan p{};
-      if (!did::plan_resident_on(r->ld, r->rq.N, r->rq.K, g[q], &p)) did::plan_resident_on(r->ld, r->rq.N, r->rq.K, r->ctas, &p);
+      if (!did::plan_resident_on(s->res_budget, r->ld, r->rq.N, r->rq.K, g[q], &p))
+        did::plan_resident_on(s->res_budget, r->ld, r->rq.N, r->rq.K, r->ctas, &p);
       b.plans.push_back(p);
       b.words += a256(p.words_bytes);
       b.ctas += p.grid;
@@ -616,7 +618,7 @@ bool run_round(did_server* s, std::vector<Req*>& act) {
     d.b.degen = s->d_degen + i;
     r->sh_last = 0;
     const double sweep_s =
-        r->rq.K * (20e-6 + (double)r->ld * r->rq.N * (s->bf16 ? 2.0 : 4.0) / 6.5e12);
+        r->rq.K * (kDeferFixedS + (double)r->ld * r->rq.N * (s->bf16 ? 2.0 : 4.0) / kDeferBytesPerS);
     const int nsw = std::max(1, std::min(std::min(s->round_sweeps, r->rq.max_iter - r->sweeps), (int)(kDeferSliceS / sweep_s)));
     double* tr = s->d_trace + (size_t)i * s->round_sweeps;
     did::DenseArgs da{};
@@ -789,6 +791,7 @@ did_status did_server_create(size_t hbm_budget_bytes, did_precision precision, i
     return DID_ECUDA;
   }
   s->max_slots = std::min(max_slots, s->grid);
+  s->res_budget = did::resident_multi_budget();
   s->dense_grid = did::dense_grid();
   bool ok = true;
   if (stream) {

@@ -31,6 +31,7 @@
 #include "did_pair.cuh"
 
 #include <algorithm>
+#include <type_traits>
 
 namespace did {
 
@@ -339,7 +340,9 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
   };
   // R += bo c_old - bn c_new on the own columns (cold, cnew) and, in the same
   // loop, the partials for the row cx of C (sent as step s) and, with obj, ||R||^2.
-  auto update = [&](const float* cx, unsigned s, bool send, bool obj, df& r2) {
+  // (obj, a compile-time constant, keeps the sum of squares out of the other steps' loop)
+  auto update_as = [&](auto objective, const float* cx, unsigned s, bool send, df& r2) {
+    constexpr bool obj = decltype(objective)::value;
     // a thread per row; where the rows leave threads over, several parts of
     // the columns (up to 512 / ld, at least 8 columns each) a row
     const int parts = min(kResThreads / ld, nc / 8);
@@ -392,6 +395,12 @@ __device__ __forceinline__ void resident_body(const ResArgs& a, const int cta, c
         st_word(mine + t, p, s);
       }
     }
+  };
+  auto update = [&](const float* cx, unsigned s, bool send, bool obj, df& r2) {
+    if (obj)
+      update_as(std::true_type{}, cx, s, send, r2);
+    else
+      update_as(std::false_type{}, cx, s, send, r2);
   };
   // c_k on the own columns from bn: a warp takes a column, or two where there
   // are more than warps.

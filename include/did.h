@@ -86,14 +86,15 @@ typedef struct {
     int32_t refresh_every;  /* recompute R = X - B C densely before every n-th sweep; 0 = never */
     int32_t stop;           /* did_stop */
     int32_t init_scale;     /* 1: scale B and C by sqrt(<X,BC>/||BC||^2) after initialisation */
-    int32_t grid_ctas;      /* persistent grid size; 0 = one per SM times occupancy */
+    int32_t grid_ctas;      /* CTAs of a sweep (at most one per SM); 0 = chosen by the library */
     const float* B_init;    /* optional start point, host or device, M x K column-major; NULL = seeded */
     const float* C_init;    /* optional start point, host or device, K x N row-major; NULL = seeded */
     void* stream;           /* cudaStream_t to order all work on; NULL = legacy default stream */
     uint64_t timeout_ns;    /* limit of every device-side wait; 0 = 4 s; values below
                                10 ms are raised to 10 ms (a wait also covers the
                                CTA's own copies and tensor-core work) */
-    int32_t debug_barrier_extra; /* test hook: arrivals a grid wait expects beyond the grid (0 in use) */
+    int32_t debug_barrier_extra; /* test hook: arrivals a grid wait expects beyond the grid (0 in use);
+                               a resident sweep waits for a word that nothing sends */
     int32_t flags;          /* DID_FLAG_* bits */
     /* Inner repeats per sweep (DID_ORDER_DID_BATCHED only; 0 means 1): the C
      * step runs inner_c times, then the B step inner_b times, each repeat the
@@ -114,25 +115,26 @@ typedef struct {
  * the tensor-core pass (BF16x3 for a bfloat16 residual with K <= 128, BF16x6
  * for a float32 one with K <= 64; larger K always takes the SIMT pass). */
 #define DID_FLAG_SIMT_REFRESH 2
-/* did_options.flags.  Without a flag of this group (or DID_FLAG_SIMT_REFRESH),
- * a residual that fits the SMs' shared memory (about 30 MB in float32) stays
- * there for a whole launch of sweeps, in float32 also when it is stored in bfloat16
- * (both per-k orders).
- * DID_ORDER_INTERLEAVED: without a flag below, sweeps of a larger residual
- * (K <= 128) only read R:
- * the changes of a sweep stay pending as vectors, and R is formed anew from X
- * after its last k (did_info then counts a periodic refresh that falls due,
- * which finds R formed from the current factors already); so do those of
- * DID_ORDER_DID (with columns up to about 8000 rows, a pass then serving several k).
- * Deferred write-back defers the
- * write of R for k to the pass for k+1 (one write per pair of k, three passes
- * over R per pair instead of four).  It needs two more M-vectors of shared
- * memory beside a ring of at least three column stages per group.  By default
- * a float32 residual uses it where it fits and a bfloat16 residual does not
- * (its passes are bound by the per-column work, which the deferred form
- * raises).  EAGER forces one write per k; LAZY requests deferral for either
- * precision.  did_info.lazy_writeback says which the sweep kernel is planned
- * with. */
+/* did_options.flags: how the sweeps of the per-k orders treat R (did_form).
+ * Without a flag below and without DID_FLAG_SIMT_REFRESH:
+ *   - a residual that fits the SMs' shared memory (about 30 MB in float32) stays
+ *     there for a whole launch of sweeps, in float32 also when it is stored in
+ *     bfloat16;
+ *   - sweeps of a larger one (K <= 128, columns of 4 K to about 17000 rows, 16 MiB
+ *     or more) only read R: the changes of a sweep stay pending as vectors, and R is
+ *     formed anew from X after its last k.  did_info then counts a periodic
+ *     refresh that falls due, which finds R formed from the current factors
+ *     already.  In DID_ORDER_DID a pass serves four k, or two where columns have
+ *     more than 8192 rows (up to 12288, a bfloat16 residual 16384);
+ *   - the sweep kernel, which reads and writes R, takes the rest.
+ * Deferred write-back (interleaved order): the sweep kernel defers the write of
+ * R for k to the pass for k+1 (one write per pair of k, three passes over R per
+ * pair instead of four).  It needs two more M-vectors of shared memory beside a
+ * ring of at least three column stages per group.  By default a float32
+ * residual uses it where it fits and a bfloat16 residual does not (its passes
+ * are bound by the per-column work, which the deferred form raises).  EAGER
+ * forces one write per k; LAZY requests deferral for either precision.  Either
+ * selects the sweep kernel; did_info.lazy_writeback says how it is planned. */
 #define DID_FLAG_EAGER_WRITEBACK 8
 #define DID_FLAG_LAZY_WRITEBACK 16
 /* did_options.flags (DID_ORDER_INTERLEAVED): c-passes take one column per
@@ -154,7 +156,7 @@ typedef struct {
     int64_t M, N;
     int32_t K;
     int32_t precision, order;
-    int32_t grid_ctas;       /* persistent grid of the sweep kernel */
+    int32_t grid_ctas;       /* CTAs of a sweep launch */
     int32_t group_threads;   /* threads cooperating on one column */
     int32_t vecs_per_thread; /* 16-byte vectors of a column each thread holds */
     int32_t column_units;    /* units (contiguous column ranges) per pass */
@@ -166,9 +168,9 @@ typedef struct {
     size_t device_bytes;     /* device memory owned by the context */
     /* Device time of the library's own launches, from CUDA events recorded on
      * the context's stream around each launch (accumulated since creation). */
-    int64_t sweep_launches;  /* persistent sweep-kernel launches */
-    int64_t prologue_launches; /* sweep launches that first re-formed R c_1^T */
-    double sweep_kernel_ms;  /* total device time of those launches */
+    int64_t sweep_launches;  /* sweep launches; DID_FORM_READ_ONLY, DID_FORM_BATCHED: sweeps, of several kernels each */
+    int64_t prologue_launches; /* sweep-kernel launches that first re-formed R c_1^T */
+    double sweep_kernel_ms;  /* total device time of those launches (read-only: with the passes that form R) */
     int64_t dense_launches;  /* refresh / objective / scaling passes */
     double dense_kernel_ms;
     int64_t tc_refreshes;    /* refreshes done on the tensor cores */
@@ -203,7 +205,8 @@ did_status did_create_ex(const float* X, int64_t M, int64_t N, int32_t K, uint64
  * the exact nonnegative minimiser of its block (Section 2, HALS closed forms;
  * Section 4.1, equations up:c and sol:b_i): with A = R + b_k c_k,
  *     b_k := [A c_k^T / (c_k c_k^T)]_+ ,   c_k := [b_k^T A / (b_k^T b_k)]_+ ,
- * and the residual is updated in place, R := A - b_k c_k (Section 4.2).
+ * and R := A - b_k c_k (Section 4.2), in place or, in DID_FORM_READ_ONLY, for
+ * all k at the end of the sweep.
  * A block whose partner has zero norm is left unchanged.  After each sweep
  * 1/2 ||R||^2 is appended to the objective trace. */
 did_status did_sweep(did_ctx* ctx, int32_t n_sweeps);
@@ -219,14 +222,15 @@ did_status did_factor(did_ctx* ctx, int32_t max_iter, double tol, int32_t* iters
  * cudaMalloc where they run: code inside another runtime's allocator or
  * memory-planning hooks, or a host that fixed its device memory budget up
  * front.  The paper has no counterpart; this is a library convenience.
- * It runs n_sweeps sweeps of the same kernel as did_sweep (interleaved order,
- * float32 residual) on caller-owned device buffers, updated in place:
+ * It runs n_sweeps sweeps (interleaved order, float32 residual) of the resident
+ * kernel, or of the sweep kernel where R does not fit the SMs' shared memory,
+ * on caller-owned device buffers, updated in place:
  *   R : ld x N column-major residual X - B C, ld a multiple of 4, ld >= M,
  *       rows M..ld-1 zero, 16-byte aligned;
  *   B : ld x K column-major, rows M..ld-1 zero, 16-byte aligned;
  *   C : K x N row-major.
  * trace (may be NULL; host or device) receives 1/2 ||R||^2 after each sweep.
- * Its scratch (grid partials, per-CTA scalars, control words) is one static
+ * Its scratch (exchange words or grid partials, per-CTA scalars, control words) is one static
  * device array of 6 MiB that every GPU which loads the library holds until
  * the process exits; limits: ld <= 8192, n_sweeps <= 1024, at most 160 CTAs
  * (DID_E_TOO_LARGE beyond them).  It calls no cudaMalloc/cudaFree.  R, B and
@@ -244,7 +248,8 @@ did_status did_sweep_static(float* R, int64_t ld, float* B, float* C, int64_t M,
                             int32_t n_sweeps, double* trace, void* stream);
 
 /* Exact objective 1/2 ||X - B C||_F^2 (Section 1) from X, B, C in a fresh
- * pass (float32 products, float64 accumulation); R is not touched. */
+ * pass; R is not touched.  Products and sums of four squares in float32, the
+ * sums of those in float64 or pairs of float32 (48 bits). */
 did_status did_objective(did_ctx* ctx, double* obj);
 
 /* 1/2 ||R||_F^2 of the stored residual E = X - B C of Section 4.2 (the

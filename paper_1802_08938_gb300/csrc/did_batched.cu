@@ -1315,7 +1315,8 @@ cudaError_t set_update_b_smem(int K) {
 // YY = Y^T Y (2K x 2K column-major) over the ld rows of Y = [D | B]: block
 // (a, b0) forms entries (a, b0..b0+15); float32 within a thread's rows, then
 // float32 pairs across threads in a fixed tree, eight entries a time (float64
-// shuffles, which issue at 1/64 the rate, took most of the former 79 us).
+// shuffles, which issue at 1/64 the rate, took most of the former 79 us; an entry
+// is rounded to float32 at the end either way).
 constexpr int kYYThreads = 256;
 __global__ void __launch_bounds__(kYYThreads) yy_kernel(const float* __restrict__ Y, int ld, int K2, float* YY) {
   __shared__ df red[kYYThreads / 32][16];

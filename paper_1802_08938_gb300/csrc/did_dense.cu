@@ -148,9 +148,10 @@ __global__ void __launch_bounds__(kDenseThreads) dense_kernel(DenseTileArgs t) {
 // sums (each of four squares in float32, as there) are float32 pairs of about
 // 48 bits until the end.  The next chunk of B and C is loaded into
 // registers while this one is used.  Each product is the same chain of FMAs in k
-// order, so R comes out bit for bit the same.  Measured: 10000 x 100000,
-// K = 100 (exact objective) 11.9 -> 5.9 ms; 8165 x 18821, K = 100, a refresh or an
-// objective 1.9 -> 0.95 ms.
+// order, so R comes out bit for bit the same.  A kernel for each mode, as the
+// sums of the others cost it up to 20 %.  Measured, against the tile above:
+// 10000 x 100000, K = 100 (exact objective) 11.9 -> 4.9 ms; 8165 x 18821, K =
+// 100, an objective 1.9 -> 0.77 ms, a refresh 1.9 -> 0.98 ms.
 constexpr int kBig = 128;
 constexpr int kBigKc = 16;
 constexpr int kBigThreads = 256;

@@ -20,7 +20,7 @@
 // carries its step number in the same 8 bytes, so the receiver polls the data
 // itself: no fence, no atomic, and no load after the barrier.  The sweep kernel's
 // per-k cost on these sizes is 27 to 32 us (two grid barriers with the
-// loads behind them); here 6.5 us at 200 x 1000 (32 CTAs), 8.5 us at 1024 x
+// loads behind them); here 6.5 us at 200 x 1000 (32 CTAs), 8.6 us at 1024 x
 // 2414 (76 CTAs), of which the exchange takes 2.4 and 3.7.  A word is
 // overwritten only after its readers have used it: a CTA sends the partials of step s + 1
 // after it has all of b'(s), and b'(s) is sent after the owner has read every
@@ -689,8 +689,9 @@ bool plan_resident(int ld, int64_t N, int K, int grid_override, ResidentPlan* pl
   // Columns of a CTA: two for each warp (32), the fewest CTAs that gives, so
   // that an exchange has few parties; fewer where a column range must be
   // shorter to fit, more where the grid is at its limit.  A k of 200 x 1000 /
-  // 1024 x 2414 / 43 x 1694: 7.5 / 8.9 / 8.1 us with 8 columns, 6.6 / 8.9 /
-  // 7.2 with 16, 6.3 / 8.7 / 6.1 with 32, 7.3 / 8.6 / 6.3 with 64.
+  // 1024 x 2414 / 43 x 1694 in one run: 7.5 / 8.9 / 8.1 us with 8 columns, 6.6 /
+  // 8.9 / 7.2 with 16, 6.3 / 8.7 / 6.1 with 32, 7.3 / 8.6 / 6.3 with 64 (GPUs
+  // differ by some 5 %, short columns by more).
   ResidentPlan P{};
   for (int nc = 32; nc >= 1 && P.grid == 0; nc /= 2) {
     const int64_t g = (N + nc - 1) / nc;
